@@ -465,6 +465,105 @@ bool build_tc_tables(const OptParams &op, TcTables &tt) {
     return ok;
 }
 
+bool build_tc_dev(const OptParams &op, TcDev &td, uint64_t beta[kRP][kRP]) {
+    std::memset(&td, 0, sizeof td);
+    ChainParams cp;
+    derive_chain(op, cp);
+    const uint64_t R = kEps, R6 = fp_pow(R, 6), R7 = fp_mul(R6, R);
+    for (int q = 0; q < kRP; ++q)
+        for (int r = 0; r < kRP; ++r) beta[q][r] = r <= q ? fp_mul(cp.beta[q][r], R7) : 0;
+
+    // constants added by each kind's bias
+    uint64_t add[kBiasKinds][kT] = {};
+    for (int i = 0; i < kT; ++i) {
+        // dense layer r feeds round r + 1; round 3's feeds the partial rounds
+        // (cell 0's S-box; cells 1..11 wait for the W contraction, which adds
+        // round 4's constants to all cells)
+        for (int r = 0; r < kRF - 1; ++r)
+            if (r != kRF / 2 - 1) add[kBiasDense + r][i] = op.full_rc[r + 1][i] % kP;
+        add[kBiasW][i] = op.full_rc[kRF / 2][i] % kP;
+        if (i < kTcUa) add[kBiasUa][i] = op.part_rc[i + 1] % kP;
+        const int q = kTcUa + i;
+        if (q < kRP - 1) add[kBiasUb][i] = op.part_rc[q + 1] % kP;
+    }
+    add[kBiasDense + kRF / 2 - 1][0] = op.part_rc[0] % kP;
+
+    // u_b(k, i) in [1407, 1665] as in tc_bias_blocks, here with the offset of
+    // tc_combine: sum_b 2^(8b) (v_b - 2^23) + 0x3F + 0x3F3F + (0x3F00 + 0x3F0000) 2^64
+    typedef unsigned __int128 u128;
+    const uint64_t G = 0x0101010101010101ull;
+    uint64_t off = fp_sub(0x3F + 0x3F3F, fp_mul(1u << 23, G % kP));
+    off = fp_add(off, fp_mul(0x3F00 + 0x3F0000, kEps));
+    static int u[kBiasKinds][kT][8];
+    for (int k = 0; k < kBiasKinds; ++k)
+        for (int i = 0; i < kT; ++i) {
+            const uint64_t t = fp_mul(fp_sub(add[k][i], off), fp_inv(8192));
+            const uint64_t umin_p = (uint64_t)(((u128)1407 * G) % kP);
+            u128 rest = fp_sub(t, umin_p);
+            for (int b = 7; b >= 0; --b) {
+                const u128 wgt = (u128)1 << (8 * b);
+                u128 e = rest / wgt;
+                if (e > 258) e = 258;
+                rest -= e * wgt;
+                u[k][i][b] = 1407 + (int)e;
+                td.b_bias[(i * 2 + k / 8) * 64 + b * 8 + k % 8] = half_of_int(4 * u[k][i][b]);
+            }
+            if (rest != 0) return false;
+        }
+    for (int j = 0; j < 8; ++j)
+        for (int r = 0; r < 8; ++r) td.a_bias[(1 + j) * 64 + r * 8 + j] = 0x0800;  // 2^-13
+
+    static uint64_t mat[kT * kT];
+    bool ok = true;
+    auto table = [&](auto &&entry, int n, uint16_t *dst, long *pos, long *neg) {
+        for (int i = 0; i < n; ++i)
+            for (int j = 0; j < kT; ++j) mat[i * kT + j] = fp_mul(entry(i, j) % kP, R6);
+        digit_table(mat, n, kT, dst, pos, neg);
+    };
+    auto check = [&](const long *pos, const long *neg, int k, int n) {
+        for (int r = 0; r < 8 * n; ++r) {
+            const long magic = 8192L * u[k][r / 8][r % 8];
+            ok = ok && magic - 255 * neg[r] >= (1L << 23) && magic + 255 * pos[r] < (1L << 24);
+        }
+    };
+    {
+        long pos[kTcN] = {}, neg[kTcN] = {};
+        table([&](int i, int j) { return op.mds[i][j]; }, kT, td.m, pos, neg);
+        for (int r = 0; r < kRF; ++r)
+            if (r != kRF / 2 - 1) check(pos, neg, kBiasDense + r, kT);
+    }
+    {
+        long pos[kTcN] = {}, neg[kTcN] = {};
+        table([&](int i, int j) { return op.pre[i][j]; }, kT, td.pre, pos, neg);
+        check(pos, neg, kBiasDense + kRF / 2 - 1, kT);
+    }
+    {
+        long pos[kTcN] = {}, neg[kTcN] = {};
+        table([&](int i, int j) { return cp.vp[i][j]; }, kTcUa, td.vpa, pos, neg);
+        check(pos, neg, kBiasUa, kTcUa);
+    }
+    {
+        long pos[kTcN] = {}, neg[kTcN] = {};
+        table([&](int i, int j) { return cp.vp[kTcUa + i][j]; }, kT, td.vpb, pos, neg);
+        table([&](int i, int j) { return kTcUa + i < kRP - 1 && j < kTcSplit ? cp.beta[kTcUa + i][j] : 0ull; }, kT, td.bs,
+              pos, neg);
+        check(pos, neg, kBiasUb, kT);
+    }
+    {
+        long pos[kTcN] = {}, neg[kTcN] = {};
+        table([&](int i, int j) { return j < kTcSplit ? cp.w[i][j] : 0ull; }, kT, td.w1, pos, neg);
+        table([&](int i, int j) { return j < kRP - kTcSplit ? cp.w[i][kTcSplit + j] : 0ull; }, kT, td.w2, pos, neg);
+        check(pos, neg, kBiasW, kT);
+    }
+    const uint64_t Rm6 = fp_inv(R6);
+    for (int j = kRate; j < kT; ++j) {
+        const uint64_t c7 = fp_mul(fp_pow(op.full_rc[0][j] % kP, 7), Rm6);
+        for (int r = 0; r < 8; ++r)
+            for (int a = 0; a < 8; ++a) td.a_zcap[(j - kRate) * 64 + r * 8 + a] = (uint16_t)((c7 >> (8 * a)) & 0xFF);
+    }
+    return ok;
+}
+
 // ------------------------------------------------------------ SHA-256
 // FIPS 180-4 SHA-256 of a byte string, used to fingerprint a parameter set.
 // Its constants are computed from their definition rather than tabulated:

@@ -214,31 +214,30 @@ __global__ void __launch_bounds__(kSmallBlock) k_merkle_level(const uint64_t *__
 // its digit tables (124 KB) and the groups' A operands take 225 KB of shared
 // memory, its groups 128 columns of tensor memory each; every thread keeps
 // its state in registers).
-// Group q of CTA c takes units c * kTcGroups + q, then every
+// Group q of CTA c takes unit c + q * gridDim.x, then every
 // gridDim.x * kTcGroups-th after: a static schedule with no shared counter,
 // so launches on different streams are independent.  A unit is 128
 // consecutive states or rows; rows past the end are computed on zeros and
 // not stored.
-// PG12_TC_CHAIN 1 (default): the partial rounds in their unrolled form on the
-// tensor cores (tc_partial, 87 KB of the tables); 0: on the integer pipes.
-#ifndef PG12_TC_CHAIN
-#define PG12_TC_CHAIN 1
-#endif
 #ifndef PG12_TC_GROUPS
 #define PG12_TC_GROUPS 4
 #endif
-constexpr bool kTcChain = PG12_TC_CHAIN != 0;
 constexpr int kTcGroups = PG12_TC_GROUPS;
 constexpr int kTcThreads = kTcGroup * kTcGroups;
-using TcL = TcLayout<kTcGroups, kTcChain>;
-using TcL1 = TcLayout<1, false>;  // one-group CTAs of small launches
+using TcL = TcLayout<kTcGroups>;
+
+// Group q's first unit: CTA index plus q times the grid, so that a launch of
+// few units spreads them over all SMs before any SM gets a second one.
+__device__ __forceinline__ uint64_t tc_first_unit() {
+    return blockIdx.x + (uint64_t)gridDim.x * (threadIdx.x / kTcGroup);
+}
 
 __global__ void __launch_bounds__(kTcThreads, 1) k_tc_permute(uint64_t *__restrict__ st, uint64_t n, int vec16) {
     extern __shared__ __align__(1024) uint8_t tc_sm[];
-    TcGroup G = tc_setup<kTcGroups, kTcChain>(tc_sm);
+    TcGroup G = tc_setup<kTcGroups>(tc_sm);
     const uint64_t units = (n + kTcGroup - 1) / kTcGroup;
     const uint64_t step = (uint64_t)gridDim.x * kTcGroups;
-    for (uint64_t u = (uint64_t)blockIdx.x * kTcGroups + threadIdx.x / kTcGroup; u < units; u += step) {
+    for (uint64_t u = tc_first_unit(); u < units; u += step) {
         const uint64_t k = u * kTcGroup + G.t;
         const bool valid = k < n;
         uint64_t *p = st + kT * k;
@@ -250,7 +249,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_permute(uint64_t *__restri
 #pragma unroll
             for (int i = 0; i < kT; ++i) x[i] = valid ? p[i] : 0ull;
         }
-        if (!tc_permute<kTcChain>(G, x, false, false)) break;
+        if (!tc_permute(G, x, false, false)) break;
         if (valid) {
             if (vec16) {
 #pragma unroll
@@ -261,28 +260,23 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_permute(uint64_t *__restri
             }
         }
     }
-    tc_teardown<kTcGroups, kTcChain>(tc_sm, G);
+    tc_teardown<kTcGroups>(tc_sm, G);
 }
 
 // Sponge digests of n rows of width w (Sec. 2.4): the leaves of a tree, or a
 // tree level (the level below read as rows of its children's 8 words), or
 // pg_hash_rows.  Launched as a dependent launch it may set up while the
 // kernel before it finishes, and reads `rows` only after pdl_wait().
-// GROUPS = kTcGroups for large launches (one CTA per SM); GROUPS = 1 with
-// the partial rounds on the integer pipes for launches of few units (62 KB
-// of shared memory and 128 tensor-memory columns per CTA, up to three CTAs
-// per SM), which spread them over more SMs.
-template <int GROUPS, bool CHAIN>
-__global__ void __launch_bounds__(kTcGroup * GROUPS, 1) k_tc_sponge(const uint64_t *__restrict__ rows, uint64_t n,
-                                                                    uint64_t w, int vec16, uint64_t *__restrict__ out) {
+__global__ void __launch_bounds__(kTcThreads, 1) k_tc_sponge(const uint64_t *__restrict__ rows, uint64_t n,
+                                                             uint64_t w, int vec16, uint64_t *__restrict__ out) {
     extern __shared__ __align__(1024) uint8_t tc_sm[];
     pdl_trigger();
-    TcGroup G = tc_setup<GROUPS, CHAIN>(tc_sm);
+    TcGroup G = tc_setup<kTcGroups>(tc_sm);
     pdl_wait();
     const uint64_t units = (n + kTcGroup - 1) / kTcGroup;
-    const uint64_t step = (uint64_t)gridDim.x * GROUPS;
+    const uint64_t step = (uint64_t)gridDim.x * kTcGroups;
     const uint64_t chunks = (w + kRate - 1) / kRate;
-    for (uint64_t u = (uint64_t)blockIdx.x * GROUPS + threadIdx.x / kTcGroup; u < units; u += step) {
+    for (uint64_t u = tc_first_unit(); u < units; u += step) {
         const uint64_t r = u * kTcGroup + G.t;
         const bool valid = r < n;
         const uint64_t *row = rows + (valid ? r : 0) * w;
@@ -295,7 +289,7 @@ __global__ void __launch_bounds__(kTcGroup * GROUPS, 1) k_tc_sponge(const uint64
             load_chunk(row, w, c, vec16 != 0, ch);
 #pragma unroll
             for (int i = 0; i < kRate; ++i) x[i] = valid ? ch[i] : 0ull;
-            ok = tc_permute<CHAIN>(G, x, c == 0, c + 1 == chunks);
+            ok = tc_permute(G, x, c == 0, c + 1 == chunks);
         }
         if (!ok) break;
         if (valid) {
@@ -303,7 +297,7 @@ __global__ void __launch_bounds__(kTcGroup * GROUPS, 1) k_tc_sponge(const uint64
             st2(out + kDigest * r + 2, canon(x[2]), canon(x[3]));
         }
     }
-    tc_teardown<GROUPS, CHAIN>(tc_sm, G);
+    tc_teardown<kTcGroups>(tc_sm, G);
 }
 
 // Leaf sponges over rows that arrive in chunks while the kernel runs
@@ -331,17 +325,16 @@ __device__ __forceinline__ bool wait_ready(const uint32_t *ready, uint32_t want)
     }
 }
 
-template <int GROUPS, bool CHAIN>
-__global__ void __launch_bounds__(kTcGroup * GROUPS, 1)
+__global__ void __launch_bounds__(kTcThreads, 1)
     k_tc_leaves_stream(const uint64_t *__restrict__ rows, uint64_t n, uint64_t w, int vec16,
                        uint64_t *__restrict__ out, const uint32_t *__restrict__ ready, const ChunkMap cm) {
     extern __shared__ __align__(1024) uint8_t tc_sm[];
-    TcGroup G = tc_setup<GROUPS, CHAIN>(tc_sm);
+    TcGroup G = tc_setup<kTcGroups>(tc_sm);
     const uint64_t units = (n + kTcGroup - 1) / kTcGroup;
-    const uint64_t step = (uint64_t)gridDim.x * GROUPS;
+    const uint64_t step = (uint64_t)gridDim.x * kTcGroups;
     const uint64_t chunks = (w + kRate - 1) / kRate;
     uint32_t have = 0;  // chunks this group has seen arrive
-    for (uint64_t u = (uint64_t)blockIdx.x * GROUPS + threadIdx.x / kTcGroup; u < units; u += step) {
+    for (uint64_t u = tc_first_unit(); u < units; u += step) {
         const uint64_t last = (u + 1) * kTcGroup < n ? (u + 1) * kTcGroup - 1 : n - 1;
         uint32_t c = 0;
         while (c + 1 < cm.count && cm.end[c] <= last) ++c;
@@ -365,7 +358,7 @@ __global__ void __launch_bounds__(kTcGroup * GROUPS, 1)
             load_chunk_cg(row, w, k, vec16 != 0, ch);
 #pragma unroll
             for (int i = 0; i < kRate; ++i) x[i] = valid ? ch[i] : 0ull;
-            ok = tc_permute<CHAIN>(G, x, k == 0, k + 1 == chunks);
+            ok = tc_permute(G, x, k == 0, k + 1 == chunks);
         }
         if (!ok) break;
         if (valid) {
@@ -373,7 +366,7 @@ __global__ void __launch_bounds__(kTcGroup * GROUPS, 1)
             st2(out + kDigest * r + 2, canon(x[2]), canon(x[3]));
         }
     }
-    tc_teardown<GROUPS, CHAIN>(tc_sm, G);
+    tc_teardown<kTcGroups>(tc_sm, G);
 }
 
 // One warp task: lane i of task u at level l hashes node 32u+i of that level
@@ -541,7 +534,7 @@ __device__ __forceinline__ bool tc_unit(TcGroup &G, const TreePlan &tp, uint32_t
         }
 #pragma unroll
         for (int i = 0; i < kRate; ++i) x[i] = valid ? ch[i] : 0ull;
-        if (!tc_permute<kTcChain>(G, x, c == 0, c + 1 == chunks)) return false;
+        if (!tc_permute(G, x, c == 0, c + 1 == chunks)) return false;
     }
     if (valid) {
         uint64_t *dst = tp.nodes + kDigest * (level_off(n, l) + k);
@@ -556,7 +549,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_batch(const TreePlan *__re
                                                             uint32_t *__restrict__ counters,
                                                             uint32_t *__restrict__ next_task) {
     extern __shared__ __align__(1024) uint8_t tc_sm[];
-    TcGroup G = tc_setup<kTcGroups, kTcChain>(tc_sm);
+    TcGroup G = tc_setup<kTcGroups>(tc_sm);
     bool ok = true;
     while (ok) {
         const uint32_t task = group_fetch_add(G, next_task);
@@ -600,7 +593,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_batch(const TreePlan *__re
             lo >>= 1;
         }
     }
-    tc_teardown<kTcGroups, kTcChain>(tc_sm, G);
+    tc_teardown<kTcGroups>(tc_sm, G);
 }
 
 // The top levels of every tree of a batch whose persistent launch stopped
@@ -998,14 +991,13 @@ pg_status upload_tables() {
     dev::make_dev_consts(g.opt, dc);
     PG_CUDA(cudaMemcpyToSymbol(dev::c_dev, &dc, sizeof(dc)));
     PG_CUDA(cudaMemcpyToSymbol(dev::g_dev, &dc, sizeof(dc)));
-    static TcTables tt;  // 105 KB; built under g_mu
-    if (!host::build_tc_tables(g.opt, tt))
+    static TcDev td;  // 131 KB; built under g_mu
+    static uint64_t beta[kRP][kRP];
+    if (!host::build_tc_dev(g.opt, td, beta))
         return fail(PG_ERR_PARAMS, "parameter set %s: a tensor-core sum could leave the exact fp32 window",
                     g.params_set == 1 ? "pg12_small" : "pg12_v1");
-    PG_CUDA(cudaMemcpyToSymbol(dev::g_tc, &tt, sizeof(tt)));
-    static ChainParams cp;
-    host::derive_chain(g.opt, cp);
-    PG_CUDA(cudaMemcpyToSymbol(dev::c_beta, cp.beta, sizeof(cp.beta)));
+    PG_CUDA(cudaMemcpyToSymbol(dev::g_tc, &td, sizeof(td)));
+    PG_CUDA(cudaMemcpyToSymbol(dev::c_beta, beta, sizeof(beta)));
     return PG_OK;
 }
 
@@ -1170,24 +1162,21 @@ cudaError_t launch_dependent(void (*kernel)(KArgs...), unsigned grid, unsigned b
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
-// Tensor-core kernels: one CTA per SM at most, each CTA four 128-row units at a time.
+// Tensor-core kernels: one CTA per SM at most; with fewer units than four per
+// SM the CTAs' groups fill evenly (tc_first_unit).
 unsigned tc_grid(uint64_t n) {
     const uint64_t units = (n + dev::kTcGroup - 1) / dev::kTcGroup;
-    const uint64_t want = (units + dev::kTcGroups - 1) / dev::kTcGroups;
-    return (unsigned)(want < (uint64_t)g.sms ? want : (uint64_t)g.sms);
+    return (unsigned)(units < (uint64_t)g.sms ? units : (uint64_t)g.sms);
 }
 
 pg_status launch_tc_sponge(const uint64_t *rows, uint64_t n, uint64_t w, uint64_t *out, cudaStream_t st, bool dependent,
                            int kid) {
     if (n == 0) return PG_OK;
     const int vec16 = ((w % 2) == 0 && (reinterpret_cast<uintptr_t>(rows) % 16) == 0) ? 1 : 0;
-    const uint64_t units = (n + dev::kTcGroup - 1) / dev::kTcGroup;
-    // fewer units than the big CTAs' groups on the whole GPU: one group per CTA
-    const bool one = units < (uint64_t)g.sms * dev::kTcGroups;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(one ? (unsigned)units : tc_grid(n));
-    cfg.blockDim = dim3(one ? dev::kTcGroup : dev::kTcThreads);
-    cfg.dynamicSmemBytes = one ? dev::TcL1::kBytes : dev::TcL::kBytes;
+    cfg.gridDim = dim3(tc_grid(n));
+    cfg.blockDim = dim3(dev::kTcThreads);
+    cfg.dynamicSmemBytes = dev::TcL::kBytes;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1195,8 +1184,7 @@ pg_status launch_tc_sponge(const uint64_t *rows, uint64_t n, uint64_t w, uint64_
     cfg.attrs = attr;
     cfg.numAttrs = dependent ? 1 : 0;
     ProfScope prof(kid, st, n * ((w + kRate - 1) / kRate));
-    if (one) PG_CUDA(cudaLaunchKernelEx(&cfg, dev::k_tc_sponge<1, false>, rows, n, w, vec16, out));
-    else PG_CUDA(cudaLaunchKernelEx(&cfg, dev::k_tc_sponge<dev::kTcGroups, dev::kTcChain>, rows, n, w, vec16, out));
+    PG_CUDA(cudaLaunchKernelEx(&cfg, dev::k_tc_sponge, rows, n, w, vec16, out));
     return PG_OK;
 }
 
@@ -1205,15 +1193,8 @@ pg_status launch_tc_sponge(const uint64_t *rows, uint64_t n, uint64_t w, uint64_
 pg_status launch_leaves_stream(const uint64_t *rows, uint64_t n, uint64_t w, uint64_t *out, const uint32_t *ready,
                                const dev::ChunkMap &cm, cudaStream_t st) {
     const int vec16 = ((w % 2) == 0 && (reinterpret_cast<uintptr_t>(rows) % 16) == 0) ? 1 : 0;
-    const uint64_t units = (n + dev::kTcGroup - 1) / dev::kTcGroup;
-    const bool one = units < (uint64_t)g.sms * dev::kTcGroups;
     ProfScope prof(kIdTcLeaves, st, n * ((w + kRate - 1) / kRate));
-    if (one)
-        dev::k_tc_leaves_stream<1, false><<<(unsigned)units, dev::kTcGroup, dev::TcL1::kBytes, st>>>(rows, n, w, vec16, out,
-                                                                                                  ready, cm);
-    else
-        dev::k_tc_leaves_stream<dev::kTcGroups, dev::kTcChain>
-            <<<tc_grid(n), dev::kTcThreads, dev::TcL::kBytes, st>>>(rows, n, w, vec16, out, ready, cm);
+    dev::k_tc_leaves_stream<<<tc_grid(n), dev::kTcThreads, dev::TcL::kBytes, st>>>(rows, n, w, vec16, out, ready, cm);
     PG_CUDA(cudaGetLastError());
     return PG_OK;
 }
@@ -1766,15 +1747,10 @@ pg_status pg_init(int device, const char *params_path) {
     s = upload_tables();
     if (s != PG_OK) return s;
     PG_CUDA(cudaFuncSetAttribute(dev::k_tc_permute, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dev::TcL::kBytes));
-    PG_CUDA(cudaFuncSetAttribute(dev::k_tc_sponge<dev::kTcGroups, dev::kTcChain>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dev::TcL::kBytes));
-    PG_CUDA(cudaFuncSetAttribute(dev::k_tc_sponge<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)dev::TcL1::kBytes));
+    PG_CUDA(cudaFuncSetAttribute(dev::k_tc_sponge, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dev::TcL::kBytes));
     PG_CUDA(cudaFuncSetAttribute(dev::k_tc_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dev::TcL::kBytes));
-    PG_CUDA(cudaFuncSetAttribute(dev::k_tc_leaves_stream<dev::kTcGroups, dev::kTcChain>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dev::TcL::kBytes));
-    PG_CUDA(cudaFuncSetAttribute(dev::k_tc_leaves_stream<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)dev::TcL1::kBytes));
+    PG_CUDA(cudaFuncSetAttribute(dev::k_tc_leaves_stream, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)dev::TcL::kBytes));
     {
         const int ns = ntt_upload_constants();
         if (ns != PG_OK) return (pg_status)ns;

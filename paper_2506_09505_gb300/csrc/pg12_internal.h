@@ -97,6 +97,34 @@ struct TcTables {
 };
 static_assert(sizeof(TcTables) % 16 == 0, "tables are copied in 16-byte pieces");
 
+// The tables the kernels read (TcTables is the exported form).  They differ
+// from TcTables in three ways:
+//   - every matrix is multiplied by R^6, R = 2^64: the S-box outputs it meets
+//     are x^7 R^-6 (field.cuh, msbox), and a_zcap holds (c_0[j])^7 R^-6;
+//   - the bias carries the constants that follow the contraction: the bias of
+//     kind k (TcBias) makes row i come out as (M y)_i + const_k[i], so no round
+//     constant is added on the integer pipes after the first.  b_bias holds, per
+//     row group i, two core matrices whose column k (of 16) has 4 u_b(k, i) in
+//     row b; a_bias selects the column: Z, H_0 .. H_7, Z with H_j the core
+//     matrix of 2^-13 in column j of 8 identical rows and Z zero, so that the K
+//     chunk pair (H_k, Z) picks kind k < 8 and (Z, H_(k-8)) kind k >= 8;
+//   - the offset the bias cancels is that of tc_combine (tcgen05.cuh): the
+//     columns' 23-bit fractions, with the constant bytes its permutes bring.
+enum TcBias { kBiasDense = 0 /* + round 0..7 */, kBiasUa = 8, kBiasUb = 9, kBiasW = 10, kBiasKinds = 11 };
+struct TcDev {
+    uint16_t m[kTcN * kTcK];
+    uint16_t pre[kTcN * kTcK];
+    uint16_t b_bias[kT * 2 * 64];
+    uint16_t a_bias[10 * 64];
+    uint16_t a_zcap[4 * 64];
+    uint16_t vpa[kTcUa * 8 * kTcK];
+    uint16_t vpb[kTcN * kTcK];
+    uint16_t bs[kTcN * kTcK];
+    uint16_t w1[kTcN * kTcK];
+    uint16_t w2[kTcN * kTcK];
+};
+static_assert(sizeof(TcDev) % 16 == 0, "tables are copied in 16-byte pieces");
+
 // Records the text returned by pg_last_error() and passes `status` through.
 int set_error(int status, const char *fmt, ...);
 
@@ -147,6 +175,9 @@ void derive_chain(const OptParams &op, ChainParams &cp);
 // Digit tables of the tensor-core contractions for an optimised set; false if
 // a sum could leave the exact window (every table is checked).
 bool build_tc_tables(const OptParams &op, TcTables &tt);
+// The same for the kernels' tables; beta receives the chain's coefficients
+// times R^7 (R^6 for the S-box outputs, R for the Montgomery reduction).
+bool build_tc_dev(const OptParams &op, TcDev &td, uint64_t beta[kRP][kRP]);
 // The bias blocks every tensor-core contraction adds (TcTables::a_bias and
 // b_bias) and their digits u_b.
 void tc_bias_blocks(uint16_t a_bias[128], uint16_t b_bias[128], int u[8]);

@@ -3,14 +3,15 @@
 //
 // Alg. 1's full rounds are x <- M S(x + c_r); the 12x12 products M y of a
 // whole group are one tensor-core contraction of byte limbs (the digit scheme
-// of TcTables in pg12_internal.h):
+// of TcTables and TcDev in pg12_internal.h):
 //
-//   thread t: y_j = S(x_j + c_rj), its 8 bytes -> row t of A (fp16
-//             subnormals, bits = byte), in shared memory
+//   thread t: y_j = S(x_j) R^-6 (Montgomery products, field.cuh), its 8 bytes
+//             -> row t of A (fp16 subnormals, bits = byte), in shared memory
 //   leader  : D[128 x 96] = A[128 x 96] * B^T + bias   (7 tcgen05.mma, K = 16
 //             each, fp32 accumulators in tensor memory), commit -> mbarrier
 //   thread t: reads row t of D (tcgen05.ld), y_i = sum_b 2^(8b) bits(D[t][8i+b])
-//             folded mod p
+//             folded mod p: M is stored times R^6 and the bias holds the next
+//             round's constants, so this is the next S-box input
 //
 // The 22 partial rounds (Alg. 1, MDSPartial) run in their unrolled form
 // (ChainParams): the dot products U_q with the partial rounds' input and the
@@ -44,20 +45,18 @@ constexpr int kTcUStore = kTcN;                 // columns 96..119 of a region h
 // tensor-memory columns one CTA of `groups` groups allocates (a power of two)
 constexpr int tc_tmem_alloc(int groups) { return groups <= 1 ? 128 : groups <= 2 ? 256 : 512; }
 
-// byte offsets of the tables inside TcTables (and inside its shared-memory copy)
-constexpr uint32_t kTabM = offsetof(TcTables, m), kTabPre = offsetof(TcTables, pre);
-constexpr uint32_t kTabBBias = offsetof(TcTables, b_bias), kTabABias = offsetof(TcTables, a_bias);
-constexpr uint32_t kTabZcap = offsetof(TcTables, a_zcap);
-constexpr uint32_t kTabVpa = offsetof(TcTables, vpa), kTabVpb = offsetof(TcTables, vpb), kTabBs = offsetof(TcTables, bs);
-constexpr uint32_t kTabW1 = offsetof(TcTables, w1), kTabW2 = offsetof(TcTables, w2);
-constexpr size_t kTabCore = offsetof(TcTables, vpa);  // what kernels without the chain copy
+// byte offsets of the tables inside TcDev (and inside its shared-memory copy)
+constexpr uint32_t kTabM = offsetof(TcDev, m), kTabPre = offsetof(TcDev, pre);
+constexpr uint32_t kTabBBias = offsetof(TcDev, b_bias), kTabABias = offsetof(TcDev, a_bias);
+constexpr uint32_t kTabZcap = offsetof(TcDev, a_zcap);
+constexpr uint32_t kTabVpa = offsetof(TcDev, vpa), kTabVpb = offsetof(TcDev, vpb), kTabBs = offsetof(TcDev, bs);
+constexpr uint32_t kTabW1 = offsetof(TcDev, w1), kTabW2 = offsetof(TcDev, w2);
 static_assert(kTabVpa % 128 == 0 && kTabVpb % 128 == 0 && kTabBs % 128 == 0 && kTabW1 % 128 == 0 &&
-                  kTabW2 % 128 == 0 &&
-                  kTabBBias % 128 == 0 && kTabZcap % 128 == 0,
+                  kTabW2 % 128 == 0 && kTabBBias % 128 == 0 && kTabABias % 128 == 0 && kTabZcap % 128 == 0,
               "tables are 128-byte aligned");
 
-__device__ __align__(16) TcTables g_tc;     // uploaded with the other constant tables
-__constant__ uint64_t c_beta[kRP][kRP];     // ChainParams::beta
+__device__ __align__(16) TcDev g_tc;        // uploaded with the other constant tables
+__constant__ uint64_t c_beta[kRP][kRP];     // the chain's coefficients times R^7
 
 // One group's share of the CTA's shared memory and tensor memory.
 struct TcGroup {
@@ -84,28 +83,29 @@ __device__ __forceinline__ uint64_t tc_get(const TcGroup &G, int j) {
 
 // One contraction into the group's D (columns 0 .. n-1): the group meets
 // (its A stores visible to the tensor cores, its earlier tensor-memory
-// accesses done), thread 0 issues the bias block (when `bias`: D starts at
-// the bias; else D accumulates) and kblocks K = 16 blocks of A (cells 8..11
-// from the zero-capacity block when z) against the table at byte offset
-// b_off with b_chunks input words per row group, and commits; every thread
-// waits.  Returns false, in every thread of the group, once a wait of the
-// group has run out.
-__device__ __forceinline__ bool tc_contract(TcGroup &G, uint32_t b_off, uint32_t b_chunks, int n, int kblocks,
-                                            bool bias, bool z) {
+// accesses done), thread 0 issues the bias block of kind `bias` (D starts at
+// the bias; bias < 0: D accumulates) and the six K = 16 blocks of A (cells
+// 8..11 from the zero-capacity block when z) against the table at byte offset
+// b_off, and commits; every thread waits.  Returns false, in every thread of
+// the group, once a wait of the group has run out.
+__device__ __forceinline__ bool tc_contract(TcGroup &G, uint32_t b_off, int n, int bias, bool z) {
     fence_async_smem();   // this thread's A stores -> the tensor cores' proxy
     tc_fence_before();    // its tensor-memory accesses are complete
     if (group_sync_or(G.bar, G.failed)) return false;
     if (G.t == 0) {
         tc_fence_after();
         const uint32_t idesc = tc_idesc(n);
-        const uint32_t sbo_b = b_chunks * kTcAChunk, sbo_a = kTcAChunks * kTcAChunk;
-        if (bias)
-            tc_mma(G.tmem, tc_desc(G.tab + kTabABias, kTcAChunk, 0), tc_desc(G.tab + kTabBBias, kTcAChunk, 0), idesc,
-                   0);
-        for (int kb = 0; kb < kblocks; ++kb) {
+        const uint32_t sbo = kTcAChunks * kTcAChunk;
+        if (bias >= 0) {
+            // K chunks (H_k, Z) for kind k < 8, (Z, H_(k-8)) above: see TcDev::a_bias
+            const uint32_t first = bias < 8 ? 1u + bias : 0u, lbo = bias < 8 ? 8u - bias : bias - 7u;
+            tc_mma(G.tmem, tc_desc(G.tab + kTabABias + first * kTcAChunk, lbo * kTcAChunk, 0),
+                   tc_desc(G.tab + kTabBBias, kTcAChunk, 2 * kTcAChunk), idesc, 0);
+        }
+        for (int kb = 0; kb < kTcK / 16; ++kb) {
             const uint64_t a = (z && kb >= 4) ? tc_desc(G.tab + kTabZcap + (kb - 4) * 2 * kTcAChunk, kTcAChunk, 0)
-                                              : tc_desc(G.a_addr + kb * 2 * kTcAChunk, kTcAChunk, sbo_a);
-            tc_mma(G.tmem, a, tc_desc(G.tab + b_off + kb * 2 * kTcAChunk, kTcAChunk, sbo_b), idesc, 1);
+                                              : tc_desc(G.a_addr + kb * 2 * kTcAChunk, kTcAChunk, sbo);
+            tc_mma(G.tmem, a, tc_desc(G.tab + b_off + kb * 2 * kTcAChunk, kTcAChunk, sbo), idesc, 1);
         }
         tc_commit(G.mbar);
     }
@@ -116,46 +116,54 @@ __device__ __forceinline__ bool tc_contract(TcGroup &G, uint32_t b_off, uint32_t
     return true;
 }
 
-// Dense layer of a full round (table at m_off) on the S-box outputs in A;
-// rows 0..rows-1 of the result go to x.  z: round 0 of states whose
-// capacity entered as zero (A holds cells 0..7; cells 8..11 come from the
-// constant zcap block).
-__device__ __forceinline__ bool tc_dense(TcGroup &G, uint32_t m_off, bool z, int rows, uint64_t (&x)[kT]) {
-    if (!tc_contract(G, m_off, kTcAChunks, kTcN, 6, true, z)) return false;
-    const uint32_t lane_base = G.tmem + ((uint32_t)(G.t & ~31) << 16);
+// Rows I .. ROWS-1 of D (two at a time) into x[].
+template <int ROWS, int I = 0>
+__device__ __forceinline__ void tc_load_rows(uint32_t lane_base, uint64_t (&x)[kT]) {
 #pragma unroll
-    for (int i = 0; i < kT; i += 2) {
-        if (i < rows) {
-            uint32_t w[16];
-            tmem_ld16(lane_base + 8 * i, w);
-            x[i] = tc_combine(w);
-            x[i + 1] = tc_combine(w + 8);
-        }
+    for (int i = I; i < ROWS; i += 2) {
+        uint32_t w[16];
+        tmem_ld16(lane_base + 8 * i, w);
+        x[i] = tc_combine(w);
+        x[i + 1] = tc_combine(w + 8);
     }
+}
+
+// Dense layer of round r (table at m_off) on the S-box outputs in A, plus the
+// next constants (the bias of kind r); with `digest` only rows 0..3 of the
+// result are formed.  z: round 0 of states whose capacity entered as zero (A
+// holds cells 0..7; cells 8..11 come from the constant zcap block).
+__device__ __forceinline__ bool tc_dense(TcGroup &G, uint32_t m_off, int r, bool z, bool digest, uint64_t (&x)[kT]) {
+    if (!tc_contract(G, m_off, kTcN, kBiasDense + r, z)) return false;
+    const uint32_t lane_base = G.tmem + ((uint32_t)(G.t & ~31) << 16);
+    tc_load_rows<kDigest>(lane_base, x);
+    if (!digest) tc_load_rows<kT, kDigest>(lane_base, x);
     return true;
 }
 
 #ifndef PG12_TC_MAC_UNROLL
-#define PG12_TC_MAC_UNROLL 2  // 1: measured 0.5% slower
+#define PG12_TC_MAC_UNROLL 4
 #endif
 constexpr int kTcMacUnroll = PG12_TC_MAC_UNROLL;
-// One half of the chain: s_q = S(c + k_q) for q = q0 .. q1 - 1, each into
-// A's chunk q - q0; between them c = U_q + sum_(r = q0 .. q) beta[q][r] s_r,
-// U_q the word in tensor-memory column kTcUStore + 2 (q - u0).
+// One half of the chain: s_q = S(c_q + k_q) for q = q0 .. q1 - 1, each into
+// A's chunk q - q0, from c = c_q0 + k_q0; between them c_(q+1) + k_(q+1) =
+// U_q + sum_(r = q0 .. q) beta[q][r] s_r, U_q (its bias includes k_(q+1)) the
+// word in tensor-memory column kTcUStore + 2 (q - u0).
 __device__ __forceinline__ void chain_half(const TcGroup &G, uint32_t lane_base, uint64_t c, int q0, int q1, int u0) {
 #pragma unroll 1
     for (int q = q0;; ++q) {
-        tc_put(G, q - q0, sbox(add_canon(c, c_dev.part_rc[q])));
+        const uint64_t s = msbox(c);
+        tc_put(G, q - q0, s);
         if (q == q1 - 1) break;
-        Acc A;
-        acc_init(A, tmem_ld_word(lane_base + kTcUStore + 2 * (q - u0)));
+        MAcc A;
+        macc_init(A, tmem_ld_word(lane_base + kTcUStore + 2 * (q - u0)));
 #pragma unroll kTcMacUnroll
-        for (int r = q0; r <= q; ++r) acc_mac(A, tc_get(G, r - q0), c_beta[q][r]);
-        c = acc_reduce(A);
+        for (int r = q0; r < q; ++r) macc(A, tc_get(G, r - q0), c_beta[q][r]);
+        macc(A, s, c_beta[q][q]);
+        c = macc_reduce(A);
     }
 }
 
-// Rows 0 .. rows-1 of D combined into words, stored at tensor-memory columns
+// Rows 0 .. ROWS-1 of D combined into words, stored at tensor-memory columns
 // kTcUStore + 2 i.
 template <int ROWS>
 __device__ __forceinline__ void tc_store_rows(uint32_t lane_base) {
@@ -169,23 +177,24 @@ __device__ __forceinline__ void tc_store_rows(uint32_t lane_base) {
 }
 
 // The 22 partial rounds in their unrolled form, after round 3's dense layer
-// (A still holds round 3's S-box bytes y3, x holds x^(0) = P y3).
+// (A still holds round 3's S-box bytes y3, x holds x^(0) = P y3, cell 0 with
+// k_0 added); x leaves with round 4's constants added.
 __device__ __forceinline__ bool tc_partial(TcGroup &G, uint64_t (&x)[kT]) {
     const uint32_t lane_base = G.tmem + ((uint32_t)(G.t & ~31) << 16);
     // U_0 .. U_9 as words
-    if (!tc_contract(G, kTabVpa, kTcAChunks, kTcUa * 8, 6, true, false)) return false;
+    if (!tc_contract(G, kTabVpa, kTcUa * 8, kBiasUa, false)) return false;
     tc_store_rows<kTcUa>(lane_base);
     // U_10 .. U_21 as column sums in D (A still holds y3)
-    if (!tc_contract(G, kTabVpb, kTcAChunks, kTcN, 6, true, false)) return false;
+    if (!tc_contract(G, kTabVpb, kTcN, kBiasUb, false)) return false;
     // first half: s_0 .. s_10 into A's chunks 0..10
     chain_half(G, lane_base, x[0], 0, kTcSplit, 0);
     // D += their terms in c_11 .. c_21: the second half's U'_q (q = 10 .. 20) and U_21, as words
-    if (!tc_contract(G, kTabBs, kTcAChunks, kTcN, 6, false, false)) return false;
+    if (!tc_contract(G, kTabBs, kTcN, -1, false)) return false;
     tc_store_rows<kT>(lane_base);
     // the deferred updates W s, from s_0 .. s_10 now, s_11 .. s_21 after the second half
-    if (!tc_contract(G, kTabW1, kTcAChunks, kTcN, 6, true, false)) return false;
+    if (!tc_contract(G, kTabW1, kTcN, kBiasW, false)) return false;
     chain_half(G, lane_base, tmem_ld_word(lane_base + kTcUStore), kTcSplit, kRP, kTcUa);
-    if (!tc_contract(G, kTabW2, kTcAChunks, kTcN, 6, false, false)) return false;
+    if (!tc_contract(G, kTabW2, kTcN, -1, false)) return false;
     // cell 0 = c_22 = U_21 + (W s)_0, cell i = x_i^(0) + (W s)_i
     const uint64_t u21 = tmem_ld_word(lane_base + kTcUStore + 2 * (kRP - 1 - kTcUa));
 #pragma unroll
@@ -198,78 +207,55 @@ __device__ __forceinline__ bool tc_partial(TcGroup &G, uint64_t (&x)[kT]) {
     return true;
 }
 
-// The 22 partial rounds on the integer pipes, state in registers (the
-// MDSPartial form of Alg. 1: 12 products for cell 0, 11 multiply-adds).
-__device__ __forceinline__ void partial_regs(uint64_t (&x)[kT]) {
-#pragma unroll 1
-    for (int q = 0; q < kRP; ++q) {
-        const uint64_t x0 = sbox(add_canon(x[0], c_dev.part_rc[q]));
-        Acc A;
-        acc_zero(A);
-        acc_mac(A, x0, c_dev.part_v[q][0]);
-#pragma unroll
-        for (int j = 1; j < kT; ++j) acc_mac(A, x[j], c_dev.part_v[q][j]);
-#pragma unroll
-        for (int i = 1; i < kT; ++i) x[i] = mul_add(c_dev.part_w[q][i], x0, x[i]);
-        x[0] = acc_reduce(A);
-    }
-}
-
-// The permutation on x, the thread's state in registers (weak words in,
-// weak words out), with the same zcap / digest shortcuts as permute_slot.
-// Each round's twelve S-boxes and twelve output folds are unrolled (the
-// state never leaves registers).  CHAIN: the partial rounds in their
-// unrolled form on the tensor cores (tc_partial); else on the integer pipes
-// (partial_regs).
-template <bool CHAIN>
+// The permutation on x, the thread's state in registers (weak words in, weak
+// words out).  zcap: cells 8..11 enter as zero (their round 0 S-box outputs
+// are constants, read from a_zcap); digest: only cells 0..3 of the result are
+// read and formed.  Each round's twelve S-boxes and twelve output rows are
+// unrolled (the state never leaves registers).  Round 0's constants are added
+// here, all later ones by the contractions' biases.
 __device__ __forceinline__ bool tc_permute(TcGroup &G, uint64_t (&x)[kT], bool zcap, bool digest) {
+#pragma unroll
+    for (int j = 0; j < kT; ++j) x[j] = add_canon(x[j], c_dev.full_rc[0][j]);
 #pragma unroll 1
     for (int r = 0; r < kRF; ++r) {
         const bool z = zcap && r == 0;
 #pragma unroll
-        for (int j = 0; j < kRate; ++j) tc_put(G, j, sbox(add_canon(x[j], c_dev.full_rc[r][j])));
+        for (int j = 0; j < kRate; ++j) tc_put(G, j, msbox(x[j]));
         if (!z) {
 #pragma unroll
-            for (int j = kRate; j < kT; ++j) tc_put(G, j, sbox(add_canon(x[j], c_dev.full_rc[r][j])));
+            for (int j = kRate; j < kT; ++j) tc_put(G, j, msbox(x[j]));
         }
         const bool mid = r == kRF / 2 - 1;
-        if (!tc_dense(G, mid ? kTabPre : kTabM, z, digest && r == kRF - 1 ? kDigest : kT, x)) return false;
-        if (mid) {
-            if (CHAIN) {
-                if (!tc_partial(G, x)) return false;
-            } else {
-                partial_regs(x);
-            }
-        }
+        if (!tc_dense(G, mid ? kTabPre : kTabM, r, z, digest && r == kRF - 1, x)) return false;
+        if (mid && !tc_partial(G, x)) return false;
     }
     return true;
 }
 
-// Shared-memory layout of a CTA of GROUPS groups: the tables (all of them
-// with CHAIN, else the full rounds' part), then each group's A operand, then
-// the barriers.
-template <int GROUPS, bool CHAIN>
+// Shared-memory layout of a CTA of GROUPS groups: the tables, then each
+// group's A operand, then the barriers.
+template <int GROUPS>
 struct TcLayout {
     static_assert(GROUPS * kTcRegion <= 512, "the groups' tensor memory exceeds the SM's");
     static constexpr int kTmemCols = tc_tmem_alloc(GROUPS);
-    static constexpr size_t kTableBytes = CHAIN ? sizeof(TcTables) : kTabCore;
     static constexpr size_t kTables = 0;
-    static constexpr size_t kA = (kTableBytes + 127) & ~(size_t)127;
+    static constexpr size_t kA = (sizeof(TcDev) + 127) & ~(size_t)127;
     static constexpr size_t kBar = kA + (size_t)GROUPS * kTcABytes;
     static constexpr size_t kBcast = kBar + 8 * GROUPS + 16;
     static constexpr size_t kBytes = kBcast + 4 * GROUPS;
+    static_assert(kBytes <= 232448, "a block has at most 227 KB of shared memory");
 };
 
 __device__ int g_tc_fault;  // set when a tensor-core wait ran out (read by pg_device_faults)
 
 // Prologue of a tensor-core kernel: tables into shared memory, the groups'
 // barriers, one tensor-memory allocation for all groups.
-template <int GROUPS, bool CHAIN>
+template <int GROUPS>
 __device__ __forceinline__ TcGroup tc_setup(uint8_t *sm) {
-    using L = TcLayout<GROUPS, CHAIN>;
+    using L = TcLayout<GROUPS>;
     const uint4 *src = reinterpret_cast<const uint4 *>(&g_tc);
     uint4 *dst = reinterpret_cast<uint4 *>(sm + L::kTables);
-    for (unsigned i = threadIdx.x; i < L::kTableBytes / 16; i += blockDim.x) dst[i] = __ldg(src + i);
+    for (unsigned i = threadIdx.x; i < sizeof(TcDev) / 16; i += blockDim.x) dst[i] = __ldg(src + i);
     uint64_t *bars = reinterpret_cast<uint64_t *>(sm + L::kBar);
     uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + GROUPS);
     if (threadIdx.x == 0) {
@@ -314,9 +300,9 @@ __device__ __forceinline__ uint32_t group_fetch_add(TcGroup &G, uint32_t *counte
 // Epilogue: every group is done with tensor memory; the allocating warp
 // frees it.  A group whose wait ran out records the fault and gives its
 // last contraction one more bounded wait before the memory is freed.
-template <int GROUPS, bool CHAIN>
+template <int GROUPS>
 __device__ __forceinline__ void tc_teardown(uint8_t *sm, TcGroup &G) {
-    using L = TcLayout<GROUPS, CHAIN>;
+    using L = TcLayout<GROUPS>;
     if (G.failed) {
         atomicExch(&g_tc_fault, 1);
         if (G.t == 0) mbar_wait(G.mbar, G.phase ^ 1u);

@@ -4,7 +4,7 @@
 // exact byte-limb arithmetic around a contraction: a 64-bit word split into
 // its 8 bytes as fp16 subnormals (bits = byte) for an A operand, and the
 // combination of eight fp32 column sums (bits 0x3E800000 + offset + Z, see
-// TcTables) back into a word mod p.
+// TcDev) back into a word mod p.
 //
 // Every contraction here is D[128 x N] (+)= A[128 x K] B[N x K]^T with fp16
 // A and B in K-major, unswizzled 8 x 8 core matrices of 128 contiguous
@@ -112,27 +112,42 @@ __device__ __forceinline__ void tmem_st_words(uint32_t taddr, uint64_t a, uint64
                  : "memory");
 }
 
-// y = sum_b 2^(8b) w[b] + x mod p for eight column words w[b] < 2^31 and a
-// 64-bit x: two 56-bit sums lo = sum_(b<4), hi = sum_(b>=4) (IMAD.WIDE with
-// the running sum as addend), V = lo + hi 2^32 + x < 2^89 = lo' + h 2^64 with
-// lo' = lo + x + hi.lo 2^32 and h = hi.hi + carries, then the fold
-// (2^64 = 2^32 - 1).
-__device__ __forceinline__ uint64_t tc_combine(const uint32_t *w, uint64_t x = 0) {
-    uint64_t lo = madw(w[1], 1u << 8, (uint64_t)w[0]);
-    lo = madw(w[2], 1u << 16, lo);
-    lo = madw(w[3], 1u << 24, lo);
-    uint64_t hi = madw(w[5], 1u << 8, (uint64_t)w[4]);
-    hi = madw(w[6], 1u << 16, hi);
-    hi = madw(w[7], 1u << 24, hi);
-    uint32_t l0, l1, h;
+// y = sum_b 2^(8b) m[b] (+ x) mod p for eight column words w[b] = 0x3F000000 +
+// m[b], m[b] < 2^23, plus the constant bytes noted below, which the bias
+// cancels (build_tc_dev).  The m[b] of b = 0, 3, 6 occupy disjoint bytes of the
+// sum, as do b = 1, 4, 7 and b = 2, 5, so byte permutes build three 80-bit
+// numbers and two carry chains add them; words w[1] and w[2] leave their top
+// byte 0x3F in bytes 0 and 0, 1, and w[6], w[7] theirs at 2^72 and 2^80.  This
+// keeps the combination off the multiplier pipe, which the S-boxes fill: with
+// six IMAD.WIDE in place of the permutes a 2^22 x 8 tree took 6.11 ms, with
+// every other row in either form 5.88 ms, with this one for all rows 5.76 ms.
+__device__ __forceinline__ void tc_bytes_sum(const uint32_t *w, uint32_t &s0, uint32_t &s1, uint32_t &s2) {
+    const uint32_t a0 = __byte_perm(w[0], w[3], 0x4210), a1 = __byte_perm(w[3], w[6], 0x5421);
+    const uint32_t b0 = __byte_perm(w[1], w[1], 0x2103), b1 = __byte_perm(w[4], w[7], 0x4210);
+    const uint32_t c0 = __byte_perm(w[2], w[2], 0x1033), c1 = __byte_perm(w[2], w[5], 0x6542);
     asm("add.cc.u32 %0, %3, %5;\n\t"
         "addc.cc.u32 %1, %4, %6;\n\t"
-        "addc.u32 %2, %8, 0;\n\t"
-        "add.cc.u32 %1, %1, %7;\n\t"
+        "addc.u32 %2, %9, %10;\n\t"
+        "add.cc.u32 %0, %0, %7;\n\t"
+        "addc.cc.u32 %1, %1, %8;\n\t"
         "addc.u32 %2, %2, 0;"
-        : "=r"(l0), "=r"(l1), "=r"(h)
-        : "r"(lo32(lo)), "r"(hi32(lo)), "r"(lo32(x)), "r"(hi32(x)), "r"(lo32(hi)), "r"(hi32(hi)));
-    return fold(((uint64_t)l1 << 32) | l0, (uint64_t)h, 0);
+        : "=&r"(s0), "=&r"(s1), "=&r"(s2)
+        : "r"(a0), "r"(a1), "r"(b0), "r"(b1), "r"(c0), "r"(c1), "r"(w[6] >> 16), "r"(w[7] >> 8));
+}
+__device__ __forceinline__ uint64_t tc_combine(const uint32_t *w) {
+    uint32_t s0, s1, s2;
+    tc_bytes_sum(w, s0, s1, s2);
+    return fold_small(s0, s1, s2);
+}
+__device__ __forceinline__ uint64_t tc_combine(const uint32_t *w, uint64_t x) {
+    uint32_t s0, s1, s2;
+    tc_bytes_sum(w, s0, s1, s2);
+    asm("add.cc.u32 %0, %0, %3;\n\t"
+        "addc.cc.u32 %1, %1, %4;\n\t"
+        "addc.u32 %2, %2, 0;"
+        : "+r"(s0), "+r"(s1), "+r"(s2)
+        : "r"(lo32(x)), "r"(hi32(x)));
+    return fold_small(s0, s1, s2);
 }
 
 // The 8 bytes of y as fp16 subnormals whose bit patterns are the bytes
