@@ -76,14 +76,9 @@ __device__ __forceinline__ void tc_put(const TcGroup &G, int j, uint64_t y) {
     *reinterpret_cast<uint4 *>(G.a + ((G.t >> 3) * kTcAChunks + j) * kTcAChunk + (G.t & 7) * 16) = tc_bytes(y);
 }
 
-// The word y that tc_put wrote to row t's chunk j (the low byte of each fp16).
-__device__ __forceinline__ uint64_t tc_get(const TcGroup &G, int j) {
-    return tc_word(*reinterpret_cast<const uint4 *>(G.a + ((G.t >> 3) * kTcAChunks + j) * kTcAChunk + (G.t & 7) * 16));
-}
-
 // One contraction into the group's D (columns 0 .. n-1): the group meets
 // (its A stores visible to the tensor cores, its earlier tensor-memory
-// accesses done), thread 0 issues the bias block of kind `bias` (D starts at
+// accesses done), a lane of warp 0 issues the bias block of kind `bias` (D starts at
 // the bias; bias < 0: D accumulates) and the six K = 16 blocks of A (cells
 // 8..11 from the zero-capacity block when z) against the table at byte offset
 // b_off, and commits; every thread waits.  Returns false, in every thread of
@@ -92,22 +87,31 @@ __device__ __forceinline__ bool tc_contract(TcGroup &G, uint32_t b_off, int n, i
     fence_async_smem();   // this thread's A stores -> the tensor cores' proxy
     tc_fence_before();    // its tensor-memory accesses are complete
     if (group_sync_or(G.bar, G.failed)) return false;
-    if (G.t == 0) {
+    if (G.t < 32) {
         tc_fence_after();
         const uint32_t idesc = tc_idesc(n);
         const uint32_t sbo = kTcAChunks * kTcAChunk;
-        if (bias >= 0) {
-            // K chunks (H_k, Z) for kind k < 8, (Z, H_(k-8)) above: see TcDev::a_bias
-            const uint32_t first = bias < 8 ? 1u + bias : 0u, lbo = bias < 8 ? 8u - bias : bias - 7u;
-            tc_mma(G.tmem, tc_desc(G.tab + kTabABias + first * kTcAChunk, lbo * kTcAChunk, 0),
-                   tc_desc(G.tab + kTabBBias, kTcAChunk, 2 * kTcAChunk), idesc, 0);
+        // warp-uniform operands and an elected lane: the descriptors stay in
+        // uniform registers, which the instruction reads
+        const uint32_t d = __shfl_sync(0xFFFFFFFFu, G.tmem, 0);
+        const uint64_t a0 = tc_desc(__shfl_sync(0xFFFFFFFFu, G.a_addr, 0), kTcAChunk, sbo);
+        const uint64_t b0 = tc_desc(G.tab + b_off, kTcAChunk, sbo);
+        if (tc_elect()) {
+            if (bias >= 0) {
+                // K chunks (H_k, Z) for kind k < 8, (Z, H_(k-8)) above: see TcDev::a_bias
+                const uint32_t first = bias < 8 ? 1u + bias : 0u, lbo = bias < 8 ? 8u - bias : bias - 7u;
+                tc_mma(d, tc_desc(G.tab + kTabABias + first * kTcAChunk, lbo * kTcAChunk, 0),
+                       tc_desc(G.tab + kTabBBias, kTcAChunk, 2 * kTcAChunk), idesc, 0);
+            }
+#pragma unroll
+            for (int kb = 0; kb < kTcK / 16; ++kb) {
+                uint64_t a = a0 + (kb * 2 * kTcAChunk >> 4);
+                if (z && kb >= 4) a = tc_desc(G.tab + kTabZcap + (kb - 4) * 2 * kTcAChunk, kTcAChunk, 0);
+                tc_mma(d, a, b0 + (kb * 2 * kTcAChunk >> 4), idesc, 1);
+            }
+            tc_commit(G.mbar);
         }
-        for (int kb = 0; kb < kTcK / 16; ++kb) {
-            const uint64_t a = (z && kb >= 4) ? tc_desc(G.tab + kTabZcap + (kb - 4) * 2 * kTcAChunk, kTcAChunk, 0)
-                                              : tc_desc(G.a_addr + kb * 2 * kTcAChunk, kTcAChunk, sbo);
-            tc_mma(G.tmem, a, tc_desc(G.tab + b_off + kb * 2 * kTcAChunk, kTcAChunk, sbo), idesc, 1);
-        }
-        tc_commit(G.mbar);
+        __syncwarp();
     }
     const bool ok = mbar_wait(G.mbar, G.phase);
     G.phase ^= 1u;
@@ -119,12 +123,16 @@ __device__ __forceinline__ bool tc_contract(TcGroup &G, uint32_t b_off, int n, i
 // Rows I .. ROWS-1 of D (two at a time) into x[].
 template <int ROWS, int I = 0>
 __device__ __forceinline__ void tc_load_rows(uint32_t lane_base, uint64_t (&x)[kT]) {
+    // the next pair's load is in flight while a pair is combined
+    uint32_t w[2][16];
+    tmem_ld16_start(lane_base + 8 * I, w[0]);
 #pragma unroll
     for (int i = I; i < ROWS; i += 2) {
-        uint32_t w[16];
-        tmem_ld16(lane_base + 8 * i, w);
-        x[i] = tc_combine(w);
-        x[i + 1] = tc_combine(w + 8);
+        const int k = ((i - I) / 2) & 1;
+        tmem_ld_wait();
+        if (i + 2 < ROWS) tmem_ld16_start(lane_base + 8 * (i + 2), w[k ^ 1]);
+        x[i] = tc_combine(w[k]);
+        x[i + 1] = tc_combine(w[k] + 8);
     }
 }
 
@@ -140,25 +148,24 @@ __device__ __forceinline__ bool tc_dense(TcGroup &G, uint32_t m_off, int r, bool
     return true;
 }
 
-#ifndef PG12_TC_MAC_UNROLL
-#define PG12_TC_MAC_UNROLL 4
-#endif
-constexpr int kTcMacUnroll = PG12_TC_MAC_UNROLL;
-// One half of the chain: s_q = S(c_q + k_q) for q = q0 .. q1 - 1, each into
+// One half of the chain: s_q = S(c_q + k_q) for q = q0 .. q0 + 10, each into
 // A's chunk q - q0, from c = c_q0 + k_q0; between them c_(q+1) + k_(q+1) =
 // U_q + sum_(r = q0 .. q) beta[q][r] s_r, U_q (its bias includes k_(q+1)) the
-// word in tensor-memory column kTcUStore + 2 (q - u0).
-__device__ __forceinline__ void chain_half(const TcGroup &G, uint32_t lane_base, uint64_t c, int q0, int q1, int u0) {
-#pragma unroll 1
-    for (int q = q0;; ++q) {
-        const uint64_t s = msbox(c);
-        tc_put(G, q - q0, s);
-        if (q == q1 - 1) break;
+// word in tensor-memory column kTcUStore + 2 (q - u0).  Unrolled, so the s_r
+// stay in registers (reading them back from A's bytes in a loop: a 2^22 x 8
+// tree 5.69 ms against 5.57).
+static_assert(kRP == 2 * kTcSplit, "the halves have the same length");
+__device__ __forceinline__ void chain_half(const TcGroup &G, uint32_t lane_base, uint64_t c, int q0, int u0) {
+    uint64_t s[kTcSplit];
+#pragma unroll
+    for (int q = 0;; ++q) {
+        s[q] = msbox(c);
+        tc_put(G, q, s[q]);
+        if (q == kTcSplit - 1) break;
         MAcc A;
-        macc_init(A, tmem_ld_word(lane_base + kTcUStore + 2 * (q - u0)));
-#pragma unroll kTcMacUnroll
-        for (int r = q0; r < q; ++r) macc(A, tc_get(G, r - q0), c_beta[q][r]);
-        macc(A, s, c_beta[q][q]);
+        macc_init(A, tmem_ld_word(lane_base + kTcUStore + 2 * (q + q0 - u0)));
+#pragma unroll
+        for (int r = 0; r <= q; ++r) macc(A, s[r], c_beta[q + q0][r + q0]);
         c = macc_reduce(A);
     }
 }
@@ -167,11 +174,14 @@ __device__ __forceinline__ void chain_half(const TcGroup &G, uint32_t lane_base,
 // kTcUStore + 2 i.
 template <int ROWS>
 __device__ __forceinline__ void tc_store_rows(uint32_t lane_base) {
+    uint32_t w[2][16];
+    tmem_ld16_start(lane_base, w[0]);
 #pragma unroll
     for (int i = 0; i < ROWS; i += 2) {
-        uint32_t w[16];
-        tmem_ld16(lane_base + 8 * i, w);
-        tmem_st_words(lane_base + kTcUStore + 2 * i, tc_combine(w), tc_combine(w + 8));
+        const int k = (i / 2) & 1;
+        tmem_ld_wait();
+        if (i + 2 < ROWS) tmem_ld16_start(lane_base + 8 * (i + 2), w[k ^ 1]);
+        tmem_st_words(lane_base + kTcUStore + 2 * i, tc_combine(w[k]), tc_combine(w[k] + 8));
     }
     asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
@@ -187,22 +197,25 @@ __device__ __forceinline__ bool tc_partial(TcGroup &G, uint64_t (&x)[kT]) {
     // U_10 .. U_21 as column sums in D (A still holds y3)
     if (!tc_contract(G, kTabVpb, kTcN, kBiasUb, false)) return false;
     // first half: s_0 .. s_10 into A's chunks 0..10
-    chain_half(G, lane_base, x[0], 0, kTcSplit, 0);
+    chain_half(G, lane_base, x[0], 0, 0);
     // D += their terms in c_11 .. c_21: the second half's U'_q (q = 10 .. 20) and U_21, as words
     if (!tc_contract(G, kTabBs, kTcN, -1, false)) return false;
     tc_store_rows<kT>(lane_base);
     // the deferred updates W s, from s_0 .. s_10 now, s_11 .. s_21 after the second half
     if (!tc_contract(G, kTabW1, kTcN, kBiasW, false)) return false;
-    chain_half(G, lane_base, tmem_ld_word(lane_base + kTcUStore), kTcSplit, kRP, kTcUa);
+    chain_half(G, lane_base, tmem_ld_word(lane_base + kTcUStore), kTcSplit, kTcUa);
     if (!tc_contract(G, kTabW2, kTcN, -1, false)) return false;
     // cell 0 = c_22 = U_21 + (W s)_0, cell i = x_i^(0) + (W s)_i
     const uint64_t u21 = tmem_ld_word(lane_base + kTcUStore + 2 * (kRP - 1 - kTcUa));
+    uint32_t w[2][16];
+    tmem_ld16_start(lane_base, w[0]);
 #pragma unroll
     for (int i = 0; i < kT; i += 2) {
-        uint32_t w[16];
-        tmem_ld16(lane_base + 8 * i, w);
-        x[i] = tc_combine(w, i == 0 ? u21 : x[i]);
-        x[i + 1] = tc_combine(w + 8, x[i + 1]);
+        const int k = (i / 2) & 1;
+        tmem_ld_wait();
+        if (i + 2 < kT) tmem_ld16_start(lane_base + 8 * (i + 2), w[k ^ 1]);
+        x[i] = tc_combine(w[k], i == 0 ? u21 : x[i]);
+        x[i + 1] = tc_combine(w[k] + 8, x[i + 1]);
     }
     return true;
 }

@@ -41,6 +41,13 @@ __device__ __forceinline__ void tc_mma(uint32_t d, uint64_t a, uint64_t b, uint3
                  : "memory");
 }
 
+// One lane of a converged warp.
+__device__ __forceinline__ bool tc_elect() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(p));
+    return p != 0;
+}
+
 __device__ __forceinline__ void tc_commit(uint64_t *mbar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_addr(mbar))
                  : "memory");
@@ -94,6 +101,14 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
                  : "r"(taddr));
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
+// The load alone: the words are there after tmem_ld_wait.
+__device__ __forceinline__ void tmem_ld16_start(uint32_t taddr, uint32_t (&r)[16]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+                 : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
@@ -151,7 +166,7 @@ __device__ __forceinline__ uint64_t tc_combine(const uint32_t *w, uint64_t x) {
 }
 
 // The 8 bytes of y as fp16 subnormals whose bit patterns are the bytes
-// (one 16-byte row of a K chunk), and the word back from such a row.
+// (one 16-byte row of a K chunk).
 __device__ __forceinline__ uint4 tc_bytes(uint64_t y) {
     const uint32_t lo = lo32(y), hi = hi32(y);
     uint4 v;
@@ -161,9 +176,5 @@ __device__ __forceinline__ uint4 tc_bytes(uint64_t y) {
     v.w = __byte_perm(hi, 0u, 0x4342);
     return v;
 }
-__device__ __forceinline__ uint64_t tc_word(uint4 v) {
-    return ((uint64_t)__byte_perm(v.z, v.w, 0x6420) << 32) | __byte_perm(v.x, v.y, 0x6420);
-}
-
 }  // namespace dev
 }  // namespace pg12
