@@ -325,6 +325,17 @@ __device__ __forceinline__ uint64_t fold_small(uint32_t w0, uint32_t w1, uint32_
     return ((uint64_t)u << 32) | l;
 }
 
+// a + b as a weak word
+__device__ __forceinline__ uint64_t add_fold(uint64_t a, uint64_t b) {
+    uint32_t l, h, k;
+    asm("add.cc.u32 %0, %3, %5;\n\t"
+        "addc.cc.u32 %1, %4, %6;\n\t"
+        "addc.u32 %2, 0, 0;"
+        : "=&r"(l), "=&r"(h), "=&r"(k)
+        : "r"(lo32(a)), "r"(hi32(a)), "r"(lo32(b)), "r"(hi32(b)));
+    return fold_small(l, h, k);
+}
+
 // Lazy dot product in Montgomery form: sum_j x_j m_j R^-1 + u.  The outer
 // partial products go into a 160-bit sum that starts at u 2^64, the middle
 // ones into a 96-bit sum; each is a multiply-add with carry, so a term is four
@@ -353,6 +364,20 @@ __device__ __forceinline__ void macc(MAcc &A, uint64_t x, uint64_t m) {
         "addc.u32 %7, %7, 0;"
         : "+r"(A.a0), "+r"(A.a1), "+r"(A.a2), "+r"(A.a3), "+r"(A.a4), "+r"(A.b0), "+r"(A.b1), "+r"(A.b2)
         : "r"(lo32(x)), "r"(hi32(x)), "r"(lo32(m)), "r"(hi32(m)));
+}
+
+// A += B
+__device__ __forceinline__ void macc_join(MAcc &A, const MAcc &B) {
+    asm("add.cc.u32 %0, %0, %8;\n\t"
+        "addc.cc.u32 %1, %1, %9;\n\t"
+        "addc.cc.u32 %2, %2, %10;\n\t"
+        "addc.cc.u32 %3, %3, %11;\n\t"
+        "addc.u32 %4, %4, %12;\n\t"
+        "add.cc.u32 %5, %5, %13;\n\t"
+        "addc.cc.u32 %6, %6, %14;\n\t"
+        "addc.u32 %7, %7, %15;"
+        : "+r"(A.a0), "+r"(A.a1), "+r"(A.a2), "+r"(A.a3), "+r"(A.a4), "+r"(A.b0), "+r"(A.b1), "+r"(A.b2)
+        : "r"(B.a0), "r"(B.a1), "r"(B.a2), "r"(B.a3), "r"(B.a4), "r"(B.b0), "r"(B.b1), "r"(B.b2));
 }
 
 // (sum of the products) R^-1 + u as a weak word: the tail on the sum's low 128

@@ -139,10 +139,11 @@ __global__ void __launch_bounds__(256) k_pipe_bench(uint64_t *out, long long *cy
 // The constant tables are arbitrary words (latency does not depend on them).
 template <int OP>
 __global__ void k_lat_bench(uint64_t *out, long long *cycles, int iters) {
-    __shared__ __align__(16) DevConsts K;
+    __shared__ __align__(16) WideConsts K;
+    __shared__ __align__(16) WideBuf<16, 32> buf;
     __shared__ uint64_t slots[kT * 32];
     uint64_t *w = reinterpret_cast<uint64_t *>(&K);
-    for (unsigned i = threadIdx.x; i < sizeof(DevConsts) / 8; i += blockDim.x) w[i] = 0x9E3779B97F4A7C15ull * (i + 1);
+    for (unsigned i = threadIdx.x; i < sizeof(WideConsts) / 8; i += blockDim.x) w[i] = 0x9E3779B97F4A7C15ull * (i + 1);
     uint64_t *slot = slots + threadIdx.x;
     for (int i = 0; i < kT; ++i) slot[i * 32] = 0x100000001ull * (threadIdx.x + 7 * i + 1);
     __syncthreads();
@@ -165,7 +166,7 @@ __global__ void k_lat_bench(uint64_t *out, long long *cycles, int iters) {
             permute_slot<32>(slot);
             x = slot[0];
         } else {
-            x = permute_wide(x, threadIdx.x & 15, 0xFFFFFFFFu, K);
+            x = permute_wide(x, buf, K, threadIdx.x);
         }
     }
     const long long t1 = clock64();

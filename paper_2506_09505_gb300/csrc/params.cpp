@@ -465,28 +465,59 @@ bool build_tc_tables(const OptParams &op, TcTables &tt) {
     return ok;
 }
 
-bool build_tc_dev(const OptParams &op, TcDev &td, uint64_t beta[kRP][kRP]) {
-    std::memset(&td, 0, sizeof td);
+// The 7th root (7 is prime to p - 1, so x -> x^7 permutes the field).
+static uint64_t root7(uint64_t v) {
+    unsigned __int128 e = 1;  // the multiple of p - 1, plus 1, that 7 divides
+    while (e % 7 != 0) e += kP - 1;
+    return fp_pow(v, (uint64_t)(e / 7));
+}
+
+bool derive_kernel(const OptParams &op, KernelParams &kp) {
+    std::memset(&kp, 0, sizeof kp);
     ChainParams cp;
     derive_chain(op, cp);
-    const uint64_t R = kEps, R6 = fp_pow(R, 6), R7 = fp_mul(R6, R);
-    for (int q = 0; q < kRP; ++q)
-        for (int r = 0; r < kRP; ++r) beta[q][r] = r <= q ? fp_mul(cp.beta[q][r], R7) : 0;
+    const uint64_t R6 = fp_pow(kEps, 6);
+    // lambda_22 = 1; lambda_q^7 R^-6 = kappa_q = lambda_(q+1) beta[q][q]
+    uint64_t lambda[kRP + 1], kappa[kRP];
+    lambda[kRP] = 1;
+    for (int q = kRP - 1; q >= 0; --q) {
+        kappa[q] = fp_mul(lambda[q + 1], cp.beta[q][q]);
+        if (kappa[q] == 0) return false;
+        lambda[q] = root7(fp_mul(kappa[q], R6));
+    }
+    for (int i = 0; i < kT; ++i) {
+        kp.rc0[i] = op.full_rc[0][i] % kP;
+        for (int r = 0; r < kRF - 1; ++r)
+            if (r != kRF / 2 - 1) kp.add[r][i] = op.full_rc[r + 1][i] % kP;
+        kp.x_add[i] = op.full_rc[kRF / 2][i] % kP;
+        for (int j = 0; j < kT; ++j) {
+            kp.m[i][j] = fp_mul(op.mds[i][j] % kP, R6);
+            kp.pre[i][j] = fp_mul(fp_mul(op.pre[i][j] % kP, R6), i == 0 ? lambda[0] : 1);
+        }
+        for (int r = 0; r < kRP; ++r) kp.w[i][r] = fp_mul(cp.w[i][r], fp_inv(kappa[r]));
+    }
+    kp.add[kRF / 2 - 1][0] = fp_mul(op.part_rc[0] % kP, lambda[0]);
+    for (int q = 0; q < kRP; ++q) {
+        if (q < kRP - 1) kp.u_add[q] = fp_mul(op.part_rc[q + 1] % kP, lambda[q + 1]);
+        for (int j = 0; j < kT; ++j) kp.u[q][j] = fp_mul(fp_mul(cp.vp[q][j], R6), lambda[q + 1]);
+        for (int r = 0; r <= q; ++r) kp.beta[q][r] = fp_mul(fp_mul(cp.beta[q][r], lambda[q + 1]), fp_inv(kappa[r]));
+    }
+    return true;
+}
 
-    // constants added by each kind's bias
+bool build_tc_dev(const OptParams &op, const KernelParams &kp, TcDev &td) {
+    std::memset(&td, 0, sizeof td);
+
+    // constants added by each kind's bias: dense layer r feeds round r + 1,
+    // round 3's the partial rounds (cell 0's S-box; cells 1..11 wait for the W
+    // contraction, which adds round 4's constants to all cells)
     uint64_t add[kBiasKinds][kT] = {};
     for (int i = 0; i < kT; ++i) {
-        // dense layer r feeds round r + 1; round 3's feeds the partial rounds
-        // (cell 0's S-box; cells 1..11 wait for the W contraction, which adds
-        // round 4's constants to all cells)
-        for (int r = 0; r < kRF - 1; ++r)
-            if (r != kRF / 2 - 1) add[kBiasDense + r][i] = op.full_rc[r + 1][i] % kP;
-        add[kBiasW][i] = op.full_rc[kRF / 2][i] % kP;
-        if (i < kTcUa) add[kBiasUa][i] = op.part_rc[i + 1] % kP;
-        const int q = kTcUa + i;
-        if (q < kRP - 1) add[kBiasUb][i] = op.part_rc[q + 1] % kP;
+        for (int r = 0; r < kRF; ++r) add[kBiasDense + r][i] = kp.add[r][i];
+        add[kBiasW][i] = kp.x_add[i];
+        if (i < kTcUa) add[kBiasUa][i] = kp.u_add[i];
+        add[kBiasUb][i] = kp.u_add[kTcUa + i];
     }
-    add[kBiasDense + kRF / 2 - 1][0] = op.part_rc[0] % kP;
 
     // u_b(k, i) in [1407, 1665] as in tc_bias_blocks, here with the offset of
     // tc_combine: sum_b 2^(8b) (v_b - 2^23) + 0x3F + 0x3F3F + (0x3F00 + 0x3F0000) 2^64
@@ -517,7 +548,7 @@ bool build_tc_dev(const OptParams &op, TcDev &td, uint64_t beta[kRP][kRP]) {
     bool ok = true;
     auto table = [&](auto &&entry, int n, uint16_t *dst, long *pos, long *neg) {
         for (int i = 0; i < n; ++i)
-            for (int j = 0; j < kT; ++j) mat[i * kT + j] = fp_mul(entry(i, j) % kP, R6);
+            for (int j = 0; j < kT; ++j) mat[i * kT + j] = entry(i, j);
         digit_table(mat, n, kT, dst, pos, neg);
     };
     auto check = [&](const long *pos, const long *neg, int k, int n) {
@@ -528,40 +559,62 @@ bool build_tc_dev(const OptParams &op, TcDev &td, uint64_t beta[kRP][kRP]) {
     };
     {
         long pos[kTcN] = {}, neg[kTcN] = {};
-        table([&](int i, int j) { return op.mds[i][j]; }, kT, td.m, pos, neg);
+        table([&](int i, int j) { return kp.m[i][j]; }, kT, td.m, pos, neg);
         for (int r = 0; r < kRF; ++r)
             if (r != kRF / 2 - 1) check(pos, neg, kBiasDense + r, kT);
     }
     {
         long pos[kTcN] = {}, neg[kTcN] = {};
-        table([&](int i, int j) { return op.pre[i][j]; }, kT, td.pre, pos, neg);
+        table([&](int i, int j) { return kp.pre[i][j]; }, kT, td.pre, pos, neg);
         check(pos, neg, kBiasDense + kRF / 2 - 1, kT);
     }
     {
         long pos[kTcN] = {}, neg[kTcN] = {};
-        table([&](int i, int j) { return cp.vp[i][j]; }, kTcUa, td.vpa, pos, neg);
+        table([&](int i, int j) { return kp.u[i][j]; }, kTcUa, td.vpa, pos, neg);
         check(pos, neg, kBiasUa, kTcUa);
     }
     {
         long pos[kTcN] = {}, neg[kTcN] = {};
-        table([&](int i, int j) { return cp.vp[kTcUa + i][j]; }, kT, td.vpb, pos, neg);
-        table([&](int i, int j) { return kTcUa + i < kRP - 1 && j < kTcSplit ? cp.beta[kTcUa + i][j] : 0ull; }, kT, td.bs,
+        table([&](int i, int j) { return kp.u[kTcUa + i][j]; }, kT, td.vpb, pos, neg);
+        table([&](int i, int j) { return kTcUa + i < kRP - 1 && j < kTcSplit ? kp.beta[kTcUa + i][j] : 0ull; }, kT, td.bs,
               pos, neg);
         check(pos, neg, kBiasUb, kT);
     }
     {
         long pos[kTcN] = {}, neg[kTcN] = {};
-        table([&](int i, int j) { return j < kTcSplit ? cp.w[i][j] : 0ull; }, kT, td.w1, pos, neg);
-        table([&](int i, int j) { return j < kRP - kTcSplit ? cp.w[i][kTcSplit + j] : 0ull; }, kT, td.w2, pos, neg);
+        table([&](int i, int j) { return j < kTcSplit ? kp.w[i][j] : 0ull; }, kT, td.w1, pos, neg);
+        table([&](int i, int j) { return j < kRP - kTcSplit ? kp.w[i][kTcSplit + j] : 0ull; }, kT, td.w2, pos, neg);
         check(pos, neg, kBiasW, kT);
     }
-    const uint64_t Rm6 = fp_inv(R6);
+    const uint64_t Rm6 = fp_inv(fp_pow(kEps, 6));
     for (int j = kRate; j < kT; ++j) {
         const uint64_t c7 = fp_mul(fp_pow(op.full_rc[0][j] % kP, 7), Rm6);
         for (int r = 0; r < 8; ++r)
             for (int a = 0; a < 8; ++a) td.a_zcap[(j - kRate) * 64 + r * 8 + a] = (uint16_t)((c7 >> (8 * a)) & 0xFF);
     }
     return ok;
+}
+
+void build_wide(const KernelParams &kp, WideConsts &wc) {
+    std::memset(&wc, 0, sizeof wc);
+    auto s = [](uint64_t v) { return fp_mul(v, kEps); };  // times R, for the sums' reduction
+    for (int i = 0; i < kT; ++i) {
+        wc.rc0[i] = kp.rc0[i];
+        wc.x_add[i] = kp.x_add[i];
+        for (int r = 0; r < kRF; ++r) wc.add[r][i] = kp.add[r][i];
+        for (int j = 0; j < kT; ++j) {
+            wc.m[j][i] = s(kp.m[i][j]);
+            wc.pre[j][i] = s(kp.pre[i][j]);
+        }
+        for (int r = 0; r < kRP; ++r) wc.w[r][i] = s(kp.w[i][r]);
+    }
+    for (int q = 0; q < kRP; ++q) {
+        const int e = q % kWide;
+        (q < kWide ? wc.ua_add : wc.ub_add)[e] = kp.u_add[q];
+        for (int j = 0; j < kT; ++j) (q < kWide ? wc.ua : wc.ub)[j][e] = s(kp.u[q][j]);
+        for (int r = 0; r < q; ++r) (q < kWide ? wc.ba : wc.bb)[r][e] = s(kp.beta[q][r]);
+    }
+    wc.ub_add[kRP - 1 - kWide] = kp.x_add[0];  // c_22 is cell 0 of round 4's input
 }
 
 // ------------------------------------------------------------ SHA-256

@@ -502,7 +502,8 @@ __global__ void __launch_bounds__(S, PG12_MERKLE_MIN_BLOCKS * 256 / S) k_merkle(
 // own, then climbs with arrival counters: when the level below has at least
 // two units, the group that completes the second of two sibling units
 // builds their parent unit and goes on, the first goes back for a new task.
-// Levels of at most 128 nodes have one unit and are climbed directly.
+// Levels of at most 128 nodes have one unit and are climbed directly, those of
+// at most 16 in the latency form (tc_climb_small).
 __device__ __forceinline__ uint64_t tc_units(uint64_t n, uint32_t l) {
     return ((n >> l) + kTcGroup - 1) / kTcGroup;
 }
@@ -544,6 +545,48 @@ __device__ __forceinline__ bool tc_unit(TcGroup &G, const TreePlan &tp, uint32_t
     return true;
 }
 
+// The levels of at most kTcSmallLevel nodes of a tree, `level` (the first of
+// them) up to the root, by one group in the latency form, eight nodes at a time
+// on 16 lanes each, the digests handed up through the group's A operand (idle
+// between contractions): a permutation of the group takes 22 us alone on an SM
+// and 45 us beside three other groups, one in this form 6.4 us.  The constants
+// are read from global memory (they stay in L1; shared memory is full).
+constexpr uint64_t kTcSmallLevel = 16;
+constexpr int kTcWideNodes = kTcGroup / 16;
+struct TcSmall {
+    WideBuf<16, kTcGroup> buf;
+    uint64_t dig[2][kTcSmallLevel * kDigest];
+};
+static_assert(sizeof(TcSmall) <= kTcABytes, "the scratch of the small levels lies in the A operand");
+__device__ __noinline__ void tc_climb_small(uint8_t *scratch, int bar, int t, uint64_t *nodes, uint64_t n, uint32_t level,
+                                            uint32_t log_n) {
+    TcSmall &S = *reinterpret_cast<TcSmall *>(scratch);
+    const int l16 = t & 15;
+    const uint64_t *below = nodes + kDigest * level_off(n, level - 1);
+    for (uint32_t l = level; l <= log_n; ++l) {
+        const uint64_t count = n >> l;
+        for (uint64_t first = 0; first < count; first += kTcWideNodes) {
+            const uint64_t node = first + (t >> 4);
+            // whole warps hold nodes 2w and 2w + 1; a warp past the level's end skips it
+            if ((node & ~1ull) < count) {
+                const bool valid = node < count;
+                const uint64_t k = valid ? node : 0;
+                uint64_t x = 0;
+                if (l16 < 2 * kDigest) {
+                    if (l == level) asm volatile("ld.global.cg.u64 %0, [%1];" : "=l"(x) : "l"(below + 2 * kDigest * k + l16));
+                    else x = S.dig[(l - level - 1) & 1][2 * kDigest * k + l16];
+                }
+                x = canon(permute_wide(x, S.buf, g_wide, (unsigned)t));
+                if (valid && l16 < kDigest) {
+                    S.dig[(l - level) & 1][kDigest * k + l16] = x;
+                    nodes[kDigest * (level_off(n, l) + k) + l16] = x;
+                }
+            }
+        }
+        group_sync(bar);
+    }
+}
+
 __global__ void __launch_bounds__(kTcThreads, 1) k_tc_batch(const TreePlan *__restrict__ plans, uint32_t n_trees,
                                                             uint32_t total_tasks, uint32_t fuse,
                                                             uint32_t *__restrict__ counters,
@@ -551,9 +594,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_batch(const TreePlan *__re
     extern __shared__ __align__(1024) uint8_t tc_sm[];
     TcGroup G = tc_setup<kTcGroups>(tc_sm);
     bool ok = true;
-    while (ok) {
-        const uint32_t task = group_fetch_add(G, next_task);
-        if (task >= total_tasks) break;
+    // every group's first task is fixed, CTA by CTA, so that few tasks spread
+    // over all SMs; the others come from the counter
+    const uint32_t groups = gridDim.x * kTcGroups;
+    for (uint32_t task = (uint32_t)tc_first_unit(); ok && task < total_tasks;
+         task = groups + group_fetch_add(G, next_task)) {
         uint32_t lo_t = 0, hi_t = n_trees - 1;
         while (lo_t < hi_t) {
             const uint32_t mid = (lo_t + hi_t + 1) / 2;
@@ -583,6 +628,13 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_batch(const TreePlan *__re
                 cnt >>= 1;
                 continue;
             }
+            if (top == log_n && (n >> (l + 1)) <= kTcSmallLevel) {
+                // the rest of the tree (the children below are this group's: one unit)
+                group_sync(G.bar);
+                tc_climb_small(G.a, G.bar, G.t, tp.nodes, n, l + 1, log_n);
+                if (G.t == 0) signal_root(tp, 0);
+                break;
+            }
             if (tc_units(n, l) >= 2) {
                 const uint32_t old = group_fetch_add(G, &counters[tp.counter_base + tp.level_counter[l + 1] + (lo >> 1)]);
                 if (old == 0) break;  // the sibling unit is not done: its group builds the parent
@@ -602,7 +654,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_batch(const TreePlan *__re
 constexpr int kBatchTopThreads = 1024;
 constexpr uint64_t kBatchTopNodes = kBatchTopThreads / 16;
 __global__ void __launch_bounds__(kBatchTopThreads) k_batch_top(const TreePlan *__restrict__ plans) {
-    __shared__ __align__(16) DevConsts K;
+    __shared__ __align__(16) WideConsts K;
+    __shared__ __align__(16) WideBuf<16, kBatchTopThreads> buf;
     load_consts(K);
     const TreePlan &tp = plans[blockIdx.x];
     const uint64_t n = tp.n_leaves;
@@ -620,7 +673,7 @@ __global__ void __launch_bounds__(kBatchTopThreads) k_batch_top(const TreePlan *
             if (l16 < 2 * kDigest) {
                 asm volatile("ld.global.cg.u64 %0, [%1];" : "=l"(x) : "l"(kids + l16));
             }
-            x = permute_wide(x, l16, 0xFFFFFFFFu, K);
+            x = permute_wide(x, buf, K, threadIdx.x);
             if (valid && l16 < kDigest) tp.nodes[kDigest * (level_off(n, level) + node) + l16] = canon(x);
         }
         __syncthreads();
@@ -674,60 +727,91 @@ __global__ void __launch_bounds__(kBlock) k_merkle_single(const TreePlan tp, uin
 }
 
 
-// Upper levels of a tree with the 16-lanes-per-state permutation: one group
-// per node of `level`, one launch per level.  Lanes 0..7 load the children,
-// lanes 0..3 store the digest.  Every lane reaches the shuffles (groups past
-// the level's end compute on a dummy node and skip the store).
-constexpr int kTopBlock = 256;
+// Upper levels of a tree in the latency form (16 or 32 lanes per state): one
+// group of lanes per node of `level`, one launch per level.  Lanes 0..7 load
+// the children, lanes 0..3 store the digest.  Every lane reaches the shuffles
+// (groups past the level's end compute on a dummy node and skip the store).
+// Four warps a block: a level of at most 608 warps then has one warp per
+// scheduler (two share the multiplier pipe and take 1.3 times as long).
+constexpr int kTopBlock = 128;
 // The last levels of a tree (at most kTailNodes nodes each) in one launch of
-// one thread-block cluster: kTailCtas blocks on as many SMs, one 16-lane
-// group per node, a cluster barrier between levels.  Saves a launch and a
-// constant copy per level where each level is one permutation's latency
-// anyway; spread over eight SMs (one warp per scheduler at the widest level)
-// the permutations do not queue for issue slots as they do in one block.
-// Children are read with ld.global.cg (from L2): a line of a small level can
-// sit in an SM's L1 from an earlier level's read before another block of the
-// cluster has written it.
+// one thread-block cluster: kTailCtas blocks on as many SMs, one warp per node
+// (two warps per scheduler at the widest level).  Block c builds nodes
+// [c per, (c + 1) per) of the first level and the nodes above them on its own,
+// handing digests up through its shared memory, until it holds one node; block
+// 0 receives those (distributed shared memory, one cluster barrier) and builds
+// the last levels.  Handing every level through global memory and a cluster
+// barrier took 8.1 us a level, a permutation being 5.4.
 constexpr int kTailCtas = 8;
-constexpr int kTailBlock = 128;
-constexpr uint64_t kTailNodes = kTailCtas * kTailBlock / 16;
+constexpr int kTailBlock = 256;
+constexpr uint64_t kTailNodes = kTailCtas * kTailBlock / 32;
 __global__ void __cluster_dims__(kTailCtas, 1, 1) __launch_bounds__(kTailBlock)
     k_merkle_top_tail(uint64_t *__restrict__ nodes, uint64_t n, uint32_t first) {
-    __shared__ __align__(16) DevConsts K;
+    __shared__ __align__(16) WideConsts K;
+    __shared__ __align__(16) WideBuf<32, kTailBlock> buf;
+    __shared__ uint64_t dig[2][kTailBlock / 32 * kDigest];  // digests of this block's nodes of a level, in turn
+    __shared__ uint64_t sub[kTailCtas * kDigest];           // block 0: every block's last node
     load_consts(K);
     pdl_trigger();
     pdl_wait();
-    const uint32_t log_n = 63 - __clzll(n);
-    const uint64_t gid = ((uint64_t)blockIdx.x * kTailBlock + threadIdx.x) >> 4;
-    const int l16 = threadIdx.x & 15;
-    for (uint32_t level = first; level <= log_n; ++level) {
-        const uint64_t count = n >> level;
-        // whole warps hold groups 2w and 2w + 1; a warp past the level's end skips it
-        if ((gid & ~1ull) < count) {
-            const bool valid = gid < count;
-            const uint64_t node = valid ? gid : 0;
-            const uint64_t *kids = nodes + kDigest * (level_off(n, level - 1) + 2 * node);
+    const uint32_t log_n = 63 - __clzll(n), warp = threadIdx.x / 32;
+    const int lane = threadIdx.x & 31, l16 = lane & 15;
+    const uint64_t count0 = n >> first;
+    // nodes per block: all in block 0 when the first level has fewer than eight
+    const uint32_t per0 = (uint32_t)(count0 >= kTailCtas ? count0 / kTailCtas : blockIdx.x == 0 ? count0 : 0);
+    uint64_t base = (uint64_t)blockIdx.x * per0;
+    const uint64_t *below = nodes + kDigest * (level_off(n, first - 1) + 2 * base);
+    // one node of `level` from its children's words at kids
+    auto build = [&](uint32_t level, uint64_t node, uint64_t x, uint64_t *up) {
+        x = canon(permute_wide(x, buf, K, threadIdx.x));
+        if (lane < kDigest) {
+            up[lane] = x;
+            nodes[kDigest * (level_off(n, level) + node) + lane] = x;
+        }
+    };
+    uint32_t level = first, cur = 0, per = per0;
+    for (; per >= 1; per >>= 1, ++level) {
+        if (warp < per) {
             uint64_t x = 0;
             if (l16 < 2 * kDigest) {
-                asm volatile("ld.global.cg.u64 %0, [%1];" : "=l"(x) : "l"(kids + l16));
+                if (level == first) asm volatile("ld.global.cg.u64 %0, [%1];" : "=l"(x) : "l"(below + 2 * kDigest * warp + l16));
+                else x = dig[cur ^ 1][2 * kDigest * warp + l16];
             }
-            x = permute_wide(x, l16, 0xFFFFFFFFu, K);
-            if (valid && l16 < kDigest) nodes[kDigest * (level_off(n, level) + node) + l16] = canon(x);
+            build(level, base + warp, x, &dig[cur][kDigest * warp]);
         }
-        // every thread of the cluster arrives: stores above are released to, and
-        // the next level's loads acquire from, the whole cluster
-        asm volatile("barrier.cluster.arrive.release.aligned;\n\t"
-                     "barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        __syncthreads();
+        cur ^= 1;
+        base >>= 1;
+    }
+    if (count0 < kTailCtas) return;  // block 0 has built the root
+    // the blocks' last nodes to block 0
+    if (threadIdx.x < kDigest) {
+        const uint32_t local = (uint32_t)__cvta_generic_to_shared(&sub[kDigest * blockIdx.x + threadIdx.x]);
+        uint32_t remote;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(remote) : "r"(local));
+        asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(remote), "l"(dig[cur ^ 1][threadIdx.x]) : "memory");
+    }
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\t"
+                 "barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (blockIdx.x != 0) return;
+    const uint64_t *kids = sub;
+    for (uint32_t c = kTailCtas / 2; level <= log_n; c >>= 1, ++level) {
+        if (warp < c) build(level, warp, l16 < 2 * kDigest ? kids[2 * kDigest * warp + l16] : 0, &dig[cur][kDigest * warp]);
+        __syncthreads();
+        kids = dig[cur];
+        cur ^= 1;
     }
 }
 
+template <int LANES>
 __global__ void __launch_bounds__(kTopBlock) k_merkle_top(uint64_t *__restrict__ nodes, uint64_t n, uint32_t level) {
-    __shared__ __align__(16) DevConsts K;
+    __shared__ __align__(16) WideConsts K;
+    __shared__ __align__(16) WideBuf<LANES, kTopBlock> buf;
     load_consts(K);
     pdl_trigger();
     pdl_wait();
     const uint64_t count = n >> level;
-    const uint64_t gid = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 4;
+    const uint64_t gid = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) / LANES;
     const int l16 = threadIdx.x & 15;
     const bool valid = gid < count;
     const uint64_t node = valid ? gid : 0;
@@ -736,18 +820,20 @@ __global__ void __launch_bounds__(kTopBlock) k_merkle_top(uint64_t *__restrict__
     if (l16 < 2 * kDigest) {
         asm volatile("ld.global.cg.u64 %0, [%1];" : "=l"(x) : "l"(kids + l16));
     }
-    x = permute_wide(x, l16, 0xFFFFFFFFu, K);
-    if (valid && l16 < kDigest) nodes[kDigest * (level_off(n, level) + node) + l16] = canon(x);
+    x = permute_wide(x, buf, K, threadIdx.x);
+    if (valid && (threadIdx.x & (LANES - 1)) < kDigest) nodes[kDigest * (level_off(n, level) + node) + l16] = canon(x);
 }
 
 // Leaf level of a small tree with the wide permutation: one group per row,
 // lanes 0..7 absorb the chunk words, lanes 8..11 carry the capacity.
+template <int LANES>
 __global__ void __launch_bounds__(kTopBlock) k_merkle_top_leaf(const uint64_t *__restrict__ rows, uint64_t n,
                                                                uint64_t w, uint64_t *__restrict__ nodes) {
-    __shared__ __align__(16) DevConsts K;
+    __shared__ __align__(16) WideConsts K;
+    __shared__ __align__(16) WideBuf<LANES, kTopBlock> buf;
     load_consts(K);
     pdl_trigger();
-    const uint64_t gid = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 4;
+    const uint64_t gid = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) / LANES;
     const int l16 = threadIdx.x & 15;
     const bool valid = gid < n;
     const uint64_t node = valid ? gid : 0;
@@ -759,9 +845,9 @@ __global__ void __launch_bounds__(kTopBlock) k_merkle_top_leaf(const uint64_t *_
             const uint64_t k = c * kRate + l16;
             x = k < w ? __ldg(row + k) : 0ull;
         }
-        x = permute_wide(x, l16, 0xFFFFFFFFu, K);
+        x = permute_wide(x, buf, K, threadIdx.x);
     }
-    if (valid && l16 < kDigest) nodes[kDigest * node + l16] = canon(x);
+    if (valid && (threadIdx.x & (LANES - 1)) < kDigest) nodes[kDigest * node + l16] = canon(x);
 }
 
 
@@ -814,6 +900,82 @@ __global__ void __launch_bounds__(kVerifyBlock) k_merkle_verify(const uint64_t *
     bool eq = in_range;
     for (int i = 0; i < kDigest; ++i) eq = eq && (cur[i] == root[i]);
     ok[q] = eq ? 1 : 0;
+}
+
+// The same with 16 or 32 lanes per query (the latency form of the
+// permutation): lanes 0..3 hold the digest so far, and lanes 0..7 of the state
+// are it and the sibling in the order of the position's bit.
+constexpr int kVerifyWideBlock = 128;
+template <int LANES>
+__global__ void __launch_bounds__(kVerifyWideBlock) k_merkle_verify_wide(const uint64_t *__restrict__ root, uint32_t depth,
+                                                                         uint64_t n, const uint64_t *__restrict__ leaves,
+                                                                         const uint64_t *__restrict__ idx, uint64_t k,
+                                                                         const uint64_t *__restrict__ paths,
+                                                                         uint8_t *__restrict__ ok) {
+    __shared__ __align__(16) WideConsts K;
+    __shared__ __align__(16) WideBuf<LANES, kVerifyWideBlock> buf;
+    load_consts(K);
+    const unsigned full = 0xFFFFFFFFu;
+    const uint64_t gid = ((uint64_t)blockIdx.x * kVerifyWideBlock + threadIdx.x) / LANES;
+    const uint64_t q = gid < k ? gid : 0;  // groups past the end repeat query 0 and store nothing
+    const int l16 = threadIdx.x & 15, l4 = l16 & 3, base = (threadIdx.x & 31) & ~15;
+    uint64_t cur = leaves[kDigest * q + l4];
+    const uint64_t pos = idx[q];
+    const uint64_t *path = paths + kDigest * q * depth + l4;
+    uint64_t next = depth > 0 ? path[0] : 0;
+    for (uint32_t l = 0; l < depth; ++l) {
+        const uint64_t sib = next;
+        if (l + 1 < depth) next = path[kDigest * (l + 1)];  // in flight during the permutation
+        const uint64_t right = (pos >> l) & 1u;
+        uint64_t x = (uint64_t)(l16 >> 2) == right ? cur : sib;
+        if (l16 >= kRate) x = 0;
+        x = canon(permute_wide(x, buf, K, threadIdx.x));
+        cur = __shfl_sync(full, x, base + l4);
+    }
+    const bool same = cur == root[l4];
+    const unsigned vote = __ballot_sync(full, same) >> base;
+    if (gid < k && (threadIdx.x & (LANES - 1)) == 0) ok[q] = (pos < n && (vote & 15u) == 15u) ? 1 : 0;
+}
+
+// The same with 128 queries per tensor-core group: a unit is 128 queries, and
+// each level is one permutation of the group.
+__global__ void __launch_bounds__(kTcThreads, 1) k_tc_verify(const uint64_t *__restrict__ root, uint32_t depth, uint64_t n,
+                                                             const uint64_t *__restrict__ leaves,
+                                                             const uint64_t *__restrict__ idx, uint64_t k,
+                                                             const uint64_t *__restrict__ paths, uint8_t *__restrict__ ok) {
+    extern __shared__ __align__(1024) uint8_t tc_sm[];
+    TcGroup G = tc_setup<kTcGroups>(tc_sm);
+    const uint64_t units = (k + kTcGroup - 1) / kTcGroup;
+    const uint64_t step = (uint64_t)gridDim.x * kTcGroups;
+    bool fine = true;
+    for (uint64_t u = tc_first_unit(); u < units && fine; u += step) {
+        const uint64_t gid = u * kTcGroup + G.t;
+        const uint64_t q = gid < k ? gid : 0;
+        uint64_t x[kT];
+#pragma unroll
+        for (int i = 0; i < kDigest; ++i) x[i] = leaves[kDigest * q + i];
+        const uint64_t pos = idx[q];
+        for (uint32_t l = 0; l < depth && fine; ++l) {
+            const uint64_t *sib = paths + kDigest * (q * depth + l);
+            const bool right = (pos >> l) & 1u;
+#pragma unroll
+            for (int i = 0; i < kDigest; ++i) {
+                const uint64_t s = sib[i], c = x[i];
+                x[i] = right ? s : c;
+                x[kDigest + i] = right ? c : s;
+                x[2 * kDigest + i] = 0;
+            }
+            fine = tc_permute(G, x, true, true);
+#pragma unroll
+            for (int i = 0; i < kDigest; ++i) x[i] = canon(x[i]);
+        }
+        if (!fine) break;
+        bool eq = pos < n;
+#pragma unroll
+        for (int i = 0; i < kDigest; ++i) eq = eq && x[i] == root[i];
+        if (gid < k) ok[gid] = eq ? 1 : 0;
+    }
+    tc_teardown<kTcGroups>(tc_sm, G);
 }
 
 }  // namespace dev
@@ -919,6 +1081,14 @@ constexpr uint64_t kWideNodes = PG12_WIDE_NODES;
 constexpr uint64_t kSmallTree = kWideNodes;
 // tensor engine: trees of at most this many leaves run in the 16-lane form
 constexpr uint64_t kTcSmallTree = PG12_TC_SMALL_TREE;
+// Latency form: 32 lanes per state while that is at most one warp per
+// scheduler, above 16 (20-level paths of 608 / 1021 queries: 132 / 174 us on 32
+// lanes, 145 / 149 us on 16).
+unsigned wide_lanes(uint64_t states);
+// pg_merkle_verify: up to this many queries in the latency form (4,864 queries
+// of 20 levels: 363 us on 16 lanes; the tensor-core kernel takes 430 us for any
+// number up to 19,456, one unit of 128 per SM).
+constexpr uint64_t kVerifyWideMax = 5120;
 constexpr size_t kPlanBytes = 4u << 20;        // first part: plans; rest: counters
 
 // ------------------------------------------------------------ launch timing
@@ -990,13 +1160,21 @@ pg_status upload_tables() {
     dev::DevConsts dc;
     dev::make_dev_consts(g.opt, dc);
     PG_CUDA(cudaMemcpyToSymbol(dev::c_dev, &dc, sizeof(dc)));
-    PG_CUDA(cudaMemcpyToSymbol(dev::g_dev, &dc, sizeof(dc)));
-    static TcDev td;  // 131 KB; built under g_mu
-    static uint64_t beta[kRP][kRP];
-    if (!host::build_tc_dev(g.opt, td, beta))
+    static KernelParams kp;  // this and the tables below: built under g_mu
+    static WideConsts wc;
+    static TcDev td;         // 131 KB
+    if (!host::derive_kernel(g.opt, kp))
+        return fail(PG_ERR_PARAMS, "parameter set %s: a partial round's coefficient is zero",
+                    g.params_set == 1 ? "pg12_small" : "pg12_v1");
+    host::build_wide(kp, wc);
+    PG_CUDA(cudaMemcpyToSymbol(dev::g_wide, &wc, sizeof(wc)));
+    if (!host::build_tc_dev(g.opt, kp, td))
         return fail(PG_ERR_PARAMS, "parameter set %s: a tensor-core sum could leave the exact fp32 window",
                     g.params_set == 1 ? "pg12_small" : "pg12_v1");
     PG_CUDA(cudaMemcpyToSymbol(dev::g_tc, &td, sizeof(td)));
+    uint64_t beta[kRP][kRP];
+    for (int q = 0; q < kRP; ++q)
+        for (int r = 0; r < kRP; ++r) beta[q][r] = host::fp_mul(kp.beta[q][r], kEps);
     PG_CUDA(cudaMemcpyToSymbol(dev::c_beta, beta, sizeof(beta)));
     return PG_OK;
 }
@@ -1052,6 +1230,8 @@ uint32_t first_small_level(uint64_t n) {
     while ((n >> l) > dev::kBatchTopNodes) ++l;
     return l;
 }
+
+unsigned wide_lanes(uint64_t states) { return states <= 4 * (uint64_t)g.sms ? 32 : 16; }
 
 cudaStream_t as_stream(void *s) { return reinterpret_cast<cudaStream_t>(s); }
 
@@ -1225,9 +1405,11 @@ pg_status launch_levels(uint64_t *nodes, uint64_t n_leaves, uint32_t first, cuda
             else
                 PG_CUDA(launch_dependent(dev::k_merkle_level<dev::kMdsFull>, grid, 128, st, below, cnt, here));
         } else {
-            const unsigned grid = (unsigned)((cnt * 16 + dev::kTopBlock - 1) / dev::kTopBlock);
+            const unsigned lanes = wide_lanes(cnt);
+            const unsigned grid = (unsigned)((cnt * lanes + dev::kTopBlock - 1) / dev::kTopBlock);
             ProfScope prof(kIdMerkleTop, st, cnt);
-            PG_CUDA(launch_dependent(dev::k_merkle_top, grid, dev::kTopBlock, st, nodes, n_leaves, l));
+            PG_CUDA(launch_dependent(lanes == 32 ? dev::k_merkle_top<32> : dev::k_merkle_top<16>, grid, dev::kTopBlock, st,
+                                     nodes, n_leaves, l));
         }
     }
     return PG_OK;
@@ -1292,8 +1474,7 @@ pg_status launch_batch(const pg_schedule *sched, const dev::TreePlan *d_plans, u
                        uint32_t *d_counters, cudaStream_t st, uint64_t perms, uint64_t top_perms) {
     if (batch_uses_tc(sched)) {
         const uint32_t fuse = sched ? sched->fuse_levels : 0;
-        const uint32_t want = (tasks + dev::kTcGroups - 1) / dev::kTcGroups;
-        const unsigned grid = want < (uint32_t)g.sms ? want : (uint32_t)g.sms;
+        const unsigned grid = tasks < (uint32_t)g.sms ? tasks : (uint32_t)g.sms;
         if (grid > 0) {
             ProfScope prof(kIdTcBatch, st, perms - top_perms);
             dev::k_tc_batch<<<grid, dev::kTcThreads, dev::TcL::kBytes, st>>>(d_plans, n_trees, tasks, fuse, d_counters + 1,
@@ -1748,6 +1929,7 @@ pg_status pg_init(int device, const char *params_path) {
     if (s != PG_OK) return s;
     PG_CUDA(cudaFuncSetAttribute(dev::k_tc_permute, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dev::TcL::kBytes));
     PG_CUDA(cudaFuncSetAttribute(dev::k_tc_sponge, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dev::TcL::kBytes));
+    PG_CUDA(cudaFuncSetAttribute(dev::k_tc_verify, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dev::TcL::kBytes));
     PG_CUDA(cudaFuncSetAttribute(dev::k_tc_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dev::TcL::kBytes));
     PG_CUDA(cudaFuncSetAttribute(dev::k_tc_leaves_stream, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)dev::TcL::kBytes));
@@ -1889,10 +2071,12 @@ pg_status pg_merkle_build(const uint64_t *rows, size_t n_leaves, size_t width, u
     // different streams are independent
     const uint32_t first_top = 1;
     if ((uint64_t)n_leaves <= (g.engine == 1 ? kTcSmallTree : kSmallTree)) {  // whole tree in the 16-lane form
-        const uint64_t threads = (uint64_t)n_leaves * 16;
+        const bool w32 = wide_lanes(n_leaves) == 32;
+        const uint64_t threads = (uint64_t)n_leaves * (w32 ? 32 : 16);
         const unsigned grid = (unsigned)((threads + dev::kTopBlock - 1) / dev::kTopBlock);
         ProfScope prof(kIdMerkleTopLeaf, st, (uint64_t)n_leaves * ((width + kRate - 1) / kRate));
-        dev::k_merkle_top_leaf<<<grid, dev::kTopBlock, 0, st>>>(rows, (uint64_t)n_leaves, (uint64_t)width, nodes);
+        (w32 ? dev::k_merkle_top_leaf<32> : dev::k_merkle_top_leaf<16>)<<<grid, dev::kTopBlock, 0, st>>>(
+            rows, (uint64_t)n_leaves, (uint64_t)width, nodes);
         PG_CUDA(cudaGetLastError());
     } else if (g.engine == 1) {
         s = launch_tc_sponge(rows, n_leaves, width, nodes, st, false, kIdTcLeaves);
@@ -2360,8 +2544,17 @@ pg_status pg_merkle_verify(const uint64_t *root, size_t n_leaves, const uint64_t
     if (!root || !leaves || !indices || !ok || (!paths && n_leaves > 1)) return fail(PG_ERR_INVALID_ARG, "NULL buffer");
     const uint32_t depth = log2u(n_leaves);
     const unsigned grid = (unsigned)((k + dev::kVerifyBlock - 1) / dev::kVerifyBlock);
-    ProfScope prof(kIdVerify, as_stream(stream), (uint64_t)k * depth);
-    if (g.params_set == 1)
+    cudaStream_t st = as_stream(stream);
+    ProfScope prof(kIdVerify, st, (uint64_t)k * depth);
+    if (k <= kVerifyWideMax) {
+        const unsigned lanes = wide_lanes(k);
+        const unsigned wide = (unsigned)((k * lanes + dev::kVerifyWideBlock - 1) / dev::kVerifyWideBlock);
+        (lanes == 32 ? dev::k_merkle_verify_wide<32> : dev::k_merkle_verify_wide<16>)<<<wide, dev::kVerifyWideBlock, 0, st>>>(
+            root, depth, (uint64_t)n_leaves, leaves, indices, (uint64_t)k, paths, ok);
+    } else if (g.engine == 1) {
+        dev::k_tc_verify<<<tc_grid(k), dev::kTcThreads, dev::TcL::kBytes, st>>>(root, depth, (uint64_t)n_leaves, leaves,
+                                                                               indices, (uint64_t)k, paths, ok);
+    } else if (g.params_set == 1)
         dev::k_merkle_verify<dev::kMdsSmall><<<grid, dev::kVerifyBlock, 0, as_stream(stream)>>>(root, depth, (uint64_t)n_leaves,
                                                                                              leaves, indices, (uint64_t)k, paths, ok);
     else

@@ -97,10 +97,36 @@ struct TcTables {
 };
 static_assert(sizeof(TcTables) % 16 == 0, "tables are copied in 16-byte pieces");
 
-// The tables the kernels read (TcTables is the exported form).  They differ
-// from TcTables in three ways:
-//   - every matrix is multiplied by R^6, R = 2^64: the S-box outputs it meets
-//     are x^7 R^-6 (field.cuh, msbox), and a_zcap holds (c_0[j])^7 R^-6;
+// The permutation's constants as the Montgomery kernels use them (R = 2^64;
+// S-box outputs there are f(x) = x^7 R^-6, field.cuh):
+//   - m, pre and u meet outputs f(x), so they are M, the transition matrix and
+//     vp (ChainParams) times R^6;
+//   - the chain runs on scaled values z_q = lambda_q (c_q + k_q), chosen so that
+//     the newest S-box output enters the next value with coefficient 1:
+//     lambda_q^7 R^-6 = kappa_q = lambda_(q+1) beta[q][q], lambda_22 = 1 (seventh
+//     roots exist: 7 is prime to p - 1).  Then f(z_q) = kappa_q s_q and
+//       z_(q+1) = u_q y3 + u_add_q + sum_(r<q) beta~[q][r] f(z_r) + f(z_q),
+//     beta~[q][r] = lambda_(q+1) beta[q][r] / kappa_r, u_q and u_add_q = k_(q+1)
+//     scaled by lambda_(q+1), row 0 of pre and k_0 by lambda_0, and
+//     w~[i][r] = w[i][r] / kappa_r.  One product less per partial round, and on
+//     the chain's critical path;
+//   - add[r] are the constants that follow dense layer r (the next round's;
+//     for r = 3 lambda_0 k_0 in cell 0), x_add round 4's.
+struct KernelParams {
+    uint64_t rc0[kT];
+    uint64_t add[kRF][kT];
+    uint64_t m[kT][kT];
+    uint64_t pre[kT][kT];
+    uint64_t u[kRP][kT];
+    uint64_t u_add[kRP];
+    uint64_t beta[kRP][kRP];  // r <= q, diagonal 1
+    uint64_t w[kT][kRP];      // row 0: beta row 21
+    uint64_t x_add[kT];
+};
+
+// The tables the kernels read (TcTables is the exported form): KernelParams'
+// matrices as digit tables, and
+//   - a_zcap holds the S-box outputs f(c_0[j]);
 //   - the bias carries the constants that follow the contraction: the bias of
 //     kind k (TcBias) makes row i come out as (M y)_i + const_k[i], so no round
 //     constant is added on the integer pipes after the first.  b_bias holds, per
@@ -124,6 +150,28 @@ struct TcDev {
     uint16_t w2[kTcN * kTcK];
 };
 static_assert(sizeof(TcDev) % 16 == 0, "tables are copied in 16-byte pieces");
+
+// Tables of the latency form (permute_wide in poseidon.cuh): KernelParams by
+// column, so that a row's load by 16 lanes is 128 contiguous bytes; the matrices
+// are stored times R for the Montgomery reduction of their sums.  Entry e
+// belongs to cell e (e < 12) and to the chain's rows q = e (ua, ba) and q = 16 +
+// e (ub, bb); unused entries are zero.
+constexpr int kWide = 16;
+struct WideConsts {
+    uint64_t rc0[kWide];
+    uint64_t add[kRF][kWide];
+    uint64_t m[kT][kWide];
+    uint64_t pre[kT][kWide];
+    uint64_t ua[kT][kWide];
+    uint64_t ub[kT][kWide];
+    uint64_t ua_add[kWide];
+    uint64_t ub_add[kWide];          // row 21: cell 0's constant of round 4
+    uint64_t x_add[kWide];
+    uint64_t ba[kRP][kWide];         // beta~[q][r] by r < q
+    uint64_t bb[kRP][kWide];
+    uint64_t w[kRP][kWide];          // w~[i][r] by r
+};
+static_assert(sizeof(WideConsts) % 16 == 0, "constant tables are copied in 16-byte pieces");
 
 // Records the text returned by pg_last_error() and passes `status` through.
 int set_error(int status, const char *fmt, ...);
@@ -175,9 +223,11 @@ void derive_chain(const OptParams &op, ChainParams &cp);
 // Digit tables of the tensor-core contractions for an optimised set; false if
 // a sum could leave the exact window (every table is checked).
 bool build_tc_tables(const OptParams &op, TcTables &tt);
-// The same for the kernels' tables; beta receives the chain's coefficients
-// times R^7 (R^6 for the S-box outputs, R for the Montgomery reduction).
-bool build_tc_dev(const OptParams &op, TcDev &td, uint64_t beta[kRP][kRP]);
+// The kernels' constants; false if a chain coefficient beta[q][q] is zero.
+bool derive_kernel(const OptParams &op, KernelParams &kp);
+// Their digit tables, checked like build_tc_tables.
+bool build_tc_dev(const OptParams &op, const KernelParams &kp, TcDev &td);
+void build_wide(const KernelParams &kp, WideConsts &wc);
 // The bias blocks every tensor-core contraction adds (TcTables::a_bias and
 // b_bias) and their digits u_b.
 void tc_bias_blocks(uint16_t a_bias[128], uint16_t b_bias[128], int u[8]);

@@ -309,74 +309,137 @@ __device__ __forceinline__ void permute_slot(uint64_t *slot, bool zcap = false, 
 
 
 // ------------------------------------------------------------ wide form
-// Sixteen lanes share one state: lane e < 12 holds cell x_e (lanes 12..15
-// carry zeros).  Used where few permutations are in flight (the top levels
-// of a tree), because its latency is about a tenth of the one-thread form.
-// Lanes index the constants by their own cell, so the kernels stage a copy
-// of the tables in shared memory (load_consts) and pass it in as K.
-__device__ __align__(16) DevConsts g_dev;
-static_assert(sizeof(DevConsts) % 16 == 0, "constant tables are copied in 16-byte pieces");
+// Sixteen lanes share one state: lane e < 12 holds cell x_e.  Used where few
+// permutations are in flight (the top levels of a tree, path checks), where
+// what counts is the latency of one.  Lanes index the constants by their own
+// column, so the kernels stage a copy of the tables in shared memory
+// (load_consts) and pass it in as K.
+__device__ __align__(16) WideConsts g_wide;
 
 // Block-wide copy of the constant tables into shared memory (16-byte loads).
-__device__ __forceinline__ void load_consts(DevConsts &dst) {
-    const uint4 *src = reinterpret_cast<const uint4 *>(&g_dev);
+__device__ __forceinline__ void load_consts(WideConsts &dst) {
+    const uint4 *src = reinterpret_cast<const uint4 *>(&g_wide);
     uint4 *d = reinterpret_cast<uint4 *>(&dst);
-    for (unsigned i = threadIdx.x; i < sizeof(DevConsts) / sizeof(uint4); i += blockDim.x) d[i] = __ldg(src + i);
+    for (unsigned i = threadIdx.x; i < sizeof(WideConsts) / sizeof(uint4); i += blockDim.x) d[i] = __ldg(src + i);
     __syncthreads();
 }
 
-__device__ __forceinline__ uint64_t add_weak(uint64_t a, uint64_t b) {
-    uint64_t s = a + b;
-    if (s < b) {
-        s += EPS;
-        if (s < EPS) s += EPS;  // second wrap (only when both inputs are >= p)
-    }
-    return s;
+// Shared memory of a block's states: the words the lanes exchange (two
+// buffers in turn, so that a layer's writes need no barrier against the reads
+// of the layer before) and the partial rounds' S-box outputs.  LANES = 16 or 32
+// lanes per state.
+constexpr int kWideS = kRP + 2;
+template <int LANES, int BLOCK>
+struct WideBuf {
+    uint64_t y[2][BLOCK / LANES][kWide];
+    uint64_t s[BLOCK / LANES][kWideS];
+};
+
+// add + sum of n terms y_j mat[j][e], j from `first`, in three accumulators (a
+// carry chain per term would otherwise run through all of them).
+template <int N>
+__device__ __forceinline__ uint64_t wide_dot(const uint64_t *y, const uint64_t *col, uint64_t add) {
+    MAcc A[3];
+    macc_init(A[0], add);
+    macc_init(A[1], 0);
+    macc_init(A[2], 0);
+#pragma unroll
+    for (int j = 0; j < N; ++j) macc(A[j % 3], y[j], col[j * kWide]);
+    macc_join(A[1], A[2]);
+    macc_join(A[0], A[1]);
+    return macc_reduce(A[0]);
 }
 
-// `lane16` = lane index within its 16-lane group, `gmask` = the warp's active
-// mask; every lane of the group must execute this.  Latency is what matters
-// here, so the critical path is kept short: in a partial round the products
-// v_e x_e (e >= 1) and their butterfly sum do not wait for the S-box; only
-// v_0 x_0^7 is added after it.  Dense rows use two accumulators.  There are
-// no lane-dependent branches (a divergent warp would run the two sides one
-// after the other): every lane computes and operands are selected.  Lanes 12
-// to 15 carry values nobody reads (dense rows gather lanes 0-11, x_0 comes
-// from lane 0, and their products are masked out of the sum).
-__device__ __forceinline__ uint64_t permute_wide(uint64_t x, int lane16, unsigned gmask, const DevConsts &K) {
-    const int e = lane16 < kT ? lane16 : 0;
-    const uint64_t pmask = (lane16 >= 1 && lane16 < kT) ? ~0ull : 0ull;
-    const bool lane0 = lane16 == 0;
-    const int base = (threadIdx.x & 31) & ~15;
+// Row sums of the chain: c += p, three words (no reduction until it is read).
+struct Lazy3 {
+    uint32_t a0, a1, a2;
+};
+__device__ __forceinline__ Lazy3 lazy3(uint64_t v) { return Lazy3{lo32(v), hi32(v), 0u}; }
+__device__ __forceinline__ void lazy3_add(Lazy3 &A, uint64_t p) {
+    asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, 0;"
+        : "+r"(A.a0), "+r"(A.a1), "+r"(A.a2)
+        : "r"(lo32(p)), "r"(hi32(p)));
+}
+__device__ __forceinline__ uint64_t lazy3_word(const Lazy3 &A) { return fold_small(A.a0, A.a1, A.a2); }
+
+// The permutation of one state on LANES lanes (16: two states per warp; 32:
+// one).  Lane l passes cell l % 16 (lanes 12..15 of each 16 pass 0 and get 0) and
+// gets it back; every lane of the warp must execute this, with its index tid
+// among the BLOCK threads that share buf.  Montgomery products
+// and the partial rounds in their unrolled, scaled form (KernelParams): round q
+// is the S-box of z_q and z_(q+1) = t + f(z_q) in every lane alike, t the row's
+// sum so far; beside it f(z_q) goes into the lanes' rows of U (rows e and 16 + e
+// on 16 lanes, row l on 32) and the next row's sum is broadcast.  The cells'
+// updates W s wait for the end.  On 32 lanes each dense row is split over two
+// lanes.  What counts is the latency of dependent instructions (a product 66
+// cycles, an S-box 207), and a lone warp overlaps little, so work beside the
+// chain is kept short and runs one round behind it.  One warp alone: 12.9 k
+// cycles a permutation on 16 lanes, 11.1 k on 32 (8 full rounds of 670 / 570, 21
+// partial rounds of 330 / 310); with the sparse partial rounds, field.cuh's
+// fold and a butterfly sum a round it was 18.3 k.
+template <int LANES, int BLOCK>
+__device__ __forceinline__ uint64_t permute_wide(uint64_t x, WideBuf<LANES, BLOCK> &buf, const WideConsts &K,
+                                                 unsigned tid) {
+    static_assert(LANES == 16 || LANES == 32, "a state takes half a warp or a warp");
+    const unsigned full = 0xFFFFFFFFu;
+    const int lane = tid & 31, e = lane & 15, h = LANES == 32 ? lane >> 4 : 0;
+    const int base = LANES == 32 ? 0 : lane & 16;
+    const unsigned st = tid / LANES;
+    // a row over its lanes: all twelve terms, or six on each half
+    auto dense = [&](const uint64_t *y, const uint64_t(&mat)[kT][kWide], uint64_t add) {
+        if (LANES == 16) return wide_dot<kT>(y, &mat[0][e], add);
+        const uint64_t v = wide_dot<kT / 2>(y + kT / 2 * h, &mat[kT / 2 * h][e], h ? 0 : add);
+        return add_fold(v, __shfl_xor_sync(full, v, 16));
+    };
+    x = add_canon(x, K.rc0[e]);
 #pragma unroll 1
     for (int r = 0; r < kRF; ++r) {
-        x = sbox(add_canon(x, K.full_rc[r][e]));
-        const int m = r == kRF / 2 - 1 ? 1 : 0;
-        Acc A, B;
-        acc_zero(A);
-        acc_zero(B);
-#pragma unroll
-        for (int j = 0; j < kT; j += 2) {
-            const uint64_t xa = __shfl_sync(gmask, x, base + j);
-            const uint64_t xb = __shfl_sync(gmask, x, base + j + 1);
-            acc_mac(A, xa, K.mat[m][e][j]);
-            acc_mac(B, xb, K.mat[m][e][j + 1]);
+        buf.y[r & 1][st][e] = msbox(x);
+        __syncwarp();
+        const uint64_t *y = buf.y[r & 1][st];
+        if (r != kRF / 2 - 1) {
+            x = dense(y, K.m, K.add[r][e]);
+            continue;
         }
-        x = add_weak(acc_reduce(A), acc_reduce(B));
-        if (r == kRF / 2 - 1) {
+        const uint64_t x0 = dense(y, K.pre, K.add[r][e]);
+        // this lane's rows of U (row 16 + e on the second half, or as a second row)
+        Lazy3 A = lazy3(wide_dot<kT>(y, h ? &K.ub[0][e] : &K.ua[0][e], h ? K.ub_add[e] : K.ua_add[e])), B = lazy3(0);
+        if (LANES == 16) B = lazy3(wide_dot<kT>(y, &K.ub[0][e], K.ub_add[e]));
+        const uint64_t *ca = h ? &K.bb[0][e] : &K.ba[0][e], *cb = &K.bb[0][e];
+        uint64_t c = __shfl_sync(full, x0, base);
+        uint64_t p = msbox(c);  // f(z_(q-1)), not yet in the rows' sums
+        buf.s[st][0] = p;
+        c = add_fold(p, __shfl_sync(full, lazy3_word(A), base));
+        // round q: f(z_q), and beside it f(z_(q-1)) into the rows and row q's sum
 #pragma unroll 1
-            for (int q = 0; q < kRP; ++q) {
-                const uint64_t x0 = __shfl_sync(gmask, x, base);
-                const uint64_t y = sbox(add_canon(x0, K.part_rc[q]));
-                // sum of v_e x_e over e = 1..11 (independent of the S-box)
-                uint64_t t = mul(x, K.part_v[q][e]) & pmask;
-#pragma unroll
-                for (int d = 8; d >= 1; d >>= 1) t = add_weak(t, __shfl_xor_sync(gmask, t, d));
-                // lane 0: v_0 y + t; lane e: x_e + w_e y
-                const uint64_t coef = lane0 ? K.part_v[q][0] : K.part_w[q][e];
-                x = mul_add(coef, y, lane0 ? t : x);
+        for (int q = 1; q < (LANES == 16 ? kWide : kRP); ++q) {
+            lazy3_add(A, mmul(p, ca[(q - 1) * kWide]));
+            if (LANES == 16) lazy3_add(B, mmul(p, cb[(q - 1) * kWide]));
+            const uint64_t t = canon(__shfl_sync(full, lazy3_word(A), base + q));
+            p = msbox(c);
+            buf.s[st][q] = p;
+            c = add_canon(p, t);
+        }
+        if (LANES == 16) {  // rows 16 .. 21 are the lanes' second ones
+#pragma unroll 1
+            for (int q = kWide; q < kRP; ++q) {
+                lazy3_add(B, mmul(p, cb[(q - 1) * kWide]));
+                const uint64_t t = canon(__shfl_sync(full, lazy3_word(B), base + q - kWide));
+                p = msbox(c);
+                buf.s[st][q] = p;
+                c = add_canon(p, t);
             }
         }
+        __syncwarp();
+        // cell 0 = c_22, cell i = x_i^(0) + (W s)_i, plus round 4's constants
+        const uint64_t x0c = add_canon(x0, K.x_add[e]);
+        if (LANES == 16) {
+            x = wide_dot<kRP>(buf.s[st], &K.w[0][e], x0c);
+        } else {
+            x = wide_dot<kRP / 2>(buf.s[st] + kRP / 2 * h, &K.w[kRP / 2 * h][e], h ? 0 : x0c);
+            x = add_fold(x, __shfl_xor_sync(full, x, 16));
+        }
+        if (e == 0) x = c;
     }
     return x;
 }

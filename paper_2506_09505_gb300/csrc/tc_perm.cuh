@@ -19,8 +19,9 @@
 // the 22 partial S-box outputs; only the chain c_q -> s_q = S(c_q + k_q) ->
 // c_(q+1) = U_q + sum_(r<=q) beta[q][r] s_r runs on the integer pipes, one
 // thread per state, in two halves: the first half's terms in the second
-// half's chain values are one more contraction, so each thread forms 110 of
-// the 231 products beta[q][r] s_r.
+// half's chain values are one more contraction, and the values are scaled so
+// that beta[q][q] = 1 (KernelParams), so each thread forms 90 of the 231
+// products beta[q][r] s_r.
 //
 // Every fp32 sum is an exact integer below 2^24 (times 2^-24), so each result
 // is the exact residue: the same function as the integer-pipe form, bit for
@@ -56,7 +57,7 @@ static_assert(kTabVpa % 128 == 0 && kTabVpb % 128 == 0 && kTabBs % 128 == 0 && k
               "tables are 128-byte aligned");
 
 __device__ __align__(16) TcDev g_tc;        // uploaded with the other constant tables
-__constant__ uint64_t c_beta[kRP][kRP];     // the chain's coefficients times R^7
+__constant__ uint64_t c_beta[kRP][kRP];     // the chain's coefficients beta~ times R
 
 // One group's share of the CTA's shared memory and tensor memory.
 struct TcGroup {
@@ -148,25 +149,33 @@ __device__ __forceinline__ bool tc_dense(TcGroup &G, uint32_t m_off, int r, bool
     return true;
 }
 
-// One half of the chain: s_q = S(c_q + k_q) for q = q0 .. q0 + 10, each into
-// A's chunk q - q0, from c = c_q0 + k_q0; between them c_(q+1) + k_(q+1) =
-// U_q + sum_(r = q0 .. q) beta[q][r] s_r, U_q (its bias includes k_(q+1)) the
-// word in tensor-memory column kTcUStore + 2 (q - u0).  Unrolled, so the s_r
-// stay in registers (reading them back from A's bytes in a loop: a 2^22 x 8
-// tree 5.69 ms against 5.57).
+// One half of the chain on the scaled values of KernelParams: s_q = f(z_q) for
+// q = q0 .. q0 + 10, each into A's chunk q - q0, from c = z_q0; between them
+// z_(q+1) = U_q + sum_(r = q0 .. q-1) beta~[q][r] s_r + s_q, U_q (its bias
+// includes the round constant) the word in tensor-memory column kTcUStore +
+// 2 (q - u0).  The sum does not wait for s_q's S-box.  Unrolled, so the s_r stay
+// in registers (reading them back from A's bytes in a loop: a 2^22 x 8 tree
+// 5.69 ms against 5.57).
 static_assert(kRP == 2 * kTcSplit, "the halves have the same length");
 __device__ __forceinline__ void chain_half(const TcGroup &G, uint32_t lane_base, uint64_t c, int q0, int u0) {
     uint64_t s[kTcSplit];
 #pragma unroll
     for (int q = 0;; ++q) {
+        uint64_t t = 0;
+        if (q < kTcSplit - 1) {
+            t = tmem_ld_word(lane_base + kTcUStore + 2 * (q + q0 - u0));
+            if (q > 0) {
+                MAcc A;
+                macc_init(A, t);
+#pragma unroll
+                for (int r = 0; r < q; ++r) macc(A, s[r], c_beta[q + q0][r + q0]);
+                t = macc_reduce(A);
+            }
+        }
         s[q] = msbox(c);
         tc_put(G, q, s[q]);
         if (q == kTcSplit - 1) break;
-        MAcc A;
-        macc_init(A, tmem_ld_word(lane_base + kTcUStore + 2 * (q + q0 - u0)));
-#pragma unroll
-        for (int r = 0; r <= q; ++r) macc(A, s[r], c_beta[q + q0][r + q0]);
-        c = macc_reduce(A);
+        c = add_fold(t, s[q]);
     }
 }
 
