@@ -73,7 +73,8 @@ __device__ __forceinline__ uint32_t group_sync_or(int id, uint32_t flag, int thr
 }
 
 // Waits for phase `parity` of the mbarrier; false if it has not completed
-// within kTcWaitClocks (the clock is read only after a first test failed).
+// within kTcWaitClocks (the clock is read only after 32 tests have failed: the
+// tests share the SM's issue slots with the groups that compute).
 __device__ __forceinline__ uint32_t mbar_try(uint32_t a, uint32_t parity) {
     uint32_t done;
     asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
@@ -85,7 +86,9 @@ __device__ __forceinline__ uint32_t mbar_try(uint32_t a, uint32_t parity) {
 }
 __device__ __forceinline__ bool mbar_wait(uint64_t *mbar, uint32_t parity) {
     const uint32_t a = smem_addr(mbar);
-    if (mbar_try(a, parity)) return true;
+#pragma unroll 1
+    for (int i = 0; i < 32; ++i)
+        if (mbar_try(a, parity)) return true;
     const long long t0 = clock64();
     for (;;) {
         if (mbar_try(a, parity)) return true;
