@@ -61,10 +61,9 @@ namespace pg12 {
 namespace ntt {
 
 using dev::canon;
-using dev::fold;
 using dev::hi32;
 using dev::lo32;
-using dev::mul;
+using dev::mmul;
 using dev::P;
 
 constexpr int kMaxLog = 30;      // at most 2^30 rows per transform
@@ -85,16 +84,15 @@ constexpr int kThreads = 256;
 constexpr int kRootTab = (1 << kMaxT) - 1;     // w_{b+1}^k at index 2^b - 1 + k
 constexpr uint64_t kShift = 7;                 // generator and LDE coset shift
 
+// All device tables hold their values times R = 2^64: products are taken as
+// mmul(x, y) = x y R^-1, so a table entry times a table entry is a table entry,
+// and a data word times one is the plain product.
 struct Consts {
-    uint64_t root[2][33];            // [0] w_k = 7^((p-1)/2^k), [1] its inverse
     uint64_t tab[2][kRootTab];       // [dir][2^b - 1 + k] = w_{b+1}^k (dir 1: inverse roots)
     uint64_t pw[2][3][1024];         // [dir][d][m] = w_30^(m 2^(10 d)) (dir 1: inverse)
     uint64_t coset[3][1024];         // [d][m] = 7^(m 2^(10 d))
 };
 __device__ Consts g_ntt;
-
-// canonical product (tables)
-__device__ __forceinline__ uint64_t mul_c(uint64_t a, uint64_t b) { return canon(mul(a, b)); }
 
 // Weak operands and results (any 64-bit word standing for its residue).  A
 // carry out of bit 63 is worth 2^64 = 2^32 - 1 (mod p); adding it back can
@@ -143,7 +141,8 @@ __device__ __forceinline__ uint64_t sub_w(uint64_t a, uint64_t b) {
 // Value l0 + l1 2^32 + t 2^64 with t a signed 32-bit word: a sum or
 // difference of two such values is one three-word carry chain, with no
 // correction.  Inside a small DFT |t| stays below 2^28 (the largest comes from
-// a 2^24 shift of a value with |t| <= 2).
+// a 2^24 shift of a value with |t| <= 2); products by 2^48 and 2^72 stay lazy
+// too.
 struct Lz {
     uint32_t l0, l1, t;
 };
@@ -170,35 +169,25 @@ __device__ __forceinline__ Lz lz_sub(Lz a, Lz b) {
     return r;
 }
 
-// (w1:w0) + tp (2^32 - 1) for the top word tp in {-1, 0, 1} of a 96-bit
-// value whose low 64 bits cannot wrap in this correction (the callers' ranges
-// guarantee it: for tp = 1 the low word is below 2^64 - 2^32, for tp = -1 at
-// least 2^32).
-__device__ __forceinline__ uint64_t fix_top(uint32_t w0, uint32_t w1, uint32_t tp) {
-    uint32_t r0, r1;
-    asm("{\n\t.reg .u32 sh;\n\t"
-        "shr.s32 sh, %4, 31;\n\t"
-        "sub.cc.u32 %0, %2, %4;\n\t"
-        "subc.u32 %1, %3, sh;\n\t"
-        "add.u32 %1, %1, %4;\n\t}"
-        : "=r"(r0), "=r"(r1)
-        : "r"(w0), "r"(w1), "r"(tp));
-    return ((uint64_t)r1 << 32) | r0;
-}
-
-// weak word of a lazy value: lo + t (2^32 - 1) as a 96-bit chain, |t| < 2^31
+// weak word of a lazy value: lo + t (2^32 - 1) = lo + t 2^32 - t, |t| < 2^31.
+// The first sum's carry out of the high word and t's sign give its top word k
+// in {-1, 0, 1}, worth k 2^32 - k; with g = t + k the subtraction of g neither
+// borrows out (t > 0: the high word is at least 1 by then) nor carries out (t <
+// 0: it is at most 2^32 - 2).
 __device__ __forceinline__ uint64_t lz_reduce(Lz a) {
-    uint32_t w0, w1, w2;
-    asm("{\n\t.reg .u32 sh;\n\t"
-        "shr.s32 sh, %5, 31;\n\t"
-        "add.cc.u32 %1, %4, %5;\n\t"       // + t 2^32
-        "addc.u32 %2, sh, 0;\n\t"
-        "sub.cc.u32 %0, %3, %5;\n\t"       // - t
-        "subc.cc.u32 %1, %1, sh;\n\t"
-        "subc.u32 %2, %2, sh;\n\t}"
-        : "=r"(w0), "=r"(w1), "=r"(w2)
+    uint32_t r0, r1;
+    asm("{\n\t.reg .u32 k, g, s;\n\t"
+        "shr.s32 s, %4, 31;\n\t"
+        "add.cc.u32 %1, %3, %4;\n\t"
+        "addc.u32 k, s, 0;\n\t"
+        "add.u32 %1, %1, k;\n\t"
+        "add.u32 g, %4, k;\n\t"
+        "shr.s32 s, g, 31;\n\t"
+        "sub.cc.u32 %0, %2, g;\n\t"
+        "subc.u32 %1, %1, s;\n\t}"
+        : "=&r"(r0), "=&r"(r1)
         : "r"(a.l0), "r"(a.l1), "r"(a.t));
-    return fix_top(w0, w1, w2);
+    return ((uint64_t)r1 << 32) | r0;
 }
 
 // a 2^24, lazy: l 2^24 = (l << 24) + (l >> 40) 2^64 and t 2^88 = (t 2^24) 2^64
@@ -207,53 +196,43 @@ __device__ __forceinline__ Lz lz_m24(Lz a) {
     return Lz{a.l0 << 24, __funnelshift_l(a.l0, a.l1, 24), (a.t << 24) + (a.l1 >> 8)};
 }
 
-// a 2^48: l 2^48 = (l << 48) + (l >> 16) 2^64, (l >> 16) = hh:hl folded as
-// hl (2^32 - 1) - hh, and t 2^112 = -t 2^16 (2^96 = -1); |t| < 2^31
-__device__ __forceinline__ uint64_t lz_m48(Lz a) {
-    const uint32_t L1 = a.l0 << 16, hl = __funnelshift_r(a.l0, a.l1, 16), hh = a.l1 >> 16;
-    uint32_t w0, w1, tp;
-    asm("{\n\t.reg .u32 e0, e1, e2;\n\t"
-        "shl.b32 e0, %6, 16;\n\t"
-        "shr.s32 e1, %6, 16;\n\t"
-        "shr.s32 e2, %6, 31;\n\t"
-        "sub.cc.u32 %0, 0, e0;\n\t"         // L1 2^32 - t 2^16
-        "subc.cc.u32 %1, %3, e1;\n\t"
-        "subc.u32 %2, 0, e2;\n\t"
-        "sub.cc.u32 %0, %0, %4;\n\t"        // - hl
-        "subc.cc.u32 %1, %1, 0;\n\t"
-        "subc.u32 %2, %2, 0;\n\t"
-        "sub.cc.u32 %0, %0, %5;\n\t"        // - hh
-        "subc.cc.u32 %1, %1, 0;\n\t"
-        "subc.u32 %2, %2, 0;\n\t"
-        "add.cc.u32 %1, %1, %4;\n\t"        // + hl 2^32
-        "addc.u32 %2, %2, 0;\n\t}"
-        : "=r"(w0), "=r"(w1), "=r"(tp)
-        : "r"(L1), "r"(hl), "r"(hh), "r"(a.t));
-    return fix_top(w0, w1, tp);
+// a 2^48, lazy: with hl = bits 16..47 of l and e = (t:l1) >> 16 (signed, 48
+// bits), 2^64 = 2^32 - 1 and 2^96 = -1 give
+//   (l0 << 16 + hl) 2^32 - hl - e;  the result's t is in [-2^15 - 1, 2^15 + 1]
+// and in [-2, 2] for |t| < 2^15.
+__device__ __forceinline__ Lz lz_m48(Lz a) {
+    const uint32_t L1 = a.l0 << 16, hl = __funnelshift_r(a.l0, a.l1, 16), e0 = __funnelshift_r(a.l1, a.t, 16);
+    Lz r;
+    asm("{\n\t.reg .u32 q0, q1, s;\n\t"
+        "shr.s32 q1, %6, 16;\n\t"
+        "add.cc.u32 q0, %4, %5;\n\t"      // hl + e
+        "addc.u32 q1, q1, 0;\n\t"
+        "shr.s32 s, q1, 31;\n\t"
+        "add.cc.u32 %1, %3, %4;\n\t"
+        "addc.u32 %2, 0, 0;\n\t"
+        "sub.cc.u32 %0, 0, q0;\n\t"
+        "subc.cc.u32 %1, %1, q1;\n\t"
+        "subc.u32 %2, %2, s;\n\t}"
+        : "=&r"(r.l0), "=&r"(r.l1), "=&r"(r.t)
+        : "r"(L1), "r"(hl), "r"(e0), "r"(a.t));
+    return r;
 }
 
-// a 2^72: l 2^72 = (l << 8) 2^64 + (l >> 56) 2^128, folded as for a product
-// (2^64 = 2^32 - 1, 2^96 = -1, 2^128 = -2^32), and t 2^136 = -t 2^40;
-// |t| < 2^23
-__device__ __forceinline__ uint64_t lz_m72(Lz a) {
-    const uint32_t hl = a.l0 << 8, hh = __funnelshift_l(a.l0, a.l1, 8), k = a.l1 >> 24;
-    uint32_t w0, w1, tp;
-    asm("{\n\t.reg .u32 e1, e2;\n\t"
-        "shl.b32 e1, %6, 8;\n\t"
-        "shr.s32 e2, %6, 31;\n\t"
-        "sub.cc.u32 %0, 0, %3;\n\t"         // - hl - k 2^32
-        "subc.cc.u32 %1, 0, %5;\n\t"
-        "subc.u32 %2, 0, 0;\n\t"
-        "sub.cc.u32 %0, %0, %4;\n\t"        // - hh
-        "subc.cc.u32 %1, %1, 0;\n\t"
-        "subc.u32 %2, %2, 0;\n\t"
-        "add.cc.u32 %1, %1, %3;\n\t"        // + hl 2^32
-        "addc.u32 %2, %2, 0;\n\t"
-        "sub.cc.u32 %1, %1, e1;\n\t"        // - t 2^40
-        "subc.u32 %2, %2, e2;\n\t}"
-        : "=r"(w0), "=r"(w1), "=r"(tp)
-        : "r"(hl), "r"(hh), "r"(k), "r"(a.t));
-    return fix_top(w0, w1, tp);
+// a 2^72, lazy: with hl = l0 << 8, hh = bits 24..55 of l and k = (t:l1) >> 24
+// (signed; |t| < 2^23), hl 2^64 + hh 2^96 + k 2^128 = (hl - k) 2^32 - hl - hh.
+__device__ __forceinline__ Lz lz_m72(Lz a) {
+    const uint32_t hl = a.l0 << 8, hh = __funnelshift_l(a.l0, a.l1, 8), k = __funnelshift_l(a.l1, a.t, 8);
+    Lz r;
+    asm("{\n\t.reg .u32 q0, k1, s;\n\t"
+        "add.cc.u32 q0, %3, %4;\n\t"
+        "addc.u32 k1, %5, 0;\n\t"
+        "shr.s32 s, k1, 31;\n\t"
+        "sub.cc.u32 %0, 0, q0;\n\t"
+        "subc.cc.u32 %1, %3, k1;\n\t"
+        "subc.u32 %2, 0, s;\n\t}"
+        : "=&r"(r.l0), "=&r"(r.l1), "=&r"(r.t)
+        : "r"(hl), "r"(hh), "r"(k));
+    return r;
 }
 
 // ---------------------------------------------------------------- small DFTs
@@ -266,20 +245,20 @@ __device__ __forceinline__ void dft8_dit(uint64_t (&a)[8]) {
     const Lz b4 = lz_add(lz(a[4]), lz(a[5])), b5 = lz_sub(lz(a[4]), lz(a[5]));
     const Lz b6 = lz_add(lz(a[6]), lz(a[7])), b7 = lz_sub(lz(a[6]), lz(a[7]));
     const Lz c0 = lz_add(b0, b2), c2 = lz_sub(b0, b2);
-    const Lz y3 = lz(lz_m48(b3));
+    const Lz y3 = lz_m48(b3);
     const Lz c1 = lz_add(b1, y3), c3 = lz_sub(b1, y3);
     const Lz c4 = lz_add(b4, b6), c6 = lz_sub(b4, b6);
-    const Lz y7 = lz(lz_m48(b7));
+    const Lz y7 = lz_m48(b7);
     const Lz c5 = lz_add(b5, y7), c7 = lz_sub(b5, y7);
     a[0] = lz_reduce(lz_add(c0, c4));
     a[4] = lz_reduce(lz_sub(c0, c4));
     const Lz z5 = lz_m24(c5);
     a[1] = lz_reduce(lz_sub(c1, z5));
     a[5] = lz_reduce(lz_add(c1, z5));
-    const Lz z6 = lz(lz_m48(c6));
+    const Lz z6 = lz_m48(c6);
     a[2] = lz_reduce(lz_add(c2, z6));
     a[6] = lz_reduce(lz_sub(c2, z6));
-    const Lz z7 = lz(lz_m72(c7));
+    const Lz z7 = lz_m72(c7);
     a[3] = lz_reduce(lz_sub(c3, z7));
     a[7] = lz_reduce(lz_add(c3, z7));
 }
@@ -289,12 +268,12 @@ __device__ __forceinline__ void dft8_dit(uint64_t (&a)[8]) {
 __device__ __forceinline__ void dft8_dif(uint64_t (&a)[8]) {
     const Lz b0 = lz_add(lz(a[0]), lz(a[4])), b4 = lz_sub(lz(a[0]), lz(a[4]));
     const Lz b1 = lz_add(lz(a[1]), lz(a[5])), b5 = lz_m24(lz_sub(lz(a[5]), lz(a[1])));
-    const Lz b2 = lz_add(lz(a[2]), lz(a[6])), b6 = lz(lz_m48(lz_sub(lz(a[2]), lz(a[6]))));
-    const Lz b3 = lz_add(lz(a[3]), lz(a[7])), b7 = lz(lz_m72(lz_sub(lz(a[7]), lz(a[3]))));
+    const Lz b2 = lz_add(lz(a[2]), lz(a[6])), b6 = lz_m48(lz_sub(lz(a[2]), lz(a[6])));
+    const Lz b3 = lz_add(lz(a[3]), lz(a[7])), b7 = lz_m72(lz_sub(lz(a[7]), lz(a[3])));
     const Lz c0 = lz_add(b0, b2), c2 = lz_sub(b0, b2);
-    const Lz c1 = lz_add(b1, b3), c3 = lz(lz_m48(lz_sub(b1, b3)));
+    const Lz c1 = lz_add(b1, b3), c3 = lz_m48(lz_sub(b1, b3));
     const Lz c4 = lz_add(b4, b6), c6 = lz_sub(b4, b6);
-    const Lz c5 = lz_add(b5, b7), c7 = lz(lz_m48(lz_sub(b5, b7)));
+    const Lz c5 = lz_add(b5, b7), c7 = lz_m48(lz_sub(b5, b7));
     a[0] = lz_reduce(lz_add(c0, c1));
     a[1] = lz_reduce(lz_sub(c0, c1));
     a[2] = lz_reduce(lz_add(c2, c3));
@@ -310,7 +289,7 @@ __device__ __forceinline__ void dft8_dif(uint64_t (&a)[8]) {
 __device__ __forceinline__ void dft4_dit(uint64_t (&a)[4]) {
     const Lz b0 = lz_add(lz(a[0]), lz(a[1])), b1 = lz_sub(lz(a[0]), lz(a[1]));
     const Lz b2 = lz_add(lz(a[2]), lz(a[3])), b3 = lz_sub(lz(a[2]), lz(a[3]));
-    const Lz y3 = lz(lz_m48(b3));
+    const Lz y3 = lz_m48(b3);
     a[0] = lz_reduce(lz_add(b0, b2));
     a[2] = lz_reduce(lz_sub(b0, b2));
     a[1] = lz_reduce(lz_add(b1, y3));
@@ -319,7 +298,7 @@ __device__ __forceinline__ void dft4_dit(uint64_t (&a)[4]) {
 
 __device__ __forceinline__ void dft4_dif(uint64_t (&a)[4]) {
     const Lz b0 = lz_add(lz(a[0]), lz(a[2])), b2 = lz_sub(lz(a[0]), lz(a[2]));
-    const Lz b1 = lz_add(lz(a[1]), lz(a[3])), b3 = lz(lz_m48(lz_sub(lz(a[1]), lz(a[3]))));
+    const Lz b1 = lz_add(lz(a[1]), lz(a[3])), b3 = lz_m48(lz_sub(lz(a[1]), lz(a[3])));
     a[0] = lz_reduce(lz_add(b0, b1));
     a[1] = lz_reduce(lz_sub(b0, b1));
     a[2] = lz_reduce(lz_add(b2, b3));
@@ -328,14 +307,14 @@ __device__ __forceinline__ void dft4_dif(uint64_t (&a)[4]) {
 
 // x^e for a 30-bit exponent from three 10-bit digit tables
 __device__ __forceinline__ uint64_t pow_tab(const uint64_t (*t)[1024], uint64_t e) {
-    return mul_c(mul_c(t[0][e & 1023], t[1][(e >> 10) & 1023]), t[2][(e >> 20) & 1023]);
+    return mmul(mmul(t[0][e & 1023], t[1][(e >> 10) & 1023]), t[2][(e >> 20) & 1023]);
 }
 
 struct Pass {
     const uint64_t *src;  // rows read (row i of the pass reads src row i >> src_shift)
     uint64_t *dst;        // rows written (may equal src)
     uint64_t ncols;
-    uint64_t scale_c;     // scale 1 and 2: constant factor (n^-1)
+    uint64_t scale_c;     // scale 1 and 2: constant factor (n^-1 R)
     uint32_t log_n;       // the transform has 2^log_n rows
     uint32_t lo, t;       // row-index bits [lo, lo + t) are transformed
     uint32_t u;           // the tile spans 2^u consecutive values of bits [0, lo) (u <= lo)
@@ -360,13 +339,13 @@ __device__ __forceinline__ void step(uint64_t *x, uint32_t s0, const uint64_t *w
     if constexpr (R == 1) {
         const uint64_t a0 = x[0], a1 = x[s0];
         if (DIT) {
-            const uint64_t y = triv ? a1 : mul(a1, w[0]);
+            const uint64_t y = triv ? a1 : mmul(a1, w[0]);
             x[0] = add_w(a0, y);
             x[s0] = sub_w(a0, y);
         } else {
             const uint64_t d = sub_w(a0, a1);
             x[0] = add_w(a0, a1);
-            x[s0] = triv ? d : mul(d, w[0]);
+            x[s0] = triv ? d : mmul(d, w[0]);
         }
     } else {
         constexpr int N = 1 << R;
@@ -378,7 +357,7 @@ __device__ __forceinline__ void step(uint64_t *x, uint32_t s0, const uint64_t *w
             for (int m = 0; m < N; ++m) a[m] = x[m * s0];
             if (!triv) {
 #pragma unroll
-                for (int m = 1; m < N; ++m) a[m] = mul(a[m], w[(kE[m] - 1) << b]);
+                for (int m = 1; m < N; ++m) a[m] = mmul(a[m], w[(kE[m] - 1) << b]);
             }
             if constexpr (R == 3) dft8_dit(a);
             else dft4_dit(a);
@@ -403,7 +382,7 @@ __device__ __forceinline__ void step(uint64_t *x, uint32_t s0, const uint64_t *w
             else dft4_dif(a);
             if (!triv) {
 #pragma unroll
-                for (int m = 1; m < N; ++m) a[m] = mul(a[m], w[(kE[m] - 1) << b]);
+                for (int m = 1; m < N; ++m) a[m] = mmul(a[m], w[(kE[m] - 1) << b]);
             }
 #pragma unroll
             for (int m = 0; m < N; ++m) x[m * s0] = a[m];
@@ -490,7 +469,7 @@ __global__ void __launch_bounds__(kThreads) k_ntt_pass(const Pass ps) {
         for (uint32_t v = threadIdx.x; v < rows; v += kThreads) {
             const uint64_t row = base + v;
             const uint64_t j = ps.log_n ? (uint64_t)(__brevll(row) >> (64 - ps.log_n)) : 0;
-            fac[v] = mul(pow_tab(g_ntt.coset, j), ps.scale_c);
+            fac[v] = mmul(pow_tab(g_ntt.coset, j), ps.scale_c);
         }
     }
     __syncthreads();
@@ -500,12 +479,12 @@ __global__ void __launch_bounds__(kThreads) k_ntt_pass(const Pass ps) {
         const uint32_t nb = 1u << b, s = b + r - 1;
         for (uint32_t q = threadIdx.x; q < (nb << u); q += kThreads) {
             const uint32_t l = q >> b, k = q & (nb - 1);
-            const uint64_t tau = mul(beta[l][i], g_ntt.tab[dir][(1u << s) - 1 + k]);
+            const uint64_t tau = mmul(beta[l][i], g_ntt.tab[dir][(1u << s) - 1 + k]);
             uint64_t *d = tw + l * tws + nb - 1 + k;
             uint64_t x = tau;
             d[0] = x;
             for (uint32_t j = 2; j < (1u << r); ++j) {
-                x = mul(x, tau);
+                x = mmul(x, tau);
                 d[(j - 1) << b] = x;
             }
         }
@@ -542,8 +521,8 @@ __global__ void __launch_bounds__(kThreads) k_ntt_pass(const Pass ps) {
         const uint64_t gstep = rstep * ps.ncols;
         for (uint32_t v = v_first, e = threadIdx.x; v < rows; v += v_step, e += kThreads, g += gstep) {
             uint64_t x = tile[e];
-            if (ps.scale == 1) x = mul(x, ps.scale_c);
-            else if (ps.scale == 2) x = mul(x, fac[v]);
+            if (ps.scale == 1) x = mmul(x, ps.scale_c);
+            else if (ps.scale == 2) x = mmul(x, fac[v]);
             *g = ps.last ? canon(x) : x;
         }
     }
@@ -724,34 +703,23 @@ int ntt_upload_constants() {
     using namespace ntt;
     static Consts h;
     const uint64_t pm1 = 0xFFFFFFFF00000000ull;  // p - 1
-    for (int k = 0; k <= 32; ++k) {
-        h.root[0][k] = host_pow(kShift, pm1 >> k);
-        h.root[1][k] = host::fp_inv(h.root[0][k]);
+    // table entries x^m R, m = 0 .. count - 1
+    auto powers = [](uint64_t x, int count, uint64_t *out) {
+        uint64_t y = kEps;  // R mod p
+        for (int m = 0; m < count; ++m) {
+            out[m] = y;
+            y = host::fp_mul(y, x);
+        }
+    };
+    for (int dir = 0; dir < 2; ++dir) {
+        auto root = [&](int k) {
+            const uint64_t w = host_pow(kShift, pm1 >> k);
+            return dir ? host::fp_inv(w) : w;
+        };
+        for (int b = 0; b < kMaxT; ++b) powers(root(b + 1), 1 << b, h.tab[dir] + (1 << b) - 1);
+        for (int d = 0; d < 3; ++d) powers(host_pow(root(30), 1ull << (10 * d)), 1024, h.pw[dir][d]);
     }
-    for (int dir = 0; dir < 2; ++dir)
-        for (int b = 0; b < kMaxT; ++b) {
-            uint64_t x = 1;
-            for (int k = 0; k < (1 << b); ++k) {
-                h.tab[dir][(1 << b) - 1 + k] = x;
-                x = host::fp_mul(x, h.root[dir][b + 1]);
-            }
-        }
-    for (int d = 0; d < 3; ++d) {
-        const uint64_t step = host_pow(kShift, 1ull << (10 * d));
-        uint64_t x = 1;
-        for (int m = 0; m < 1024; ++m) {
-            h.coset[d][m] = x;
-            x = host::fp_mul(x, step);
-        }
-        for (int dir = 0; dir < 2; ++dir) {
-            const uint64_t wstep = host_pow(h.root[dir][30], 1ull << (10 * d));
-            uint64_t y = 1;
-            for (int m = 0; m < 1024; ++m) {
-                h.pw[dir][d][m] = y;
-                y = host::fp_mul(y, wstep);
-            }
-        }
-    }
+    for (int d = 0; d < 3; ++d) powers(host_pow(kShift, 1ull << (10 * d)), 1024, h.coset[d]);
     cudaError_t e = cudaMemcpyToSymbol(g_ntt, &h, sizeof h);
     if (e != cudaSuccess) return set_error(PG_ERR_CUDA, "NTT constants: %s", cudaGetErrorString(e));
     return PG_OK;
@@ -772,7 +740,7 @@ pg_status pg_ntt(uint64_t *data, size_t n, size_t ncols, int inverse, void *stre
     if (s != PG_OK) return (pg_status)s;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const uint32_t log_n = log2u(n);
-    const uint64_t ninv = pg12::host::fp_inv((uint64_t)n);
+    const uint64_t ninv = pg12::host::fp_mul(pg12::host::fp_inv((uint64_t)n), pg12::kEps);
     s = run_dif(data, data, log_n, ncols, inverse != 0, inverse ? 1u : 0u, ninv, st);
     if (s != PG_OK) return (pg_status)s;
     if (log_n > 0) {
@@ -812,7 +780,7 @@ pg_status pg_lde(const uint64_t *evals, size_t n, size_t ncols, uint32_t log_blo
     if (s != PG_OK) return (pg_status)s;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     // coefficients c_j 7^j in bit-reversed order into scratch
-    s = run_dif(evals, scratch, log_n, ncols, true, 2u, pg12::host::fp_inv((uint64_t)n), st);
+    s = run_dif(evals, scratch, log_n, ncols, true, 2u, pg12::host::fp_mul(pg12::host::fp_inv((uint64_t)n), pg12::kEps), st);
     if (s != PG_OK) return (pg_status)s;
     // DIT passes over bits [b, log N) of out; the first reads coefficient row i >> b
     const uint32_t log_big = log_n + log_blowup;
