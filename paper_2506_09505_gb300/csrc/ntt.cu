@@ -10,7 +10,7 @@
 //
 // Everything runs as passes of one kernel.  A block loads the 2^t rows of
 // up to eight columns whose row indices differ only in bits [lo, lo + t)
-// (a 64 KiB tile: t <= 10 for eight columns, up to 11 for fewer), performs
+// (a tile of 4 to 64 KiB, plan_shape; t <= 11), performs
 // the t radix-2 stages of those bits in shared memory and stores the rows
 // back; a transform of 2^L rows reads and writes its data ceil(L / t) times.
 //   DIF (Gentleman-Sande) stages: natural order in, bit-reversed order out;
@@ -68,19 +68,12 @@ using dev::P;
 
 constexpr int kMaxLog = 30;      // at most 2^30 rows per transform
 constexpr int kMaxT = 11;        // stages per pass
-#ifndef PG12_NTT_MAXU
-#define PG12_NTT_MAXU 5
-#endif
 #ifndef PG12_NTT_CPASYNC
 #define PG12_NTT_CPASYNC 1       // 1: tile loads as asynchronous copies overlapping the table setup
 #endif
-#ifndef PG12_NTT_TILE_BITS8
-#define PG12_NTT_TILE_BITS8 10   // log2 tile rows with eight columns (64 KiB of words)
-#endif
-constexpr int kMaxU = PG12_NTT_MAXU;  // a tile spans up to 2^kMaxU consecutive values of the low bits
+constexpr int kMaxU = 5;  // a tile spans up to 2^kMaxU consecutive values of the low bits
 constexpr int kMaxLogC = 3;      // and at most 8 columns
 constexpr int kMaxSteps = 4;     // radix-8/4/2 steps of one pass (t <= 11)
-constexpr int kThreads = 256;
 constexpr int kRootTab = (1 << kMaxT) - 1;     // w_{b+1}^k at index 2^b - 1 + k
 constexpr uint64_t kShift = 7;                 // generator and LDE coset shift
 
@@ -198,8 +191,7 @@ __device__ __forceinline__ Lz lz_m24(Lz a) {
 
 // a 2^48, lazy: with hl = bits 16..47 of l and e = (t:l1) >> 16 (signed, 48
 // bits), 2^64 = 2^32 - 1 and 2^96 = -1 give
-//   (l0 << 16 + hl) 2^32 - hl - e;  the result's t is in [-2^15 - 1, 2^15 + 1]
-// and in [-2, 2] for |t| < 2^15.
+//   (l0 << 16 + hl) 2^32 - hl - e; the result's t is in [-2, 2] (|t| < 2^31).
 __device__ __forceinline__ Lz lz_m48(Lz a) {
     const uint32_t L1 = a.l0 << 16, hl = __funnelshift_r(a.l0, a.l1, 16), e0 = __funnelshift_r(a.l1, a.t, 16);
     Lz r;
@@ -219,7 +211,7 @@ __device__ __forceinline__ Lz lz_m48(Lz a) {
 }
 
 // a 2^72, lazy: with hl = l0 << 8, hh = bits 24..55 of l and k = (t:l1) >> 24
-// (signed; |t| < 2^23), hl 2^64 + hh 2^96 + k 2^128 = (hl - k) 2^32 - hl - hh.
+// (signed; |t| < 2^22), hl 2^64 + hh 2^96 + k 2^128 = (hl - k) 2^32 - hl - hh.
 __device__ __forceinline__ Lz lz_m72(Lz a) {
     const uint32_t hl = a.l0 << 8, hh = __funnelshift_l(a.l0, a.l1, 8), k = __funnelshift_l(a.l1, a.t, 8);
     Lz r;
@@ -390,14 +382,18 @@ __device__ __forceinline__ void step(uint64_t *x, uint32_t s0, const uint64_t *w
     }
 }
 
+// Programmatic dependent launch: see pg12.cu.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // One pass.  The tile holds 2^t values of the transformed bits x 2^u
 // consecutive values of the low bits x 2^LOG_C columns; element (v, l, c) at
 // ((v 2^u + l) 2^LOG_C + c), so for fixed v the 2^u rows are one contiguous
 // run in memory.  Columns past ncols are zero and not stored.  Each low value
 // l has its own table of root powers (2^t - 1 of them, rows padded by one
 // word so that different l fall in different banks).
-template <int DIT, int LOG_C>
-__global__ void __launch_bounds__(kThreads) k_ntt_pass(const Pass ps) {
+template <int DIT, int LOG_C, int NT>
+__global__ void __launch_bounds__(NT) k_ntt_pass(const Pass ps) {
     constexpr uint32_t C = 1u << LOG_C;
     extern __shared__ uint64_t sm[];
     const uint32_t t = ps.t, u = ps.u;
@@ -407,7 +403,7 @@ __global__ void __launch_bounds__(kThreads) k_ntt_pass(const Pass ps) {
     uint64_t *tile = sm;                 // [rows][2^u][C]
     uint64_t *tw = sm + words;           // [2^u][tws]
     uint64_t *fac = tw + (tws << u);     // [rows], scale 2 only
-    __shared__ uint64_t beta[1 << kMaxU][kMaxSteps];
+    uint64_t *beta = fac + (ps.scale == 2 ? rows : 0);  // [2^u][kMaxSteps]
 
     const uint64_t chunks = (ps.ncols + C - 1) >> LOG_C;
     const uint64_t outer = chunks == 1 ? blockIdx.x : blockIdx.x / chunks;
@@ -427,12 +423,31 @@ __global__ void __launch_bounds__(kThreads) k_ntt_pass(const Pass ps) {
         plan_b |= (DIT ? done : t - done - r) << (4 * nsteps);
         done += r;
     }
-    // Each thread keeps one (low value, column) slot: kThreads is a multiple
-    // of 2^(u + LOG_C) <= 256, so its rows advance by a fixed stride.
+    // Each thread keeps one (low value, column) slot: NT is a multiple
+    // of 2^(u + LOG_C) (tile_u), so its rows advance by a fixed stride.
     const uint32_t slot = threadIdx.x & ((C << u) - 1);
     const uint32_t c_me = slot & (C - 1), l_me = slot >> LOG_C;
-    const uint32_t v_first = threadIdx.x >> (u + LOG_C), v_step = kThreads >> (u + LOG_C);
+    const uint32_t v_first = threadIdx.x >> (u + LOG_C), v_step = NT >> (u + LOG_C);
     const bool col_ok = c_me < c_eff;
+    // The pass before may still be running: until pdl_wait only the constant
+    // tables are read, and the tile's loads go out between the two halves of the
+    // root-power tables' construction.
+    pdl_trigger();
+    // beta[l * kMaxSteps + i] = w_{lo+b+r}^(low0 + l) for step i over bits [b, b + r)
+    for (uint32_t q = threadIdx.x; q < (nsteps << u); q += NT) {
+        const uint32_t i = q >> u, l = q & ((1u << u) - 1);
+        const uint32_t top = ((plan_b >> (4 * i)) & 15) + ((plan_r >> (2 * i)) & 3);
+        beta[l * kMaxSteps + i] = pow_tab(g_ntt.pw[dir], (low0 + l) << (30 - ps.lo - top));
+    }
+    if (ps.scale == 2) {
+        // row factors scale_c 7^bitrev(row) (here lo = u = 0: row = base + v)
+        for (uint32_t v = threadIdx.x; v < rows; v += NT) {
+            const uint64_t row = base + v;
+            const uint64_t j = ps.log_n ? (uint64_t)(__brevll(row) >> (64 - ps.log_n)) : 0;
+            fac[v] = mmul(pow_tab(g_ntt.coset, j), ps.scale_c);
+        }
+    }
+    pdl_wait();
     {
         // source row of tile row v: ((base | v << lo | l) >> src_shift); src_shift is
         // 0 or equal to lo, so it is linear in v either way.  With PG12_NTT_CPASYNC the
@@ -442,7 +457,7 @@ __global__ void __launch_bounds__(kThreads) k_ntt_pass(const Pass ps) {
         const uint64_t rstep = ((uint64_t)v_step << ps.lo) >> ps.src_shift;
         const uint64_t *g = ps.src + r0 * ps.ncols + col0 + c_me;
         const uint64_t gstep = rstep * ps.ncols;
-        for (uint32_t v = v_first, e = threadIdx.x; v < rows; v += v_step, e += kThreads, g += gstep) {
+        for (uint32_t v = v_first, e = threadIdx.x; v < rows; v += v_step, e += NT, g += gstep) {
 #if PG12_NTT_CPASYNC
             if (col_ok)
                 asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(tile + e)),
@@ -458,28 +473,14 @@ __global__ void __launch_bounds__(kThreads) k_ntt_pass(const Pass ps) {
         asm volatile("cp.async.commit_group;" ::: "memory");
 #endif
     }
-    // beta[l][i] = w_{lo+b+r}^(low0 + l) for step i over bits [b, b + r)
-    for (uint32_t q = threadIdx.x; q < (nsteps << u); q += kThreads) {
-        const uint32_t i = q >> u, l = q & ((1u << u) - 1);
-        const uint32_t top = ((plan_b >> (4 * i)) & 15) + ((plan_r >> (2 * i)) & 3);
-        beta[l][i] = pow_tab(g_ntt.pw[dir], (low0 + l) << (30 - ps.lo - top));
-    }
-    if (ps.scale == 2) {
-        // row factors scale_c 7^bitrev(row) (here lo = u = 0: row = base + v)
-        for (uint32_t v = threadIdx.x; v < rows; v += kThreads) {
-            const uint64_t row = base + v;
-            const uint64_t j = ps.log_n ? (uint64_t)(__brevll(row) >> (64 - ps.log_n)) : 0;
-            fac[v] = mmul(pow_tab(g_ntt.coset, j), ps.scale_c);
-        }
-    }
     __syncthreads();
     // tau^j tables: step i at bit b, low value l, rows with low bits k < 2^b
     for (uint32_t i = 0; i < nsteps; ++i) {
         const uint32_t r = (plan_r >> (2 * i)) & 3, b = (plan_b >> (4 * i)) & 15;
         const uint32_t nb = 1u << b, s = b + r - 1;
-        for (uint32_t q = threadIdx.x; q < (nb << u); q += kThreads) {
+        for (uint32_t q = threadIdx.x; q < (nb << u); q += NT) {
             const uint32_t l = q >> b, k = q & (nb - 1);
-            const uint64_t tau = mmul(beta[l][i], g_ntt.tab[dir][(1u << s) - 1 + k]);
+            const uint64_t tau = mmul(beta[l * kMaxSteps + i], g_ntt.tab[dir][(1u << s) - 1 + k]);
             uint64_t *d = tw + l * tws + nb - 1 + k;
             uint64_t x = tau;
             d[0] = x;
@@ -500,7 +501,7 @@ __global__ void __launch_bounds__(kThreads) k_ntt_pass(const Pass ps) {
         const uint32_t nb = 1u << b, s0 = 1u << (b + sh);
         const uint32_t groups = (rows >> r) << sh;
         const bool triv = b == 0 && ps.lo == 0;  // tau = w^0 (lo = 0 means u = 0)
-        for (uint32_t p = threadIdx.x; p < groups; p += kThreads) {
+        for (uint32_t p = threadIdx.x; p < groups; p += NT) {
             const uint32_t lc = p & ((C << u) - 1), g = p >> sh;
             const uint32_t k = g & (nb - 1);
             const uint32_t v0 = ((g >> b) << (b + r)) | k;
@@ -519,7 +520,7 @@ __global__ void __launch_bounds__(kThreads) k_ntt_pass(const Pass ps) {
         const uint64_t rstep = (uint64_t)v_step << ps.lo;
         uint64_t *g = ps.dst + r0 * ps.ncols + col0 + c_me;
         const uint64_t gstep = rstep * ps.ncols;
-        for (uint32_t v = v_first, e = threadIdx.x; v < rows; v += v_step, e += kThreads, g += gstep) {
+        for (uint32_t v = v_first, e = threadIdx.x; v < rows; v += v_step, e += NT, g += gstep) {
             uint64_t x = tile[e];
             if (ps.scale == 1) x = mmul(x, ps.scale_c);
             else if (ps.scale == 2) x = mmul(x, fac[v]);
@@ -532,6 +533,8 @@ __global__ void __launch_bounds__(kThreads) k_ntt_pass(const Pass ps) {
 __global__ void k_ntt_bitrev(uint64_t *__restrict__ data, uint32_t log_n, uint64_t ncols) {
     const uint64_t total = (ncols << log_n);
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+    pdl_trigger();
+    pdl_wait();
     for (uint64_t e = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += stride) {
         const uint64_t i = e / ncols, c = e - i * ncols;
         const uint64_t r = log_n ? (__brevll(i) >> (64 - log_n)) : 0;
@@ -543,24 +546,19 @@ __global__ void k_ntt_bitrev(uint64_t *__restrict__ data, uint32_t log_n, uint64
     }
 }
 
-// log2 of the tile's rows (transformed x low values) for 2^log_c columns:
-// tile plus tables stay within 72-98 KiB of shared memory.
-uint32_t tile_bits(uint32_t log_c) { return log_c >= 3 ? (uint32_t)PG12_NTT_TILE_BITS8 : log_c == 2 ? 11u : 12u; }
-uint32_t max_t(uint32_t log_c) { return tile_bits(log_c) < (uint32_t)kMaxT ? tile_bits(log_c) : (uint32_t)kMaxT; }
-
-// tile, root-power tables (2^t + 1 words per low value) and, for the LDE
-// scaling, one factor per row
-size_t pass_smem(uint32_t t, uint32_t u, uint32_t log_c, bool row_factors) {
-    return (((size_t)1 << (t + u + log_c)) + ((((size_t)1 << t) + 1) << u) + (row_factors ? (size_t)1 << t : 0)) *
-           sizeof(uint64_t);
-}
-
-// the largest pass_smem over the passes of 2^log_c columns (t + u <= tile_bits)
-size_t max_pass_smem(uint32_t log_c) {
-    const uint32_t tb = tile_bits(log_c);
-    return (((size_t)1 << (tb + log_c)) + ((size_t)1 << tb) + ((size_t)1 << kMaxU) + ((size_t)1 << max_t(log_c))) *
-           sizeof(uint64_t);
-}
+// Threads per block and log2 of the tile's rows (transformed x low values) of a
+// transform's passes.  Large transforms: blocks of 128 threads, six of them
+// resident per SM at 36 KB each (eight columns), so that the barrier after a step
+// holds up four warps; 21 rows-bits x 8 columns, blowup 2: 0.80 ms against 0.84
+// with 256 threads on 72 KB.  Below 2^19 rows (times column chunks) the grid
+// would not fill the SMs several times over and a block's serial work counts:
+// 256 threads, on tiles that shrink until there are 2^9 of them (but not below
+// 2^6 rows: more passes then cost more than they spread).  2^16 rows x 3: 16.6 us
+// against 33 with 2^11-row tiles; 2^18 x 8: 44.6 against 51.6.
+struct PassShape {
+    uint32_t threads, tile;
+};
+constexpr uint32_t kBigLog = 19;
 
 // columns per tile: the smallest power of two >= min(ncols, 8)
 uint32_t tile_log_c(uint64_t ncols) {
@@ -569,59 +567,85 @@ uint32_t tile_log_c(uint64_t ncols) {
     return lc;
 }
 
+PassShape plan_shape(uint32_t log_n, uint64_t ncols) {
+    const uint32_t lc = tile_log_c(ncols);
+    uint32_t work = log_n;  // log2 of rows x column chunks (rounded down)
+    while ((2ull << (work - log_n)) <= ((ncols + (1ull << lc) - 1) >> lc)) ++work;
+    if (work >= kBigLog) return {128, lc >= 2 ? 9u : lc == 1 ? 11u : 10u};
+    uint32_t tile = lc == 3 ? 10 : lc == 2 ? 11 : 12;
+    while (tile > 6 && work < tile + 9) --tile;
+    return {256, tile};
+}
+uint32_t max_t(const PassShape &sh) { return sh.tile < (uint32_t)kMaxT ? sh.tile : (uint32_t)kMaxT; }
+
+// tile, root-power tables (2^t + 1 words per low value), for the LDE scaling one
+// factor per row, and the steps' root powers
+size_t pass_smem(uint32_t t, uint32_t u, uint32_t log_c, bool row_factors) {
+    return (((size_t)1 << (t + u + log_c)) + ((((size_t)1 << t) + 1) << u) + (row_factors ? (size_t)1 << t : 0) +
+            ((size_t)kMaxSteps << u)) *
+           sizeof(uint64_t);
+}
+
 // low-bit span of a pass over bits [lo, lo + t)
-uint32_t tile_u(uint32_t lo, uint32_t t, uint32_t log_c) {
-    uint32_t u = tile_bits(log_c) - t;
+uint32_t tile_u(uint32_t lo, uint32_t t, const PassShape &sh, uint32_t log_c) {
+    uint32_t u = sh.tile - t, threads_log = sh.threads == 256 ? 8 : 7;
     if (u > (uint32_t)kMaxU) u = kMaxU;
+    if (u > threads_log - log_c) u = threads_log - log_c;
     return u < lo ? u : lo;
 }
 
 bool g_attr_set[64];
 
-template <int DIT, int LOG_C>
-cudaError_t set_smem_attr() {
-    return cudaFuncSetAttribute(k_ntt_pass<DIT, LOG_C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)max_pass_smem(LOG_C));
-}
+using PassKernel = void (*)(const Pass);
+template <int NT>
+constexpr PassKernel kPass[8] = {k_ntt_pass<0, 0, NT>, k_ntt_pass<0, 1, NT>, k_ntt_pass<0, 2, NT>, k_ntt_pass<0, 3, NT>,
+                                 k_ntt_pass<1, 0, NT>, k_ntt_pass<1, 1, NT>, k_ntt_pass<1, 2, NT>, k_ntt_pass<1, 3, NT>};
+// more than any pass of plan_shape needs (the largest: 2^10 rows x 8 columns with row factors, 80 KB)
+constexpr int kPassSmemMax = 112 << 10;
 
-template <int DIT, int LOG_C>
-void launch_one(const Pass &ps, unsigned blocks, size_t smem, cudaStream_t st) {
-    k_ntt_pass<DIT, LOG_C><<<blocks, kThreads, smem, st>>>(ps);
+// Launches with programmatic stream serialisation: the kernel may be scheduled
+// while the one before it on `st` finishes (both kernels here wait for it before
+// they touch the data).
+template <typename... KArgs, typename... Args>
+cudaError_t launch_dependent(void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t st,
+                             Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
 // Launches one pass; the grid is 2^(log_n - t) row groups x column chunks.
-int launch_pass(Pass ps, cudaStream_t st) {
+int launch_pass(Pass ps, const PassShape &sh, cudaStream_t st) {
     const uint32_t lc = tile_log_c(ps.ncols);
-    ps.u = tile_u(ps.lo, ps.t, lc);
+    ps.u = tile_u(ps.lo, ps.t, sh, lc);
     const uint64_t chunks = (ps.ncols + (1ull << lc) - 1) >> lc;
     const uint64_t blocks = (1ull << (ps.log_n - ps.t - ps.u)) * chunks;
     if (blocks > 0x7FFFFFFFull) return set_error(PG_ERR_INVALID_ARG, "NTT pass needs %llu blocks", (unsigned long long)blocks);
-    if (ps.t > max_t(lc)) return set_error(PG_ERR_INVALID_ARG, "NTT pass of %u bits", ps.t);
+    if (ps.t > max_t(sh)) return set_error(PG_ERR_INVALID_ARG, "NTT pass of %u bits", ps.t);
     if (ps.scale == 2 && (ps.lo != 0 || ps.u != 0)) return set_error(PG_ERR_INVALID_ARG, "row factors need lo = 0");
     const size_t smem = pass_smem(ps.t, ps.u, lc, ps.scale == 2);
     int device = 0;
     cudaGetDevice(&device);
     if (device >= 0 && device < 64 && !g_attr_set[device]) {
-        const cudaError_t es[8] = {set_smem_attr<0, 0>(), set_smem_attr<0, 1>(), set_smem_attr<0, 2>(),
-                                   set_smem_attr<0, 3>(), set_smem_attr<1, 0>(), set_smem_attr<1, 1>(),
-                                   set_smem_attr<1, 2>(), set_smem_attr<1, 3>()};
-        for (cudaError_t e : es)
+        for (int k = 0; k < 16; ++k) {
+            const PassKernel f = k < 8 ? kPass<128>[k] : kPass<256>[k - 8];
+            const cudaError_t e =
+                cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kPassSmemMax);
             if (e != cudaSuccess) return set_error(PG_ERR_CUDA, "NTT shared-memory attribute: %s", cudaGetErrorString(e));
+        }
         g_attr_set[device] = true;
     }
     ProfScope prof(kIdNttPass, st, 0);
-    const unsigned nb = (unsigned)blocks;
-    switch (lc + (ps.dit ? 4u : 0u)) {
-        case 0: launch_one<0, 0>(ps, nb, smem, st); break;
-        case 1: launch_one<0, 1>(ps, nb, smem, st); break;
-        case 2: launch_one<0, 2>(ps, nb, smem, st); break;
-        case 3: launch_one<0, 3>(ps, nb, smem, st); break;
-        case 4: launch_one<1, 0>(ps, nb, smem, st); break;
-        case 5: launch_one<1, 1>(ps, nb, smem, st); break;
-        case 6: launch_one<1, 2>(ps, nb, smem, st); break;
-        default: launch_one<1, 3>(ps, nb, smem, st); break;
-    }
-    cudaError_t e = cudaGetLastError();
+    const PassKernel f = (sh.threads == 128 ? kPass<128> : kPass<256>)[lc + (ps.dit ? 4u : 0u)];
+    const cudaError_t e = launch_dependent(f, (unsigned)blocks, sh.threads, smem, st, ps);
     if (e != cudaSuccess) return set_error(PG_ERR_CUDA, "k_ntt_pass: %s", cudaGetErrorString(e));
     return PG_OK;
 }
@@ -657,7 +681,8 @@ int plan_passes(uint32_t bits, uint32_t tmax, bool low_first, uint32_t *t_out) {
 int run_dif(const uint64_t *src, uint64_t *dst, uint32_t log_n, uint64_t ncols, bool inverse, uint32_t scale,
             uint64_t scale_c, cudaStream_t st) {
     uint32_t ts[32];
-    const int np = plan_passes(log_n, max_t(tile_log_c(ncols)), false, ts);
+    const PassShape sh = plan_shape(log_n, ncols);
+    const int np = plan_passes(log_n, max_t(sh), false, ts);
     uint32_t top = log_n;
     for (int k = 0; k < np; ++k) {
         Pass ps;
@@ -673,7 +698,7 @@ int run_dif(const uint64_t *src, uint64_t *dst, uint32_t log_n, uint64_t ncols, 
         ps.scale = k == np - 1 ? scale : 0u;
         ps.scale_c = scale_c;
         ps.last = k == np - 1 ? 1u : 0u;
-        int s = launch_pass(ps, st);
+        int s = launch_pass(ps, sh, st);
         if (s != PG_OK) return s;
         top -= ts[k];
     }
@@ -748,8 +773,7 @@ pg_status pg_ntt(uint64_t *data, size_t n, size_t ncols, int inverse, void *stre
         const uint64_t total = (uint64_t)ncols << log_n;
         const uint64_t want = (total + 255) / 256;
         const unsigned grid = (unsigned)(want < 152ull * 16 ? want : 152ull * 16);
-        k_ntt_bitrev<<<grid, 256, 0, st>>>(data, log_n, (uint64_t)ncols);
-        cudaError_t e = cudaGetLastError();
+        const cudaError_t e = launch_dependent(k_ntt_bitrev, grid, 256, 0, st, data, log_n, (uint64_t)ncols);
         if (e != cudaSuccess) return (pg_status)pg12::set_error(PG_ERR_CUDA, "k_ntt_bitrev: %s", cudaGetErrorString(e));
     }
     return PG_OK;
@@ -785,7 +809,8 @@ pg_status pg_lde(const uint64_t *evals, size_t n, size_t ncols, uint32_t log_blo
     // DIT passes over bits [b, log N) of out; the first reads coefficient row i >> b
     const uint32_t log_big = log_n + log_blowup;
     uint32_t ts[32];
-    const int np = plan_passes(log_n, max_t(tile_log_c(ncols)), true, ts);
+    const PassShape sh = plan_shape(log_big, ncols);
+    const int np = plan_passes(log_n, max_t(sh), true, ts);
     uint32_t lo = log_blowup;
     for (int k = 0; k < np; ++k) {
         Pass ps;
@@ -799,7 +824,7 @@ pg_status pg_lde(const uint64_t *evals, size_t n, size_t ncols, uint32_t log_blo
         ps.dit = 1;
         ps.src_shift = k == 0 ? log_blowup : 0;
         ps.last = k == np - 1 ? 1u : 0u;
-        s = launch_pass(ps, st);
+        s = launch_pass(ps, sh, st);
         if (s != PG_OK) return (pg_status)s;
         lo += ts[k];
     }
