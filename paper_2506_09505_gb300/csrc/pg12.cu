@@ -210,94 +210,132 @@ __global__ void __launch_bounds__(kSmallBlock) k_merkle_level(const uint64_t *__
 }
 
 // ------------------------------------------------- tensor-core kernels
-// Persistent kernels of kTcGroups groups of 128 threads (one CTA per SM:
-// its digit tables (124 KB) and the groups' A operands take 225 KB of shared
-// memory, its groups 128 columns of tensor memory each; every thread keeps
-// its state in registers).
-// Group q of CTA c takes unit c + q * gridDim.x, then every
-// gridDim.x * kTcGroups-th after: a static schedule with no shared counter,
-// so launches on different streams are independent.  A unit is 128
-// consecutive states or rows; rows past the end are computed on zeros and
-// not stored.
+// Persistent kernels, one CTA per SM, in two shapes (TPS threads per state x
+// groups per CTA): the tables (131 KB) and a group's A operand (24 KB) in shared
+// memory, 128 columns of tensor memory per group.
+//   1 x 4  one thread per state, four groups: the most permutations per second.
+//   4 x 1  four threads per state, one group: a quarter of the S-boxes and
+//          combinations per thread, for launches of few units (tc_small).
+// Group q of CTA c takes unit c + q * gridDim.x, then every (groups *
+// gridDim.x)-th after: a static schedule with no shared counter, so launches on
+// different streams are independent, and a launch of few units spreads them
+// over all SMs before any SM gets a second one.  A unit is 128 consecutive states
+// or rows; rows past the end are computed on zeros and not stored.
 #ifndef PG12_TC_GROUPS
 #define PG12_TC_GROUPS 4
 #endif
 constexpr int kTcGroups = PG12_TC_GROUPS;
-constexpr int kTcThreads = kTcGroup * kTcGroups;
-using TcL = TcLayout<kTcGroups>;
+template <int TPS>
+struct TcShape {
+    static constexpr int kGroups = TPS == 1 ? kTcGroups : 1;
+    static constexpr int kThreads = TcGroup<TPS>::kThreads * kGroups;
+    static constexpr size_t kBytes = TcLayout<kGroups>::kBytes;
+};
 
-// Group q's first unit: CTA index plus q times the grid, so that a launch of
-// few units spreads them over all SMs before any SM gets a second one.
+template <int TPS>
 __device__ __forceinline__ uint64_t tc_first_unit() {
-    return blockIdx.x + (uint64_t)gridDim.x * (threadIdx.x / kTcGroup);
+    return blockIdx.x + (uint64_t)gridDim.x * (threadIdx.x / TcGroup<TPS>::kThreads);
 }
 
-__global__ void __launch_bounds__(kTcThreads, 1) k_tc_permute(uint64_t *__restrict__ st, uint64_t n, int vec16) {
+// A tensor-core thread's words of chunk c of a row (word(i) of the chunk, i <
+// kRate / TPS; zero-filled past the row's end).  L2: through L2 only, for rows
+// written while the kernel runs.
+template <bool L2, int TPS>
+__device__ __forceinline__ void load_words(const TcGroup<TPS> &G, const uint64_t *row, uint64_t w, uint64_t c, bool vec16,
+                                           uint64_t (&ch)[kRate / TPS]) {
+    if constexpr (TPS == 1) {
+        if (L2) load_chunk_cg(row, w, c, vec16, ch);
+        else load_chunk(row, w, c, vec16, ch);
+    } else {
+#pragma unroll
+        for (int i = 0; i < kRate / TPS; ++i) {
+            const uint64_t k = c * kRate + G.word(i);
+            ch[i] = k < w ? (L2 ? __ldcg(row + k) : __ldg(row + k)) : 0ull;
+        }
+    }
+}
+// Stores the thread's words of a digest.
+template <int TPS>
+__device__ __forceinline__ void store_digest(const TcGroup<TPS> &G, uint64_t *out, const uint64_t (&x)[kT / TPS]) {
+    if constexpr (TPS == 1) {
+        st2(out, canon(x[0]), canon(x[1]));
+        st2(out + 2, canon(x[2]), canon(x[3]));
+    } else {
+        out[G.word(0)] = canon(x[0]);
+    }
+}
+
+template <int TPS>
+__global__ void __launch_bounds__(TcShape<TPS>::kThreads, 1) k_tc_permute(uint64_t *__restrict__ st, uint64_t n, int vec16) {
     extern __shared__ __align__(1024) uint8_t tc_sm[];
-    TcGroup G = tc_setup<kTcGroups>(tc_sm);
+    constexpr int kGroups = TcShape<TPS>::kGroups;
+    pdl_trigger();
+    TcGroup<TPS> G = tc_setup<TPS, kGroups>(tc_sm);
+    pdl_wait();
+    tc_tables_ready<TPS, kGroups>(tc_sm, G);
     const uint64_t units = (n + kTcGroup - 1) / kTcGroup;
-    const uint64_t step = (uint64_t)gridDim.x * kTcGroups;
-    for (uint64_t u = tc_first_unit(); u < units; u += step) {
-        const uint64_t k = u * kTcGroup + G.t;
+    const uint64_t step = (uint64_t)gridDim.x * kGroups;
+    for (uint64_t u = tc_first_unit<TPS>(); u < units; u += step) {
+        const uint64_t k = u * kTcGroup + G.row();
         const bool valid = k < n;
         uint64_t *p = st + kT * k;
-        uint64_t x[kT];
-        if (valid && vec16) {
+        uint64_t x[kT / TPS];
+        if (TPS == 1 && valid && vec16) {
 #pragma unroll
-            for (int i = 0; i < kT; i += 2) ld2_nc(p + i, x[i], x[i + 1]);
+            for (int i = 0; i < kT / TPS; i += 2) ld2_nc(p + i, x[i], x[i + 1]);
         } else {
 #pragma unroll
-            for (int i = 0; i < kT; ++i) x[i] = valid ? p[i] : 0ull;
+            for (int i = 0; i < kT / TPS; ++i) x[i] = valid ? p[G.word(i)] : 0ull;
         }
         if (!tc_permute(G, x, false, false)) break;
         if (valid) {
-            if (vec16) {
+            if (TPS == 1 && vec16) {
 #pragma unroll
-                for (int i = 0; i < kT; i += 2) st2(p + i, canon(x[i]), canon(x[i + 1]));
+                for (int i = 0; i < kT / TPS; i += 2) st2(p + i, canon(x[i]), canon(x[i + 1]));
             } else {
 #pragma unroll
-                for (int i = 0; i < kT; ++i) p[i] = canon(x[i]);
+                for (int i = 0; i < kT / TPS; ++i) p[G.word(i)] = canon(x[i]);
             }
         }
     }
-    tc_teardown<kTcGroups>(tc_sm, G);
+    tc_teardown<TPS, kGroups>(tc_sm, G);
 }
 
 // Sponge digests of n rows of width w (Sec. 2.4): the leaves of a tree, or a
 // tree level (the level below read as rows of its children's 8 words), or
 // pg_hash_rows.  Launched as a dependent launch it may set up while the
 // kernel before it finishes, and reads `rows` only after pdl_wait().
-__global__ void __launch_bounds__(kTcThreads, 1) k_tc_sponge(const uint64_t *__restrict__ rows, uint64_t n,
-                                                             uint64_t w, int vec16, uint64_t *__restrict__ out) {
+template <int TPS>
+__global__ void __launch_bounds__(TcShape<TPS>::kThreads, 1) k_tc_sponge(const uint64_t *__restrict__ rows, uint64_t n,
+                                                                         uint64_t w, int vec16, uint64_t *__restrict__ out) {
     extern __shared__ __align__(1024) uint8_t tc_sm[];
+    constexpr int kGroups = TcShape<TPS>::kGroups;
     pdl_trigger();
-    TcGroup G = tc_setup<kTcGroups>(tc_sm);
+    TcGroup<TPS> G = tc_setup<TPS, kGroups>(tc_sm);
     pdl_wait();
+    tc_tables_ready<TPS, kGroups>(tc_sm, G);
     const uint64_t units = (n + kTcGroup - 1) / kTcGroup;
-    const uint64_t step = (uint64_t)gridDim.x * kTcGroups;
+    const uint64_t step = (uint64_t)gridDim.x * kGroups;
     const uint64_t chunks = (w + kRate - 1) / kRate;
-    for (uint64_t u = tc_first_unit(); u < units; u += step) {
-        const uint64_t r = u * kTcGroup + G.t;
+    for (uint64_t u = tc_first_unit<TPS>(); u < units; u += step) {
+        const uint64_t r = u * kTcGroup + G.row();
         const bool valid = r < n;
         const uint64_t *row = rows + (valid ? r : 0) * w;
-        uint64_t x[kT];
+        uint64_t x[kT / TPS];
 #pragma unroll
-        for (int i = kRate; i < kT; ++i) x[i] = 0;
+        for (int i = kRate / TPS; i < kT / TPS; ++i) x[i] = 0;
         bool ok = true;
         for (uint64_t c = 0; c < chunks && ok; ++c) {
-            uint64_t ch[kRate];
-            load_chunk(row, w, c, vec16 != 0, ch);
+            uint64_t ch[kRate / TPS];
+            load_words<false>(G, row, w, c, vec16 != 0, ch);
 #pragma unroll
-            for (int i = 0; i < kRate; ++i) x[i] = valid ? ch[i] : 0ull;
+            for (int i = 0; i < kRate / TPS; ++i) x[i] = valid ? ch[i] : 0ull;
             ok = tc_permute(G, x, c == 0, c + 1 == chunks);
         }
         if (!ok) break;
-        if (valid) {
-            st2(out + kDigest * r, canon(x[0]), canon(x[1]));
-            st2(out + kDigest * r + 2, canon(x[2]), canon(x[3]));
-        }
+        if (valid) store_digest(G, out + kDigest * r, x);
     }
-    tc_teardown<kTcGroups>(tc_sm, G);
+    tc_teardown<TPS, kGroups>(tc_sm, G);
 }
 
 // Leaf sponges over rows that arrive in chunks while the kernel runs
@@ -325,16 +363,17 @@ __device__ __forceinline__ bool wait_ready(const uint32_t *ready, uint32_t want)
     }
 }
 
-__global__ void __launch_bounds__(kTcThreads, 1)
+__global__ void __launch_bounds__(TcShape<1>::kThreads, 1)
     k_tc_leaves_stream(const uint64_t *__restrict__ rows, uint64_t n, uint64_t w, int vec16,
                        uint64_t *__restrict__ out, const uint32_t *__restrict__ ready, const ChunkMap cm) {
     extern __shared__ __align__(1024) uint8_t tc_sm[];
-    TcGroup G = tc_setup<kTcGroups>(tc_sm);
+    TcGroup<1> G = tc_setup<1, kTcGroups>(tc_sm);
+    tc_tables_ready<1, kTcGroups>(tc_sm, G);
     const uint64_t units = (n + kTcGroup - 1) / kTcGroup;
     const uint64_t step = (uint64_t)gridDim.x * kTcGroups;
     const uint64_t chunks = (w + kRate - 1) / kRate;
     uint32_t have = 0;  // chunks this group has seen arrive
-    for (uint64_t u = tc_first_unit(); u < units; u += step) {
+    for (uint64_t u = tc_first_unit<1>(); u < units; u += step) {
         const uint64_t last = (u + 1) * kTcGroup < n ? (u + 1) * kTcGroup - 1 : n - 1;
         uint32_t c = 0;
         while (c + 1 < cm.count && cm.end[c] <= last) ++c;
@@ -361,12 +400,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             ok = tc_permute(G, x, k == 0, k + 1 == chunks);
         }
         if (!ok) break;
-        if (valid) {
-            st2(out + kDigest * r, canon(x[0]), canon(x[1]));
-            st2(out + kDigest * r + 2, canon(x[2]), canon(x[3]));
-        }
+        if (valid) store_digest(G, out + kDigest * r, x);
     }
-    tc_teardown<kTcGroups>(tc_sm, G);
+    tc_teardown<1, kTcGroups>(tc_sm, G);
 }
 
 // One warp task: lane i of task u at level l hashes node 32u+i of that level
@@ -512,9 +548,10 @@ __device__ __forceinline__ uint64_t tc_units(uint64_t n, uint32_t l) {
 // sponge of leaf row k (l = 0) or the compression of children 2k, 2k + 1
 // (read from L2: other groups of this launch wrote them).  Rows past the
 // level's end are computed on zeros and not stored.
-__device__ __forceinline__ bool tc_unit(TcGroup &G, const TreePlan &tp, uint32_t l, uint64_t u) {
+template <int TPS>
+__device__ __forceinline__ bool tc_unit(TcGroup<TPS> &G, const TreePlan &tp, uint32_t l, uint64_t u) {
     const uint64_t n = tp.n_leaves, cnt = n >> l;
-    const uint64_t k = u * kTcGroup + G.t;
+    const uint64_t k = u * kTcGroup + G.row();
     const bool valid = k < cnt;
     // a node is the one-chunk sponge of its children's 8 words; one
     // permutation call site for leaves and nodes keeps the kernel's code small
@@ -522,26 +559,18 @@ __device__ __forceinline__ bool tc_unit(TcGroup &G, const TreePlan &tp, uint32_t
     const uint64_t w = leaf ? tp.width : 2 * kDigest, chunks = (w + kRate - 1) / kRate;
     const uint64_t *row = leaf ? tp.rows + (valid ? k : 0) * w
                                : tp.nodes + kDigest * (level_off(n, l - 1) + 2 * (valid ? k : 0));
-    uint64_t x[kT];
+    uint64_t x[kT / TPS];
 #pragma unroll
-    for (int i = kRate; i < kT; ++i) x[i] = 0;
+    for (int i = kRate / TPS; i < kT / TPS; ++i) x[i] = 0;
     for (uint64_t c = 0; c < chunks; ++c) {
-        uint64_t ch[kRate];
-        if (leaf) {
-            load_chunk(row, w, c, tp.vec16 != 0, ch);
-        } else {  // written by this launch: coherent loads
+        uint64_t ch[kRate / TPS];
+        if (leaf) load_words<false>(G, row, w, c, tp.vec16 != 0, ch);
+        else load_words<true>(G, row, w, c, true, ch);  // written by this launch: coherent loads
 #pragma unroll
-            for (int i = 0; i < kRate; i += 2) ld2_cg(row + i, ch[i], ch[i + 1]);
-        }
-#pragma unroll
-        for (int i = 0; i < kRate; ++i) x[i] = valid ? ch[i] : 0ull;
+        for (int i = 0; i < kRate / TPS; ++i) x[i] = valid ? ch[i] : 0ull;
         if (!tc_permute(G, x, c == 0, c + 1 == chunks)) return false;
     }
-    if (valid) {
-        uint64_t *dst = tp.nodes + kDigest * (level_off(n, l) + k);
-        st2(dst, canon(x[0]), canon(x[1]));
-        st2(dst + 2, canon(x[2]), canon(x[3]));
-    }
+    if (valid) store_digest(G, tp.nodes + kDigest * (level_off(n, l) + k), x);
     return true;
 }
 
@@ -552,20 +581,24 @@ __device__ __forceinline__ bool tc_unit(TcGroup &G, const TreePlan &tp, uint32_t
 // and 45 us beside three other groups, one in this form 6.4 us.  The constants
 // are read from global memory (they stay in L1; shared memory is full).
 constexpr uint64_t kTcSmallLevel = 16;
-constexpr int kTcWideNodes = kTcGroup / 16;
+template <int TPS>
 struct TcSmall {
-    WideBuf<16, kTcGroup> buf;
+    static constexpr int kNodes = TcGroup<TPS>::kThreads / 16;  // built at a time
+    WideBuf<16, TcGroup<TPS>::kThreads> buf;
     uint64_t dig[2][kTcSmallLevel * kDigest];
+    static_assert(TcGroup<TPS>::kThreads % 32 == 0, "whole warps");
 };
-static_assert(sizeof(TcSmall) <= kTcABytes, "the scratch of the small levels lies in the A operand");
+static_assert(sizeof(TcSmall<1>) <= kTcABytes && sizeof(TcSmall<4>) <= kTcABytes,
+              "the scratch of the small levels lies in the A operand");
+template <int TPS>
 __device__ __noinline__ void tc_climb_small(uint8_t *scratch, int bar, int t, uint64_t *nodes, uint64_t n, uint32_t level,
                                             uint32_t log_n) {
-    TcSmall &S = *reinterpret_cast<TcSmall *>(scratch);
+    TcSmall<TPS> &S = *reinterpret_cast<TcSmall<TPS> *>(scratch);
     const int l16 = t & 15;
     const uint64_t *below = nodes + kDigest * level_off(n, level - 1);
     for (uint32_t l = level; l <= log_n; ++l) {
         const uint64_t count = n >> l;
-        for (uint64_t first = 0; first < count; first += kTcWideNodes) {
+        for (uint64_t first = 0; first < count; first += TcSmall<TPS>::kNodes) {
             const uint64_t node = first + (t >> 4);
             // whole warps hold nodes 2w and 2w + 1; a warp past the level's end skips it
             if ((node & ~1ull) < count) {
@@ -583,21 +616,24 @@ __device__ __noinline__ void tc_climb_small(uint8_t *scratch, int bar, int t, ui
                 }
             }
         }
-        group_sync(bar);
+        group_sync(bar, TcGroup<TPS>::kThreads);
     }
 }
 
-__global__ void __launch_bounds__(kTcThreads, 1) k_tc_batch(const TreePlan *__restrict__ plans, uint32_t n_trees,
+template <int TPS>
+__global__ void __launch_bounds__(TcShape<TPS>::kThreads, 1) k_tc_batch(const TreePlan *__restrict__ plans, uint32_t n_trees,
                                                             uint32_t total_tasks, uint32_t fuse,
                                                             uint32_t *__restrict__ counters,
                                                             uint32_t *__restrict__ next_task) {
     extern __shared__ __align__(1024) uint8_t tc_sm[];
-    TcGroup G = tc_setup<kTcGroups>(tc_sm);
+    constexpr int kGroups = TcShape<TPS>::kGroups;
+    TcGroup<TPS> G = tc_setup<TPS, kGroups>(tc_sm);
+    tc_tables_ready<TPS, kGroups>(tc_sm, G);
     bool ok = true;
     // every group's first task is fixed, CTA by CTA, so that few tasks spread
     // over all SMs; the others come from the counter
-    const uint32_t groups = gridDim.x * kTcGroups;
-    for (uint32_t task = (uint32_t)tc_first_unit(); ok && task < total_tasks;
+    const uint32_t groups = gridDim.x * kGroups;
+    for (uint32_t task = (uint32_t)tc_first_unit<TPS>(); ok && task < total_tasks;
          task = groups + group_fetch_add(G, next_task)) {
         uint32_t lo_t = 0, hi_t = n_trees - 1;
         while (lo_t < hi_t) {
@@ -623,15 +659,15 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_batch(const TreePlan *__re
             __threadfence();
             if (cnt >= 2) {
                 // both children of every parent unit are this task's: no counter
-                group_sync(G.bar);
+                group_sync(G.bar, TcGroup<TPS>::kThreads);
                 lo >>= 1;
                 cnt >>= 1;
                 continue;
             }
             if (top == log_n && (n >> (l + 1)) <= kTcSmallLevel) {
                 // the rest of the tree (the children below are this group's: one unit)
-                group_sync(G.bar);
-                tc_climb_small(G.a, G.bar, G.t, tp.nodes, n, l + 1, log_n);
+                group_sync(G.bar, TcGroup<TPS>::kThreads);
+                tc_climb_small<TPS>(G.a, G.bar, G.t, tp.nodes, n, l + 1, log_n);
                 if (G.t == 0) signal_root(tp, 0);
                 break;
             }
@@ -640,12 +676,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_batch(const TreePlan *__re
                 if (old == 0) break;  // the sibling unit is not done: its group builds the parent
                 __threadfence();
             } else {
-                group_sync(G.bar);
+                group_sync(G.bar, TcGroup<TPS>::kThreads);
             }
             lo >>= 1;
         }
     }
-    tc_teardown<kTcGroups>(tc_sm, G);
+    tc_teardown<TPS, kGroups>(tc_sm, G);
 }
 
 // The top levels of every tree of a batch whose persistent launch stopped
@@ -854,6 +890,8 @@ __global__ void __launch_bounds__(kTopBlock) k_merkle_top_leaf(const uint64_t *_
 // Authentication paths: thread per (query, level) copies one sibling digest.
 __global__ void k_merkle_open(const uint64_t *__restrict__ nodes, uint64_t n, uint32_t depth,
                               const uint64_t *__restrict__ idx, uint64_t k, uint64_t *__restrict__ paths) {
+    pdl_trigger();
+    pdl_wait();
     const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= k * depth) return;
     const uint64_t q = t / depth;
@@ -914,7 +952,9 @@ __global__ void __launch_bounds__(kVerifyWideBlock) k_merkle_verify_wide(const u
                                                                          uint8_t *__restrict__ ok) {
     __shared__ __align__(16) WideConsts K;
     __shared__ __align__(16) WideBuf<LANES, kVerifyWideBlock> buf;
+    pdl_trigger();
     load_consts(K);
+    pdl_wait();
     const unsigned full = 0xFFFFFFFFu;
     const uint64_t gid = ((uint64_t)blockIdx.x * kVerifyWideBlock + threadIdx.x) / LANES;
     const uint64_t q = gid < k ? gid : 0;  // groups past the end repeat query 0 and store nothing
@@ -939,43 +979,56 @@ __global__ void __launch_bounds__(kVerifyWideBlock) k_merkle_verify_wide(const u
 
 // The same with 128 queries per tensor-core group: a unit is 128 queries, and
 // each level is one permutation of the group.
-__global__ void __launch_bounds__(kTcThreads, 1) k_tc_verify(const uint64_t *__restrict__ root, uint32_t depth, uint64_t n,
-                                                             const uint64_t *__restrict__ leaves,
-                                                             const uint64_t *__restrict__ idx, uint64_t k,
-                                                             const uint64_t *__restrict__ paths, uint8_t *__restrict__ ok) {
+template <int TPS>
+__global__ void __launch_bounds__(TcShape<TPS>::kThreads, 1) k_tc_verify(const uint64_t *__restrict__ root, uint32_t depth,
+                                                                         uint64_t n, const uint64_t *__restrict__ leaves,
+                                                                         const uint64_t *__restrict__ idx, uint64_t k,
+                                                                         const uint64_t *__restrict__ paths,
+                                                                         uint8_t *__restrict__ ok) {
     extern __shared__ __align__(1024) uint8_t tc_sm[];
-    TcGroup G = tc_setup<kTcGroups>(tc_sm);
+    constexpr int kGroups = TcShape<TPS>::kGroups, kOwn = kDigest / TPS, kThreads = TcGroup<TPS>::kThreads;
+    pdl_trigger();
+    TcGroup<TPS> G = tc_setup<TPS, kGroups>(tc_sm);
+    pdl_wait();
+    tc_tables_ready<TPS, kGroups>(tc_sm, G);
     const uint64_t units = (k + kTcGroup - 1) / kTcGroup;
-    const uint64_t step = (uint64_t)gridDim.x * kTcGroups;
+    const uint64_t step = (uint64_t)gridDim.x * kGroups;
     bool fine = true;
-    for (uint64_t u = tc_first_unit(); u < units && fine; u += step) {
-        const uint64_t gid = u * kTcGroup + G.t;
+    for (uint64_t u = tc_first_unit<TPS>(); u < units && fine; u += step) {
+        const uint64_t gid = u * kTcGroup + G.row();
         const uint64_t q = gid < k ? gid : 0;
-        uint64_t x[kT];
+        uint64_t x[kT / TPS];  // words: left child, right child, zero capacity
 #pragma unroll
-        for (int i = 0; i < kDigest; ++i) x[i] = leaves[kDigest * q + i];
+        for (int i = 0; i < kOwn; ++i) x[i] = leaves[kDigest * q + G.word(i)];
         const uint64_t pos = idx[q];
         for (uint32_t l = 0; l < depth && fine; ++l) {
             const uint64_t *sib = paths + kDigest * (q * depth + l);
             const bool right = (pos >> l) & 1u;
 #pragma unroll
-            for (int i = 0; i < kDigest; ++i) {
-                const uint64_t s = sib[i], c = x[i];
+            for (int i = 0; i < kOwn; ++i) {
+                const uint64_t s = sib[G.word(i)], c = x[i];
                 x[i] = right ? s : c;
-                x[kDigest + i] = right ? c : s;
-                x[2 * kDigest + i] = 0;
+                x[kOwn + i] = right ? c : s;
+                x[2 * kOwn + i] = 0;
             }
             fine = tc_permute(G, x, true, true);
 #pragma unroll
-            for (int i = 0; i < kDigest; ++i) x[i] = canon(x[i]);
+            for (int i = 0; i < kOwn; ++i) x[i] = canon(x[i]);
         }
         if (!fine) break;
         bool eq = pos < n;
 #pragma unroll
-        for (int i = 0; i < kDigest; ++i) eq = eq && x[i] == root[i];
-        if (gid < k) ok[gid] = eq ? 1 : 0;
+        for (int i = 0; i < kOwn; ++i) eq = eq && x[i] == root[G.word(i)];
+        if constexpr (TPS > 1) {  // the parts' answers through the idle A operand
+            G.a[G.t] = eq ? 1 : 0;
+            group_sync(G.bar, kThreads);
+#pragma unroll
+            for (int h = 0; h < TPS; ++h) eq = eq && G.a[h * kTcGroup + G.row()];
+            group_sync(G.bar, kThreads);
+        }
+        if (G.part() == 0 && gid < k) ok[gid] = eq ? 1 : 0;
     }
-    tc_teardown<kTcGroups>(tc_sm, G);
+    tc_teardown<TPS, kGroups>(tc_sm, G);
 }
 
 }  // namespace dev
@@ -1328,11 +1381,12 @@ pg_status plan_batch(const pg_tree *trees, size_t n_trees, const pg_schedule *sc
 // pdl_trigger / pdl_wait): it may start, and copy its constants, while the
 // kernel before it on `st` finishes.
 template <typename... KArgs, typename... Args>
-cudaError_t launch_dependent(void (*kernel)(KArgs...), unsigned grid, unsigned block, cudaStream_t st, Args... args) {
+cudaError_t launch_dependent(void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t st,
+                             Args... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1342,29 +1396,30 @@ cudaError_t launch_dependent(void (*kernel)(KArgs...), unsigned grid, unsigned b
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
-// Tensor-core kernels: one CTA per SM at most; with fewer units than four per
-// SM the CTAs' groups fill evenly (tc_first_unit).
+// Four threads per state for launches of at most one unit per SM (a permutation
+// 18.8 us against 22; with a second unit per SM 38 us, two groups side by side
+// 26.6) and for batches of at most four leaf tasks per SM, whose time is the
+// climb (32 trees of 2^8 .. 2^12 leaves, 426 tasks: 409 against 479 us; 772 tasks:
+// 711 against 695).
+bool tc_small(uint64_t units) { return units <= (uint64_t)g.sms; }
+bool tc_small_batch(uint64_t tasks) { return tasks <= 4 * (uint64_t)g.sms; }
+uint64_t tc_units_of(uint64_t n) { return (n + dev::kTcGroup - 1) / dev::kTcGroup; }
+
+// Tensor-core kernels: one CTA per SM at most; with fewer units than groups the
+// CTAs fill evenly (tc_first_unit).
 unsigned tc_grid(uint64_t n) {
     const uint64_t units = (n + dev::kTcGroup - 1) / dev::kTcGroup;
     return (unsigned)(units < (uint64_t)g.sms ? units : (uint64_t)g.sms);
 }
 
-pg_status launch_tc_sponge(const uint64_t *rows, uint64_t n, uint64_t w, uint64_t *out, cudaStream_t st, bool dependent,
-                           int kid) {
+pg_status launch_tc_sponge(const uint64_t *rows, uint64_t n, uint64_t w, uint64_t *out, cudaStream_t st, int kid) {
     if (n == 0) return PG_OK;
     const int vec16 = ((w % 2) == 0 && (reinterpret_cast<uintptr_t>(rows) % 16) == 0) ? 1 : 0;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(tc_grid(n));
-    cfg.blockDim = dim3(dev::kTcThreads);
-    cfg.dynamicSmemBytes = dev::TcL::kBytes;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = dependent ? 1 : 0;
+    const bool small = tc_small(tc_units_of(n));
     ProfScope prof(kid, st, n * ((w + kRate - 1) / kRate));
-    PG_CUDA(cudaLaunchKernelEx(&cfg, dev::k_tc_sponge, rows, n, w, vec16, out));
+    PG_CUDA(launch_dependent(small ? dev::k_tc_sponge<4> : dev::k_tc_sponge<1>, tc_grid(n),
+                             small ? dev::TcShape<4>::kThreads : dev::TcShape<1>::kThreads,
+                             small ? dev::TcShape<4>::kBytes : dev::TcShape<1>::kBytes, st, rows, n, w, vec16, out));
     return PG_OK;
 }
 
@@ -1374,7 +1429,7 @@ pg_status launch_leaves_stream(const uint64_t *rows, uint64_t n, uint64_t w, uin
                                const dev::ChunkMap &cm, cudaStream_t st) {
     const int vec16 = ((w % 2) == 0 && (reinterpret_cast<uintptr_t>(rows) % 16) == 0) ? 1 : 0;
     ProfScope prof(kIdTcLeaves, st, n * ((w + kRate - 1) / kRate));
-    dev::k_tc_leaves_stream<<<tc_grid(n), dev::kTcThreads, dev::TcL::kBytes, st>>>(rows, n, w, vec16, out, ready, cm);
+    dev::k_tc_leaves_stream<<<tc_grid(n), dev::TcShape<1>::kThreads, dev::TcShape<1>::kBytes, st>>>(rows, n, w, vec16, out, ready, cm);
     PG_CUDA(cudaGetLastError());
     return PG_OK;
 }
@@ -1386,14 +1441,14 @@ pg_status launch_levels(uint64_t *nodes, uint64_t n_leaves, uint32_t first, cuda
         if (cnt <= dev::kTailNodes && l < log_n) {
             // this level and all above it in one cluster
             ProfScope prof(kIdMerkleTopTail, st, 2 * cnt - 1);
-            PG_CUDA(launch_dependent(dev::k_merkle_top_tail, dev::kTailCtas, dev::kTailBlock, st, nodes, n_leaves, l));
+            PG_CUDA(launch_dependent(dev::k_merkle_top_tail, dev::kTailCtas, dev::kTailBlock, 0, st, nodes, n_leaves, l));
             break;
         }
         if (g.engine == 1 && cnt >= g.tc_min_nodes) {
             // the level below, read as cnt rows of 8 words (children 2k, 2k+1)
             const uint64_t *below = nodes + 4 * (2 * n_leaves - ((2 * n_leaves) >> (l - 1)));
             uint64_t *here = nodes + 4 * (2 * n_leaves - ((2 * n_leaves) >> l));
-            pg_status s = launch_tc_sponge(below, cnt, 2 * kDigest, here, st, true, kIdTcLevel);
+            pg_status s = launch_tc_sponge(below, cnt, 2 * kDigest, here, st, kIdTcLevel);
             if (s != PG_OK) return s;
         } else if (cnt > kWideNodes) {
             const uint64_t *below = nodes + 4 * (2 * n_leaves - ((2 * n_leaves) >> (l - 1)));
@@ -1401,14 +1456,14 @@ pg_status launch_levels(uint64_t *nodes, uint64_t n_leaves, uint32_t first, cuda
             const unsigned grid = (unsigned)((cnt + 127) / 128);
             ProfScope prof(kIdMerkleLevel, st, cnt);
             if (g.params_set == 1)
-                PG_CUDA(launch_dependent(dev::k_merkle_level<dev::kMdsSmall>, grid, 128, st, below, cnt, here));
+                PG_CUDA(launch_dependent(dev::k_merkle_level<dev::kMdsSmall>, grid, 128, 0, st, below, cnt, here));
             else
-                PG_CUDA(launch_dependent(dev::k_merkle_level<dev::kMdsFull>, grid, 128, st, below, cnt, here));
+                PG_CUDA(launch_dependent(dev::k_merkle_level<dev::kMdsFull>, grid, 128, 0, st, below, cnt, here));
         } else {
             const unsigned lanes = wide_lanes(cnt);
             const unsigned grid = (unsigned)((cnt * lanes + dev::kTopBlock - 1) / dev::kTopBlock);
             ProfScope prof(kIdMerkleTop, st, cnt);
-            PG_CUDA(launch_dependent(lanes == 32 ? dev::k_merkle_top<32> : dev::k_merkle_top<16>, grid, dev::kTopBlock, st,
+            PG_CUDA(launch_dependent(lanes == 32 ? dev::k_merkle_top<32> : dev::k_merkle_top<16>, grid, dev::kTopBlock, 0, st,
                                      nodes, n_leaves, l));
         }
     }
@@ -1417,7 +1472,7 @@ pg_status launch_levels(uint64_t *nodes, uint64_t n_leaves, uint32_t first, cuda
 
 // Leaf digests of rows[0 .. n) on `st` (k_hash_rows, grid capped like pg_hash_rows).
 pg_status launch_leaves(const uint64_t *rows, uint64_t n, uint64_t width, uint64_t *digests, cudaStream_t st) {
-    if (g.engine == 1) return launch_tc_sponge(rows, n, width, digests, st, false, kIdTcRows);
+    if (g.engine == 1) return launch_tc_sponge(rows, n, width, digests, st, kIdTcRows);
     const int vec16 = ((width % 2) == 0 && (reinterpret_cast<uintptr_t>(rows) % 16) == 0) ? 1 : 0;
     const uint64_t want = (n + 127) / 128;
     const uint64_t cap = (uint64_t)g.sms * g.permute_blocks_per_sm * 8;
@@ -1477,8 +1532,12 @@ pg_status launch_batch(const pg_schedule *sched, const dev::TreePlan *d_plans, u
         const unsigned grid = tasks < (uint32_t)g.sms ? tasks : (uint32_t)g.sms;
         if (grid > 0) {
             ProfScope prof(kIdTcBatch, st, perms - top_perms);
-            dev::k_tc_batch<<<grid, dev::kTcThreads, dev::TcL::kBytes, st>>>(d_plans, n_trees, tasks, fuse, d_counters + 1,
-                                                                              d_counters);
+            if (tc_small_batch(tasks))
+                dev::k_tc_batch<4><<<grid, dev::TcShape<4>::kThreads, dev::TcShape<4>::kBytes, st>>>(
+                    d_plans, n_trees, tasks, fuse, d_counters + 1, d_counters);
+            else
+                dev::k_tc_batch<1><<<grid, dev::TcShape<1>::kThreads, dev::TcShape<1>::kBytes, st>>>(
+                    d_plans, n_trees, tasks, fuse, d_counters + 1, d_counters);
             PG_CUDA(cudaGetLastError());
         }
     } else {
@@ -1927,12 +1986,18 @@ pg_status pg_init(int device, const char *params_path) {
     PG_CUDA(cudaSetDevice(device));
     s = upload_tables();
     if (s != PG_OK) return s;
-    PG_CUDA(cudaFuncSetAttribute(dev::k_tc_permute, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dev::TcL::kBytes));
-    PG_CUDA(cudaFuncSetAttribute(dev::k_tc_sponge, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dev::TcL::kBytes));
-    PG_CUDA(cudaFuncSetAttribute(dev::k_tc_verify, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dev::TcL::kBytes));
-    PG_CUDA(cudaFuncSetAttribute(dev::k_tc_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dev::TcL::kBytes));
-    PG_CUDA(cudaFuncSetAttribute(dev::k_tc_leaves_stream, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)dev::TcL::kBytes));
+    const auto dyn = [](auto kernel, size_t bytes) {
+        return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    };
+    PG_CUDA(dyn(dev::k_tc_permute<1>, dev::TcShape<1>::kBytes));
+    PG_CUDA(dyn(dev::k_tc_permute<4>, dev::TcShape<4>::kBytes));
+    PG_CUDA(dyn(dev::k_tc_sponge<1>, dev::TcShape<1>::kBytes));
+    PG_CUDA(dyn(dev::k_tc_sponge<4>, dev::TcShape<4>::kBytes));
+    PG_CUDA(dyn(dev::k_tc_verify<1>, dev::TcShape<1>::kBytes));
+    PG_CUDA(dyn(dev::k_tc_verify<4>, dev::TcShape<4>::kBytes));
+    PG_CUDA(dyn(dev::k_tc_batch<1>, dev::TcShape<1>::kBytes));
+    PG_CUDA(dyn(dev::k_tc_batch<4>, dev::TcShape<4>::kBytes));
+    PG_CUDA(dyn(dev::k_tc_leaves_stream, dev::TcShape<1>::kBytes));
     {
         const int ns = ntt_upload_constants();
         if (ns != PG_OK) return (pg_status)ns;
@@ -2017,8 +2082,11 @@ pg_status pg_permute_batch(uint64_t *states, size_t n, void *stream) {
     const int vec16 = (reinterpret_cast<uintptr_t>(states) % 16) == 0;
     if (g.engine == 1) {
         ProfScope prof(kIdTcPermute, as_stream(stream), (uint64_t)n);
-        dev::k_tc_permute<<<tc_grid(n), dev::kTcThreads, dev::TcL::kBytes, as_stream(stream)>>>(states, (uint64_t)n, vec16);
-        PG_CUDA(cudaGetLastError());
+        const bool small = tc_small(tc_units_of(n));
+        PG_CUDA(launch_dependent(small ? dev::k_tc_permute<4> : dev::k_tc_permute<1>, tc_grid(n),
+                                 small ? dev::TcShape<4>::kThreads : dev::TcShape<1>::kThreads,
+                                 small ? dev::TcShape<4>::kBytes : dev::TcShape<1>::kBytes, as_stream(stream), states,
+                                 (uint64_t)n, vec16));
         return PG_OK;
     }
     const uint64_t want = (n + 127) / 128;
@@ -2039,7 +2107,7 @@ pg_status pg_hash_rows(const uint64_t *rows, size_t n_rows, size_t width, uint64
     if (!rows || !digests) return fail(PG_ERR_INVALID_ARG, "rows or digests is NULL");
     if (reinterpret_cast<uintptr_t>(rows) % 8) return fail(PG_ERR_INVALID_ARG, "rows not 8-byte aligned");
     if (reinterpret_cast<uintptr_t>(digests) % 16) return fail(PG_ERR_INVALID_ARG, "digests not 16-byte aligned");
-    if (g.engine == 1) return launch_tc_sponge(rows, n_rows, width, digests, as_stream(stream), false, kIdTcRows);
+    if (g.engine == 1) return launch_tc_sponge(rows, n_rows, width, digests, as_stream(stream), kIdTcRows);
     const int vec16 = (width % 2 == 0) && (reinterpret_cast<uintptr_t>(rows) % 16) == 0;
     const uint64_t want = (n_rows + 127) / 128;
     const uint64_t cap = (uint64_t)g.sms * g.permute_blocks_per_sm * 8;
@@ -2079,7 +2147,7 @@ pg_status pg_merkle_build(const uint64_t *rows, size_t n_leaves, size_t width, u
             rows, (uint64_t)n_leaves, (uint64_t)width, nodes);
         PG_CUDA(cudaGetLastError());
     } else if (g.engine == 1) {
-        s = launch_tc_sponge(rows, n_leaves, width, nodes, st, false, kIdTcLeaves);
+        s = launch_tc_sponge(rows, n_leaves, width, nodes, st, kIdTcLeaves);
         if (s != PG_OK) return s;
     } else {
         dev::TreePlan tp;
@@ -2530,8 +2598,8 @@ pg_status pg_merkle_open(const uint64_t *nodes, size_t n_leaves, const uint64_t 
     const uint64_t threads = (uint64_t)k * depth;
     const unsigned grid = (unsigned)((threads + 255) / 256);
     pg12::ProfScope prof(pg12::kIdOpen, as_stream(stream), 0);
-    dev::k_merkle_open<<<grid, 256, 0, as_stream(stream)>>>(nodes, (uint64_t)n_leaves, depth, indices, (uint64_t)k, paths);
-    PG_CUDA(cudaGetLastError());
+    PG_CUDA(launch_dependent(dev::k_merkle_open, grid, 256, 0, as_stream(stream), nodes, (uint64_t)n_leaves, depth, indices,
+                             (uint64_t)k, paths));
     return PG_OK;
 }
 
@@ -2549,11 +2617,15 @@ pg_status pg_merkle_verify(const uint64_t *root, size_t n_leaves, const uint64_t
     if (k <= kVerifyWideMax) {
         const unsigned lanes = wide_lanes(k);
         const unsigned wide = (unsigned)((k * lanes + dev::kVerifyWideBlock - 1) / dev::kVerifyWideBlock);
-        (lanes == 32 ? dev::k_merkle_verify_wide<32> : dev::k_merkle_verify_wide<16>)<<<wide, dev::kVerifyWideBlock, 0, st>>>(
-            root, depth, (uint64_t)n_leaves, leaves, indices, (uint64_t)k, paths, ok);
+        PG_CUDA(launch_dependent(lanes == 32 ? dev::k_merkle_verify_wide<32> : dev::k_merkle_verify_wide<16>, wide,
+                                 dev::kVerifyWideBlock, 0, st, root, depth, (uint64_t)n_leaves, leaves, indices, (uint64_t)k,
+                                 paths, ok));
     } else if (g.engine == 1) {
-        dev::k_tc_verify<<<tc_grid(k), dev::kTcThreads, dev::TcL::kBytes, st>>>(root, depth, (uint64_t)n_leaves, leaves,
-                                                                               indices, (uint64_t)k, paths, ok);
+        const bool small = tc_small(tc_units_of(k));
+        PG_CUDA(launch_dependent(small ? dev::k_tc_verify<4> : dev::k_tc_verify<1>, tc_grid(k),
+                                 small ? dev::TcShape<4>::kThreads : dev::TcShape<1>::kThreads,
+                                 small ? dev::TcShape<4>::kBytes : dev::TcShape<1>::kBytes, st, root, depth,
+                                 (uint64_t)n_leaves, leaves, indices, (uint64_t)k, paths, ok));
     } else if (g.params_set == 1)
         dev::k_merkle_verify<dev::kMdsSmall><<<grid, dev::kVerifyBlock, 0, as_stream(stream)>>>(root, depth, (uint64_t)n_leaves,
                                                                                              leaves, indices, (uint64_t)k, paths, ok);

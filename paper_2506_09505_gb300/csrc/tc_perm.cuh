@@ -37,7 +37,7 @@
 namespace pg12 {
 namespace dev {
 
-constexpr int kTcGroup = 128;                   // states (threads) per group
+constexpr int kTcGroup = 128;                   // states per group
 constexpr int kTcAChunk = 128;                  // bytes of one 8 x 8 fp16 core matrix
 constexpr int kTcAChunks = kTcK / 8;            // core-matrix columns of A (12 input words)
 constexpr int kTcABytes = kTcGroup * kTcK * 2;  // A operand of a group: 24 KiB
@@ -59,22 +59,39 @@ static_assert(kTabVpa % 128 == 0 && kTabVpb % 128 == 0 && kTabBs % 128 == 0 && k
 __device__ __align__(16) TcDev g_tc;        // uploaded with the other constant tables
 __constant__ uint64_t c_beta[kRP][kRP];     // the chain's coefficients beta~ times R
 
-// One group's share of the CTA's shared memory and tensor memory.
+// One group's share of the CTA's shared memory and tensor memory.  A state is
+// held by TPS threads: 1 where many groups are in flight (the fewest
+// instructions), 4 where a launch leaves SMs with one group or two and the
+// latency of a permutation counts (each thread then does a quarter of the
+// S-boxes and combinations of a round; the chain stays in one thread per state).
+template <int TPS>
 struct TcGroup {
+    static constexpr int kThreads = kTcGroup * TPS;
+    static constexpr int kWords = kT / TPS;  // words of a state held by one thread
     uint8_t *a;           // A operand, kTcABytes
     uint64_t *mbar;       // tensor-core completion barrier
     uint32_t tmem;        // the group's kTcRegion columns, lanes 0..127
     uint32_t phase;       // parity of the mbarrier's next completion
-    int bar;              // named barrier of the group's 128 threads
+    int bar;              // named barrier of the group's threads
     int t;                // thread index within the group
     uint32_t failed;      // this thread saw a tensor-core wait run out
     volatile uint32_t *bcast;  // one word through which thread 0 hands the group a value
     uint32_t a_addr, tab;      // shared addresses of A and of the tables
+
+    __device__ __forceinline__ int row() const { return TPS == 1 ? t : t % kTcGroup; }   // its state
+    __device__ __forceinline__ int part() const { return TPS == 1 ? 0 : t / kTcGroup; }  // which of the TPS threads
+    // word i of the thread is word TPS i + part of the state: every part holds the
+    // same number of rate, capacity and digest words
+    __device__ __forceinline__ int word(int i) const { return TPS * i + part(); }
+    // its warp's lanes of the group's tensor memory
+    __device__ __forceinline__ uint32_t lane_base() const { return tmem + ((uint32_t)(row() & ~31) << 16); }
 };
 
-// Row t's chunk j of A (K columns 8j..8j+7) <- the 8 bytes of y as fp16 subnormals.
-__device__ __forceinline__ void tc_put(const TcGroup &G, int j, uint64_t y) {
-    *reinterpret_cast<uint4 *>(G.a + ((G.t >> 3) * kTcAChunks + j) * kTcAChunk + (G.t & 7) * 16) = tc_bytes(y);
+// The row's chunk j of A (K columns 8j..8j+7) <- the 8 bytes of y as fp16 subnormals.
+template <int TPS>
+__device__ __forceinline__ void tc_put(const TcGroup<TPS> &G, int j, uint64_t y) {
+    const int r = G.row();
+    *reinterpret_cast<uint4 *>(G.a + ((r >> 3) * kTcAChunks + j) * kTcAChunk + (r & 7) * 16) = tc_bytes(y);
 }
 
 // One contraction into the group's D (columns 0 .. n-1): the group meets
@@ -84,10 +101,11 @@ __device__ __forceinline__ void tc_put(const TcGroup &G, int j, uint64_t y) {
 // 8..11 from the zero-capacity block when z) against the table at byte offset
 // b_off, and commits; every thread waits.  Returns false, in every thread of
 // the group, once a wait of the group has run out.
-__device__ __forceinline__ bool tc_contract(TcGroup &G, uint32_t b_off, int n, int bias, bool z) {
+template <int TPS>
+__device__ __forceinline__ bool tc_contract(TcGroup<TPS> &G, uint32_t b_off, int n, int bias, bool z) {
     fence_async_smem();   // this thread's A stores -> the tensor cores' proxy
     tc_fence_before();    // its tensor-memory accesses are complete
-    if (group_sync_or(G.bar, G.failed)) return false;
+    if (group_sync_or(G.bar, G.failed, TcGroup<TPS>::kThreads)) return false;
     if (G.t < 32) {
         tc_fence_after();
         const uint32_t idesc = tc_idesc(n);
@@ -121,31 +139,44 @@ __device__ __forceinline__ bool tc_contract(TcGroup &G, uint32_t b_off, int n, i
     return true;
 }
 
-// Rows I .. ROWS-1 of D (two at a time) into x[].
-template <int ROWS, int I = 0>
-__device__ __forceinline__ void tc_load_rows(uint32_t lane_base, uint64_t (&x)[kT]) {
-    // the next pair's load is in flight while a pair is combined
+// f(i, w) for the rows G.word(i) < ROWS of D, i = 0 .. n-1, w their eight column
+// words; the next load is in flight during f.  One thread per state loads pairs
+// of rows.  Row counts that are no multiple of TPS leave the last row to some
+// parts (whole warps).
+template <int TPS, int ROWS, class F>
+__device__ __forceinline__ void tc_rows(const TcGroup<TPS> &G, F &&f) {
+    constexpr int kStep = TPS == 1 ? 2 : 1, kN = (ROWS + TPS - 1) / TPS;
+    const uint32_t base = G.lane_base();
+    auto has = [&](int i) { return ROWS % TPS == 0 || i < ROWS / TPS || G.word(i) < ROWS; };
+    auto load = [&](int i, uint32_t(&w)[16]) {
+        if (TPS == 1) tmem_ld16_start(base + 8 * i, w);
+        else tmem_ld8_start(base + 8 * G.word(i), w);
+    };
     uint32_t w[2][16];
-    tmem_ld16_start(lane_base + 8 * I, w[0]);
+    load(0, w[0]);
 #pragma unroll
-    for (int i = I; i < ROWS; i += 2) {
-        const int k = ((i - I) / 2) & 1;
+    for (int i = 0; i < kN; i += kStep) {
+        const int k = (i / kStep) & 1;
         tmem_ld_wait();
-        if (i + 2 < ROWS) tmem_ld16_start(lane_base + 8 * (i + 2), w[k ^ 1]);
-        x[i] = tc_combine(w[k]);
-        x[i + 1] = tc_combine(w[k] + 8);
+        if (i + kStep < kN && has(i + kStep)) load(i + kStep, w[k ^ 1]);
+        if (has(i)) {
+            f(i, w[k]);
+            if (kStep == 2) f(i + 1, w[k] + 8);
+        }
     }
 }
 
 // Dense layer of round r (table at m_off) on the S-box outputs in A, plus the
-// next constants (the bias of kind r); with `digest` only rows 0..3 of the
+// next constants (the bias of kind r); with `digest` only words 0..3 of the
 // result are formed.  z: round 0 of states whose capacity entered as zero (A
 // holds cells 0..7; cells 8..11 come from the constant zcap block).
-__device__ __forceinline__ bool tc_dense(TcGroup &G, uint32_t m_off, int r, bool z, bool digest, uint64_t (&x)[kT]) {
+template <int TPS>
+__device__ __forceinline__ bool tc_dense(TcGroup<TPS> &G, uint32_t m_off, int r, bool z, bool digest,
+                                         uint64_t (&x)[kT / TPS]) {
     if (!tc_contract(G, m_off, kTcN, kBiasDense + r, z)) return false;
-    const uint32_t lane_base = G.tmem + ((uint32_t)(G.t & ~31) << 16);
-    tc_load_rows<kDigest>(lane_base, x);
-    if (!digest) tc_load_rows<kT, kDigest>(lane_base, x);
+    auto out = [&](int i, const uint32_t *w) { x[i] = tc_combine(w); };
+    if (digest) tc_rows<TPS, kDigest>(G, out);
+    else tc_rows<TPS, kT>(G, out);
     return true;
 }
 
@@ -157,7 +188,9 @@ __device__ __forceinline__ bool tc_dense(TcGroup &G, uint32_t m_off, int r, bool
 // in registers (reading them back from A's bytes in a loop: a 2^22 x 8 tree
 // 5.69 ms against 5.57).
 static_assert(kRP == 2 * kTcSplit, "the halves have the same length");
-__device__ __forceinline__ void chain_half(const TcGroup &G, uint32_t lane_base, uint64_t c, int q0, int u0) {
+template <int TPS>
+__device__ __forceinline__ void chain_half(const TcGroup<TPS> &G, uint64_t c, int q0, int u0) {
+    const uint32_t lane_base = G.lane_base();
     uint64_t s[kTcSplit];
 #pragma unroll
     for (int q = 0;; ++q) {
@@ -181,71 +214,65 @@ __device__ __forceinline__ void chain_half(const TcGroup &G, uint32_t lane_base,
 
 // Rows 0 .. ROWS-1 of D combined into words, stored at tensor-memory columns
 // kTcUStore + 2 i.
-template <int ROWS>
-__device__ __forceinline__ void tc_store_rows(uint32_t lane_base) {
-    uint32_t w[2][16];
-    tmem_ld16_start(lane_base, w[0]);
-#pragma unroll
-    for (int i = 0; i < ROWS; i += 2) {
-        const int k = (i / 2) & 1;
-        tmem_ld_wait();
-        if (i + 2 < ROWS) tmem_ld16_start(lane_base + 8 * (i + 2), w[k ^ 1]);
-        tmem_st_words(lane_base + kTcUStore + 2 * i, tc_combine(w[k]), tc_combine(w[k] + 8));
-    }
+template <int ROWS, int TPS>
+__device__ __forceinline__ void tc_store_rows(const TcGroup<TPS> &G) {
+    const uint32_t base = G.lane_base() + kTcUStore;
+    uint64_t even = 0;
+    tc_rows<TPS, ROWS>(G, [&](int i, const uint32_t *w) {
+        const uint64_t v = tc_combine(w);
+        if (TPS > 1) tmem_st_word(base + 2 * G.word(i), v);
+        else if (i & 1) tmem_st_words(base + 2 * (i - 1), even, v);
+        else even = v;
+    });
     asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 
 // The 22 partial rounds in their unrolled form, after round 3's dense layer
-// (A still holds round 3's S-box bytes y3, x holds x^(0) = P y3, cell 0 with
-// k_0 added); x leaves with round 4's constants added.
-__device__ __forceinline__ bool tc_partial(TcGroup &G, uint64_t (&x)[kT]) {
-    const uint32_t lane_base = G.tmem + ((uint32_t)(G.t & ~31) << 16);
+// (A still holds round 3's S-box bytes y3, x holds x^(0) = P y3, cell 0 as z_0);
+// x leaves with round 4's constants added.  The chain runs in the threads that
+// hold cell 0; the others wait at the next contraction.
+template <int TPS>
+__device__ __forceinline__ bool tc_partial(TcGroup<TPS> &G, uint64_t (&x)[kT / TPS]) {
+    const uint32_t lane_base = G.lane_base();
     // U_0 .. U_9 as words
     if (!tc_contract(G, kTabVpa, kTcUa * 8, kBiasUa, false)) return false;
-    tc_store_rows<kTcUa>(lane_base);
+    tc_store_rows<kTcUa>(G);
     // U_10 .. U_21 as column sums in D (A still holds y3)
     if (!tc_contract(G, kTabVpb, kTcN, kBiasUb, false)) return false;
     // first half: s_0 .. s_10 into A's chunks 0..10
-    chain_half(G, lane_base, x[0], 0, 0);
-    // D += their terms in c_11 .. c_21: the second half's U'_q (q = 10 .. 20) and U_21, as words
+    if (G.part() == 0) chain_half(G, x[0], 0, 0);
+    // D += their terms in z_11 .. z_21: the second half's U'_q (q = 10 .. 20) and U_21, as words
     if (!tc_contract(G, kTabBs, kTcN, -1, false)) return false;
-    tc_store_rows<kT>(lane_base);
+    tc_store_rows<kT>(G);
     // the deferred updates W s, from s_0 .. s_10 now, s_11 .. s_21 after the second half
     if (!tc_contract(G, kTabW1, kTcN, kBiasW, false)) return false;
-    chain_half(G, lane_base, tmem_ld_word(lane_base + kTcUStore), kTcSplit, kTcUa);
+    if (G.part() == 0) chain_half(G, tmem_ld_word(lane_base + kTcUStore), kTcSplit, kTcUa);
     if (!tc_contract(G, kTabW2, kTcN, -1, false)) return false;
     // cell 0 = c_22 = U_21 + (W s)_0, cell i = x_i^(0) + (W s)_i
     const uint64_t u21 = tmem_ld_word(lane_base + kTcUStore + 2 * (kRP - 1 - kTcUa));
-    uint32_t w[2][16];
-    tmem_ld16_start(lane_base, w[0]);
-#pragma unroll
-    for (int i = 0; i < kT; i += 2) {
-        const int k = (i / 2) & 1;
-        tmem_ld_wait();
-        if (i + 2 < kT) tmem_ld16_start(lane_base + 8 * (i + 2), w[k ^ 1]);
-        x[i] = tc_combine(w[k], i == 0 ? u21 : x[i]);
-        x[i + 1] = tc_combine(w[k] + 8, x[i + 1]);
-    }
+    if (G.part() == 0) x[0] = u21;
+    tc_rows<TPS, kT>(G, [&](int i, const uint32_t *w) { x[i] = tc_combine(w, x[i]); });
     return true;
 }
 
-// The permutation on x, the thread's state in registers (weak words in, weak
-// words out).  zcap: cells 8..11 enter as zero (their round 0 S-box outputs
-// are constants, read from a_zcap); digest: only cells 0..3 of the result are
-// read and formed.  Each round's twelve S-boxes and twelve output rows are
+// The permutation on x, the thread's words of a state in registers (weak words
+// in, weak words out).  zcap: cells 8..11 enter as zero (their round 0 S-box
+// outputs are constants, read from a_zcap); digest: only cells 0..3 of the
+// result are read and formed.  Each round's S-boxes and output rows are
 // unrolled (the state never leaves registers).  Round 0's constants are added
 // here, all later ones by the contractions' biases.
-__device__ __forceinline__ bool tc_permute(TcGroup &G, uint64_t (&x)[kT], bool zcap, bool digest) {
+template <int TPS>
+__device__ __forceinline__ bool tc_permute(TcGroup<TPS> &G, uint64_t (&x)[kT / TPS], bool zcap, bool digest) {
 #pragma unroll
-    for (int j = 0; j < kT; ++j) x[j] = add_canon(x[j], c_dev.full_rc[0][j]);
+    for (int i = 0; i < kT / TPS; ++i) x[i] = add_canon(x[i], c_dev.full_rc[0][G.word(i)]);
 #pragma unroll 1
     for (int r = 0; r < kRF; ++r) {
         const bool z = zcap && r == 0;
 #pragma unroll
-        for (int j = 0; j < kRate; ++j) tc_put(G, j, msbox(x[j]));
+        for (int i = 0; i < kRate / TPS; ++i) tc_put(G, G.word(i), msbox(x[i]));
         if (!z) {
 #pragma unroll
-            for (int j = kRate; j < kT; ++j) tc_put(G, j, msbox(x[j]));
+            for (int i = kRate / TPS; i < kT / TPS; ++i) tc_put(G, G.word(i), msbox(x[i]));
         }
         const bool mid = r == kRF / 2 - 1;
         if (!tc_dense(G, mid ? kTabPre : kTabM, r, z, digest && r == kRF - 1, x)) return false;
@@ -263,28 +290,34 @@ struct TcLayout {
     static constexpr size_t kTables = 0;
     static constexpr size_t kA = (sizeof(TcDev) + 127) & ~(size_t)127;
     static constexpr size_t kBar = kA + (size_t)GROUPS * kTcABytes;
-    static constexpr size_t kBcast = kBar + 8 * GROUPS + 16;
+    static constexpr size_t kTabBar = kBar + 8 * GROUPS;
+    static constexpr size_t kTmemSlot = kTabBar + 8;
+    static constexpr size_t kBcast = kTmemSlot + 8;
     static constexpr size_t kBytes = kBcast + 4 * GROUPS;
     static_assert(kBytes <= 232448, "a block has at most 227 KB of shared memory");
 };
 
 __device__ int g_tc_fault;  // set when a tensor-core wait ran out (read by pg_device_faults)
 
-// Prologue of a tensor-core kernel: tables into shared memory, the groups'
-// barriers, one tensor-memory allocation for all groups.
-template <int GROUPS>
-__device__ __forceinline__ TcGroup tc_setup(uint8_t *sm) {
+// Prologue of a tensor-core kernel: the copy of the tables into shared memory
+// started (one bulk copy; with 131 KB of 16-byte loads through registers a launch
+// of one unit took 28.7 us instead of 21.6), the groups' barriers, one
+// tensor-memory allocation for all groups.  tc_tables_ready follows.
+template <int TPS, int GROUPS>
+__device__ __forceinline__ TcGroup<TPS> tc_setup(uint8_t *sm) {
     using L = TcLayout<GROUPS>;
-    const uint4 *src = reinterpret_cast<const uint4 *>(&g_tc);
-    uint4 *dst = reinterpret_cast<uint4 *>(sm + L::kTables);
-    for (unsigned i = threadIdx.x; i < sizeof(TcDev) / 16; i += blockDim.x) dst[i] = __ldg(src + i);
     uint64_t *bars = reinterpret_cast<uint64_t *>(sm + L::kBar);
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(bars + GROUPS);
+    uint64_t *tab_bar = reinterpret_cast<uint64_t *>(sm + L::kTabBar);
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(sm + L::kTmemSlot);
     if (threadIdx.x == 0) {
-        for (int g = 0; g < GROUPS; ++g) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(bars + g)));
+        for (int g = 0; g <= GROUPS; ++g)  // the groups' barriers, then the tables'
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(bars + g)));
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        fence_async_smem();
+        bulk_copy(sm + L::kTables, &g_tc, sizeof(TcDev), tab_bar);
     }
     if (threadIdx.x < 32) {
+        __syncwarp();
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(tslot)),
                      "r"(L::kTmemCols));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
@@ -293,9 +326,9 @@ __device__ __forceinline__ TcGroup tc_setup(uint8_t *sm) {
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const int g = threadIdx.x / kTcGroup;
-    TcGroup G;
-    G.t = threadIdx.x % kTcGroup;
+    const int g = threadIdx.x / TcGroup<TPS>::kThreads;
+    TcGroup<TPS> G;
+    G.t = threadIdx.x % TcGroup<TPS>::kThreads;
     G.failed = 0;
     G.a = sm + L::kA + (size_t)g * kTcABytes;
     G.mbar = bars + g;
@@ -308,22 +341,30 @@ __device__ __forceinline__ TcGroup tc_setup(uint8_t *sm) {
     return G;
 }
 
+// The warps that issue the contractions wait for the tables (bounded); every
+// kernel calls this once, after whatever else it has to wait for.
+template <int TPS, int GROUPS>
+__device__ __forceinline__ void tc_tables_ready(uint8_t *sm, TcGroup<TPS> &G) {
+    if (G.t < 32 && !mbar_wait(reinterpret_cast<uint64_t *>(sm + TcLayout<GROUPS>::kTabBar), 0)) G.failed = 1;
+}
+
 // Thread 0 adds one to *counter; every thread of the group gets the old
 // value.  The first barrier orders the group's earlier stores (each thread
 // fences its own first) before the atomic and keeps thread 0 from
 // overwriting a value others have not read yet.
-__device__ __forceinline__ uint32_t group_fetch_add(TcGroup &G, uint32_t *counter) {
-    group_sync(G.bar);
+template <int TPS>
+__device__ __forceinline__ uint32_t group_fetch_add(TcGroup<TPS> &G, uint32_t *counter) {
+    group_sync(G.bar, TcGroup<TPS>::kThreads);
     if (G.t == 0) *G.bcast = atomicAdd(counter, 1u);
-    group_sync(G.bar);
+    group_sync(G.bar, TcGroup<TPS>::kThreads);
     return *G.bcast;
 }
 
 // Epilogue: every group is done with tensor memory; the allocating warp
 // frees it.  A group whose wait ran out records the fault and gives its
 // last contraction one more bounded wait before the memory is freed.
-template <int GROUPS>
-__device__ __forceinline__ void tc_teardown(uint8_t *sm, TcGroup &G) {
+template <int TPS, int GROUPS>
+__device__ __forceinline__ void tc_teardown(uint8_t *sm, TcGroup<TPS> &G) {
     using L = TcLayout<GROUPS>;
     if (G.failed) {
         atomicExch(&g_tc_fault, 1);
@@ -333,7 +374,7 @@ __device__ __forceinline__ void tc_teardown(uint8_t *sm, TcGroup &G) {
     __syncthreads();
     if (threadIdx.x < 32) {
         tc_fence_after();
-        const uint32_t base = *reinterpret_cast<uint32_t *>(sm + L::kBar + 8 * GROUPS);
+        const uint32_t base = *reinterpret_cast<uint32_t *>(sm + L::kTmemSlot);
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(base), "r"(L::kTmemCols));
     }
 }
