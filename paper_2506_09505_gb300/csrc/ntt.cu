@@ -326,8 +326,8 @@ __host__ __device__ __forceinline__ uint32_t step_log_radix(uint32_t t, uint32_t
 
 // One step of radix 2^R over the rows x[m s0] (m < 2^R) with tau^j at
 // w[(j - 1) << b] (triv: tau = 1).
-template <int DIT, int R>
-__device__ __forceinline__ void step(uint64_t *x, uint32_t s0, const uint64_t *w, uint32_t b, bool inv, bool triv) {
+template <int DIT, int INV, int R>
+__device__ __forceinline__ void step(uint64_t *x, uint32_t s0, const uint64_t *w, uint32_t b, bool triv) {
     if constexpr (R == 1) {
         const uint64_t a0 = x[0], a1 = x[s0];
         if (DIT) {
@@ -343,6 +343,7 @@ __device__ __forceinline__ void step(uint64_t *x, uint32_t s0, const uint64_t *w
         constexpr int N = 1 << R;
         // position m takes tau^bitrev(m): radix 8 {-, 4, 2, 6, 1, 5, 3, 7}, radix 4 {-, 2, 1, 3}
         constexpr int kE[8] = {0, R == 3 ? 4 : 2, R == 3 ? 2 : 1, R == 3 ? 6 : 3, 1, 5, 3, 7};
+        static_assert(!(DIT && INV), "inverse transforms run DIF passes");
         uint64_t a[N];
         if (DIT) {
 #pragma unroll
@@ -353,23 +354,11 @@ __device__ __forceinline__ void step(uint64_t *x, uint32_t s0, const uint64_t *w
             }
             if constexpr (R == 3) dft8_dit(a);
             else dft4_dit(a);
-            x[0] = a[0];
-            if (inv) {
 #pragma unroll
-                for (int m = 1; m < N; ++m) x[(N - m) * s0] = a[m];
-            } else {
-#pragma unroll
-                for (int m = 1; m < N; ++m) x[m * s0] = a[m];
-            }
+            for (int m = 0; m < N; ++m) x[m * s0] = a[m];
         } else {
-            a[0] = x[0];
-            if (inv) {
 #pragma unroll
-                for (int m = 1; m < N; ++m) a[m] = x[(N - m) * s0];
-            } else {
-#pragma unroll
-                for (int m = 1; m < N; ++m) a[m] = x[m * s0];
-            }
+            for (int m = 0; m < N; ++m) a[m] = x[(INV ? (N - m) & (N - 1) : m) * s0];
             if constexpr (R == 3) dft8_dif(a);
             else dft4_dif(a);
             if (!triv) {
@@ -392,7 +381,7 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 // run in memory.  Columns past ncols are zero and not stored.  Each low value
 // l has its own table of root powers (2^t - 1 of them, rows padded by one
 // word so that different l fall in different banks).
-template <int DIT, int LOG_C, int NT>
+template <int DIT, int INV, int LOG_C, int NT>
 __global__ void __launch_bounds__(NT) k_ntt_pass(const Pass ps) {
     constexpr uint32_t C = 1u << LOG_C;
     extern __shared__ uint64_t sm[];
@@ -412,8 +401,7 @@ __global__ void __launch_bounds__(NT) k_ntt_pass(const Pass ps) {
     const uint64_t low0 = (outer & ((1ull << (ps.lo - u)) - 1)) << u;
     const uint64_t high = outer >> (ps.lo - u);
     const uint64_t base = (high << (ps.lo + t)) | low0;
-    const uint32_t dir = ps.inverse ? 1u : 0u;
-    const bool inv = ps.inverse != 0;
+    constexpr uint32_t dir = INV;
 
     // the steps: log radix (2 bits each) and lowest bit (4 bits each)
     uint32_t plan_r = 0, plan_b = 0, nsteps = 0;
@@ -507,9 +495,9 @@ __global__ void __launch_bounds__(NT) k_ntt_pass(const Pass ps) {
             const uint32_t v0 = ((g >> b) << (b + r)) | k;
             uint64_t *x = tile + ((v0 << sh) + lc);
             const uint64_t *w = tw + (lc >> LOG_C) * tws + nb - 1 + k;
-            if (r == 3) step<DIT, 3>(x, s0, w, b, inv, triv);
-            else if (r == 2) step<DIT, 2>(x, s0, w, b, inv, triv);
-            else step<DIT, 1>(x, s0, w, b, inv, triv);
+            if (r == 3) step<DIT, INV, 3>(x, s0, w, b, triv);
+            else if (r == 2) step<DIT, INV, 2>(x, s0, w, b, triv);
+            else step<DIT, INV, 1>(x, s0, w, b, triv);
         }
         __syncthreads();
     }
@@ -597,9 +585,12 @@ uint32_t tile_u(uint32_t lo, uint32_t t, const PassShape &sh, uint32_t log_c) {
 bool g_attr_set[64];
 
 using PassKernel = void (*)(const Pass);
+// by log2 columns + 4 x {DIF, inverse DIF, DIT}
 template <int NT>
-constexpr PassKernel kPass[8] = {k_ntt_pass<0, 0, NT>, k_ntt_pass<0, 1, NT>, k_ntt_pass<0, 2, NT>, k_ntt_pass<0, 3, NT>,
-                                 k_ntt_pass<1, 0, NT>, k_ntt_pass<1, 1, NT>, k_ntt_pass<1, 2, NT>, k_ntt_pass<1, 3, NT>};
+constexpr PassKernel kPass[12] = {
+    k_ntt_pass<0, 0, 0, NT>, k_ntt_pass<0, 0, 1, NT>, k_ntt_pass<0, 0, 2, NT>, k_ntt_pass<0, 0, 3, NT>,
+    k_ntt_pass<0, 1, 0, NT>, k_ntt_pass<0, 1, 1, NT>, k_ntt_pass<0, 1, 2, NT>, k_ntt_pass<0, 1, 3, NT>,
+    k_ntt_pass<1, 0, 0, NT>, k_ntt_pass<1, 0, 1, NT>, k_ntt_pass<1, 0, 2, NT>, k_ntt_pass<1, 0, 3, NT>};
 // more than any pass of plan_shape needs (the largest: 2^10 rows x 8 columns with row factors, 80 KB)
 constexpr int kPassSmemMax = 112 << 10;
 
@@ -635,8 +626,8 @@ int launch_pass(Pass ps, const PassShape &sh, cudaStream_t st) {
     int device = 0;
     cudaGetDevice(&device);
     if (device >= 0 && device < 64 && !g_attr_set[device]) {
-        for (int k = 0; k < 16; ++k) {
-            const PassKernel f = k < 8 ? kPass<128>[k] : kPass<256>[k - 8];
+        for (int k = 0; k < 24; ++k) {
+            const PassKernel f = k < 12 ? kPass<128>[k] : kPass<256>[k - 12];
             const cudaError_t e =
                 cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kPassSmemMax);
             if (e != cudaSuccess) return set_error(PG_ERR_CUDA, "NTT shared-memory attribute: %s", cudaGetErrorString(e));
@@ -644,7 +635,7 @@ int launch_pass(Pass ps, const PassShape &sh, cudaStream_t st) {
         g_attr_set[device] = true;
     }
     ProfScope prof(kIdNttPass, st, 0);
-    const PassKernel f = (sh.threads == 128 ? kPass<128> : kPass<256>)[lc + (ps.dit ? 4u : 0u)];
+    const PassKernel f = (sh.threads == 128 ? kPass<128> : kPass<256>)[lc + (ps.dit ? 8u : ps.inverse ? 4u : 0u)];
     const cudaError_t e = launch_dependent(f, (unsigned)blocks, sh.threads, smem, st, ps);
     if (e != cudaSuccess) return set_error(PG_ERR_CUDA, "k_ntt_pass: %s", cudaGetErrorString(e));
     return PG_OK;
@@ -715,6 +706,9 @@ uint64_t host_pow(uint64_t a, uint64_t e) {
     return r;
 }
 
+// 2^-k R mod p for k <= 32: 2^k (p - (p - 1) / 2^k) = 1 (mod p)
+uint64_t inverse_of_pow2(uint32_t k) { return host::fp_mul(kP - ((kP - 1) >> k), kEps); }
+
 bool is_pow2(uint64_t x) { return x && !(x & (x - 1)); }
 uint32_t log2u(uint64_t x) {
     uint32_t k = 0;
@@ -765,7 +759,7 @@ pg_status pg_ntt(uint64_t *data, size_t n, size_t ncols, int inverse, void *stre
     if (s != PG_OK) return (pg_status)s;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const uint32_t log_n = log2u(n);
-    const uint64_t ninv = pg12::host::fp_mul(pg12::host::fp_inv((uint64_t)n), pg12::kEps);
+    const uint64_t ninv = inverse_of_pow2(log_n);
     s = run_dif(data, data, log_n, ncols, inverse != 0, inverse ? 1u : 0u, ninv, st);
     if (s != PG_OK) return (pg_status)s;
     if (log_n > 0) {
@@ -804,7 +798,7 @@ pg_status pg_lde(const uint64_t *evals, size_t n, size_t ncols, uint32_t log_blo
     if (s != PG_OK) return (pg_status)s;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     // coefficients c_j 7^j in bit-reversed order into scratch
-    s = run_dif(evals, scratch, log_n, ncols, true, 2u, pg12::host::fp_mul(pg12::host::fp_inv((uint64_t)n), pg12::kEps), st);
+    s = run_dif(evals, scratch, log_n, ncols, true, 2u, inverse_of_pow2(log_n), st);
     if (s != PG_OK) return (pg_status)s;
     // DIT passes over bits [b, log N) of out; the first reads coefficient row i >> b
     const uint32_t log_big = log_n + log_blowup;
