@@ -1056,7 +1056,6 @@ struct Context {
     bool params_ready = false;
     int params_set = 0;  // 0 = pg12_v1, 1 = pg12_small
     int params_gen = 1;  // bumped whenever the active set changes
-    int tables_device = -1, tables_gen = 0;  // where upload_tables() last put the tables of which generation
     uint32_t small_row[kT] = {};
     PlainParams plain;
     OptParams opt;
@@ -1207,44 +1206,29 @@ pg_status ensure_params() {
     return PG_OK;
 }
 
-// The kernels' tables of each built-in set, built once (under g_mu).
-struct SetTables {
-    bool ready = false;
-    dev::DevConsts dc;
-    WideConsts wc;
-    TcDev td;
-    uint64_t beta[kRP][kRP];
-};
-SetTables g_tables[2];
-
 // Constant tables of the active parameter set onto the current device: the
 // permutation constants of both permutation forms and the digit tables of
-// the tensor-core contractions.  Nothing to do while the device holds them.
+// the tensor-core dense layers.
 pg_status upload_tables() {
-    int device = 0;
-    PG_CUDA(cudaGetDevice(&device));
-    if (g.tables_device == device && g.tables_gen == g.params_gen) return PG_OK;
-    SetTables &t = g_tables[g.params_set];
-    if (!t.ready) {
-        const char *set = g.params_set == 1 ? "pg12_small" : "pg12_v1";
-        static KernelParams kp;
-        dev::make_dev_consts(g.opt, t.dc);
-        if (!host::derive_kernel(g.opt, kp))
-            return fail(PG_ERR_PARAMS, "parameter set %s: a partial round's coefficient is zero", set);
-        host::build_wide(kp, t.wc);
-        if (!host::build_tc_dev(g.opt, kp, t.td))
-            return fail(PG_ERR_PARAMS, "parameter set %s: a tensor-core sum could leave the exact fp32 window", set);
-        for (int q = 0; q < kRP; ++q)
-            for (int r = 0; r < kRP; ++r) t.beta[q][r] = host::fp_mul(kp.beta[q][r], kEps);
-        t.ready = true;
-    }
-    g.tables_device = -1;
-    PG_CUDA(cudaMemcpyToSymbol(dev::c_dev, &t.dc, sizeof(t.dc)));
-    PG_CUDA(cudaMemcpyToSymbol(dev::g_wide, &t.wc, sizeof(t.wc)));
-    PG_CUDA(cudaMemcpyToSymbol(dev::g_tc, &t.td, sizeof(t.td)));
-    PG_CUDA(cudaMemcpyToSymbol(dev::c_beta, t.beta, sizeof(t.beta)));
-    g.tables_device = device;
-    g.tables_gen = g.params_gen;
+    dev::DevConsts dc;
+    dev::make_dev_consts(g.opt, dc);
+    PG_CUDA(cudaMemcpyToSymbol(dev::c_dev, &dc, sizeof(dc)));
+    static KernelParams kp;  // this and the tables below: built under g_mu
+    static WideConsts wc;
+    static TcDev td;         // 131 KB
+    if (!host::derive_kernel(g.opt, kp))
+        return fail(PG_ERR_PARAMS, "parameter set %s: a partial round's coefficient is zero",
+                    g.params_set == 1 ? "pg12_small" : "pg12_v1");
+    host::build_wide(kp, wc);
+    PG_CUDA(cudaMemcpyToSymbol(dev::g_wide, &wc, sizeof(wc)));
+    if (!host::build_tc_dev(g.opt, kp, td))
+        return fail(PG_ERR_PARAMS, "parameter set %s: a tensor-core sum could leave the exact fp32 window",
+                    g.params_set == 1 ? "pg12_small" : "pg12_v1");
+    PG_CUDA(cudaMemcpyToSymbol(dev::g_tc, &td, sizeof(td)));
+    uint64_t beta[kRP][kRP];
+    for (int q = 0; q < kRP; ++q)
+        for (int r = 0; r < kRP; ++r) beta[q][r] = host::fp_mul(kp.beta[q][r], kEps);
+    PG_CUDA(cudaMemcpyToSymbol(dev::c_beta, beta, sizeof(beta)));
     return PG_OK;
 }
 
@@ -2084,7 +2068,6 @@ pg_status pg_shutdown(void) {
     g.ready_vals = nullptr;
     if (g.ready_ev) cudaEventDestroy(g.ready_ev);
     g.ready_ev = nullptr;
-    g.tables_device = -1;
     g.init = false;
     g.device = -1;
     return PG_OK;
