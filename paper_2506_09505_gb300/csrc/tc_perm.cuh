@@ -188,15 +188,15 @@ __device__ __forceinline__ bool tc_dense(TcGroup<TPS> &G, uint32_t m_off, int r,
 // in registers (reading them back from A's bytes in a loop: a 2^22 x 8 tree
 // 5.69 ms against 5.57).
 static_assert(kRP == 2 * kTcSplit, "the halves have the same length");
+// u: the words U_(q0) .. as pairs, u[2 k] and u[2 k + 1] from column kTcUStore + 2 k.
 template <int TPS>
-__device__ __forceinline__ void chain_half(const TcGroup<TPS> &G, uint64_t c, int q0, int u0) {
-    const uint32_t lane_base = G.lane_base();
+__device__ __forceinline__ void chain_half(const TcGroup<TPS> &G, uint64_t c, int q0, const uint32_t *u) {
     uint64_t s[kTcSplit];
 #pragma unroll
     for (int q = 0;; ++q) {
         uint64_t t = 0;
         if (q < kTcSplit - 1) {
-            t = tmem_ld_word(lane_base + kTcUStore + 2 * (q + q0 - u0));
+            t = ((uint64_t)u[2 * q + 1] << 32) | u[2 * q];
             if (q > 0) {
                 MAcc A;
                 macc_init(A, t);
@@ -210,6 +210,17 @@ __device__ __forceinline__ void chain_half(const TcGroup<TPS> &G, uint64_t c, in
         if (q == kTcSplit - 1) break;
         c = add_fold(t, s[q]);
     }
+}
+// The stored words 0 .. 11 of the thread's state as 24 columns.
+__device__ __forceinline__ void tc_load_words(uint32_t base, uint32_t (&u)[32]) {
+    uint32_t a[16], b[16];
+    tmem_ld16_start(base, a);
+    tmem_ld8_start(base + 16, b);
+    tmem_ld_wait();
+#pragma unroll
+    for (int i = 0; i < 16; ++i) u[i] = a[i];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) u[16 + i] = b[i];
 }
 
 // Rows 0 .. ROWS-1 of D combined into words, stored at tensor-memory columns
@@ -240,13 +251,21 @@ __device__ __forceinline__ bool tc_partial(TcGroup<TPS> &G, uint64_t (&x)[kT / T
     // U_10 .. U_21 as column sums in D (A still holds y3)
     if (!tc_contract(G, kTabVpb, kTcN, kBiasUb, false)) return false;
     // first half: s_0 .. s_10 into A's chunks 0..10
-    if (G.part() == 0) chain_half(G, x[0], 0, 0);
+    if (G.part() == 0) {
+        uint32_t u[32];
+        tc_load_words(lane_base + kTcUStore, u);
+        chain_half(G, x[0], 0, u);
+    }
     // D += their terms in z_11 .. z_21: the second half's U'_q (q = 10 .. 20) and U_21, as words
     if (!tc_contract(G, kTabBs, kTcN, -1, false)) return false;
     tc_store_rows<kT>(G);
     // the deferred updates W s, from s_0 .. s_10 now, s_11 .. s_21 after the second half
     if (!tc_contract(G, kTabW1, kTcN, kBiasW, false)) return false;
-    if (G.part() == 0) chain_half(G, tmem_ld_word(lane_base + kTcUStore), kTcSplit, kTcUa);
+    if (G.part() == 0) {
+        uint32_t u[32];
+        tc_load_words(lane_base + kTcUStore, u);
+        chain_half(G, ((uint64_t)u[1] << 32) | u[0], kTcSplit, u + 2);
+    }
     if (!tc_contract(G, kTabW2, kTcN, -1, false)) return false;
     // cell 0 = c_22 = U_21 + (W s)_0, cell i = x_i^(0) + (W s)_i
     const uint64_t u21 = tmem_ld_word(lane_base + kTcUStore + 2 * (kRP - 1 - kTcUa));
