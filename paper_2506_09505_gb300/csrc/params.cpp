@@ -358,7 +358,7 @@ void digit_table(const uint64_t *mat, int n, int k, uint16_t *dst, long *pos, lo
         for (int j = 0; j < k; ++j)
             for (int a = 0; a < 8; ++a) {
                 int d[8];
-                balanced_digits(fp_mul(mat[i * k + j] % kP, fp_pow(2, 8 * (uint64_t)a)), d);
+                balanced_digits(fp_mul(mat[i * k + j] % kP, 1ull << (8 * a)), d);
                 for (int b = 0; b < 8; ++b) {
                     const int row = 8 * i + b;
                     dst[(row / 8 * k + j) * 64 + (row % 8) * 8 + a] = half_of_int(d[b]);
@@ -478,12 +478,13 @@ bool derive_kernel(const OptParams &op, KernelParams &kp) {
     derive_chain(op, cp);
     const uint64_t R6 = fp_pow(kEps, 6);
     // lambda_22 = 1; lambda_q^7 R^-6 = kappa_q = lambda_(q+1) beta[q][q]
-    uint64_t lambda[kRP + 1], kappa[kRP];
+    uint64_t lambda[kRP + 1], kappa_inv[kRP];
     lambda[kRP] = 1;
     for (int q = kRP - 1; q >= 0; --q) {
-        kappa[q] = fp_mul(lambda[q + 1], cp.beta[q][q]);
-        if (kappa[q] == 0) return false;
-        lambda[q] = root7(fp_mul(kappa[q], R6));
+        const uint64_t kappa = fp_mul(lambda[q + 1], cp.beta[q][q]);
+        if (kappa == 0) return false;
+        lambda[q] = root7(fp_mul(kappa, R6));
+        kappa_inv[q] = fp_inv(kappa);
     }
     for (int i = 0; i < kT; ++i) {
         kp.rc0[i] = op.full_rc[0][i] % kP;
@@ -494,13 +495,13 @@ bool derive_kernel(const OptParams &op, KernelParams &kp) {
             kp.m[i][j] = fp_mul(op.mds[i][j] % kP, R6);
             kp.pre[i][j] = fp_mul(fp_mul(op.pre[i][j] % kP, R6), i == 0 ? lambda[0] : 1);
         }
-        for (int r = 0; r < kRP; ++r) kp.w[i][r] = fp_mul(cp.w[i][r], fp_inv(kappa[r]));
+        for (int r = 0; r < kRP; ++r) kp.w[i][r] = fp_mul(cp.w[i][r], kappa_inv[r]);
     }
     kp.add[kRF / 2 - 1][0] = fp_mul(op.part_rc[0] % kP, lambda[0]);
     for (int q = 0; q < kRP; ++q) {
         if (q < kRP - 1) kp.u_add[q] = fp_mul(op.part_rc[q + 1] % kP, lambda[q + 1]);
         for (int j = 0; j < kT; ++j) kp.u[q][j] = fp_mul(fp_mul(cp.vp[q][j], R6), lambda[q + 1]);
-        for (int r = 0; r <= q; ++r) kp.beta[q][r] = fp_mul(fp_mul(cp.beta[q][r], lambda[q + 1]), fp_inv(kappa[r]));
+        for (int r = 0; r <= q; ++r) kp.beta[q][r] = fp_mul(fp_mul(cp.beta[q][r], lambda[q + 1]), kappa_inv[r]);
     }
     return true;
 }
@@ -525,10 +526,11 @@ bool build_tc_dev(const OptParams &op, const KernelParams &kp, TcDev &td) {
     const uint64_t G = 0x0101010101010101ull;
     uint64_t off = fp_sub(0x3F + 0x3F3F, fp_mul(1u << 23, G % kP));
     off = fp_add(off, fp_mul(0x3F00 + 0x3F0000, kEps));
+    const uint64_t inv8192 = fp_inv(8192);
     static int u[kBiasKinds][kT][8];
     for (int k = 0; k < kBiasKinds; ++k)
         for (int i = 0; i < kT; ++i) {
-            const uint64_t t = fp_mul(fp_sub(add[k][i], off), fp_inv(8192));
+            const uint64_t t = fp_mul(fp_sub(add[k][i], off), inv8192);
             const uint64_t umin_p = (uint64_t)(((u128)1407 * G) % kP);
             u128 rest = fp_sub(t, umin_p);
             for (int b = 7; b >= 0; --b) {

@@ -1206,29 +1206,39 @@ pg_status ensure_params() {
     return PG_OK;
 }
 
+// The kernels' tables of each built-in set, built once (under g_mu): building
+// them takes longer than their upload, and every pg_init uploads them.
+struct SetTables {
+    bool ready = false;
+    dev::DevConsts dc;
+    WideConsts wc;
+    TcDev td;
+    uint64_t beta[kRP][kRP];
+};
+SetTables g_tables[2];
+
 // Constant tables of the active parameter set onto the current device: the
 // permutation constants of both permutation forms and the digit tables of
-// the tensor-core dense layers.
+// the tensor-core contractions.
 pg_status upload_tables() {
-    dev::DevConsts dc;
-    dev::make_dev_consts(g.opt, dc);
-    PG_CUDA(cudaMemcpyToSymbol(dev::c_dev, &dc, sizeof(dc)));
-    static KernelParams kp;  // this and the tables below: built under g_mu
-    static WideConsts wc;
-    static TcDev td;         // 131 KB
-    if (!host::derive_kernel(g.opt, kp))
-        return fail(PG_ERR_PARAMS, "parameter set %s: a partial round's coefficient is zero",
-                    g.params_set == 1 ? "pg12_small" : "pg12_v1");
-    host::build_wide(kp, wc);
-    PG_CUDA(cudaMemcpyToSymbol(dev::g_wide, &wc, sizeof(wc)));
-    if (!host::build_tc_dev(g.opt, kp, td))
-        return fail(PG_ERR_PARAMS, "parameter set %s: a tensor-core sum could leave the exact fp32 window",
-                    g.params_set == 1 ? "pg12_small" : "pg12_v1");
-    PG_CUDA(cudaMemcpyToSymbol(dev::g_tc, &td, sizeof(td)));
-    uint64_t beta[kRP][kRP];
-    for (int q = 0; q < kRP; ++q)
-        for (int r = 0; r < kRP; ++r) beta[q][r] = host::fp_mul(kp.beta[q][r], kEps);
-    PG_CUDA(cudaMemcpyToSymbol(dev::c_beta, beta, sizeof(beta)));
+    SetTables &t = g_tables[g.params_set];
+    if (!t.ready) {
+        const char *set = g.params_set == 1 ? "pg12_small" : "pg12_v1";
+        static KernelParams kp;
+        dev::make_dev_consts(g.opt, t.dc);
+        if (!host::derive_kernel(g.opt, kp))
+            return fail(PG_ERR_PARAMS, "parameter set %s: a partial round's coefficient is zero", set);
+        host::build_wide(kp, t.wc);
+        if (!host::build_tc_dev(g.opt, kp, t.td))
+            return fail(PG_ERR_PARAMS, "parameter set %s: a tensor-core sum could leave the exact fp32 window", set);
+        for (int q = 0; q < kRP; ++q)
+            for (int r = 0; r < kRP; ++r) t.beta[q][r] = host::fp_mul(kp.beta[q][r], kEps);
+        t.ready = true;
+    }
+    PG_CUDA(cudaMemcpyToSymbol(dev::c_dev, &t.dc, sizeof(t.dc)));
+    PG_CUDA(cudaMemcpyToSymbol(dev::g_wide, &t.wc, sizeof(t.wc)));
+    PG_CUDA(cudaMemcpyToSymbol(dev::g_tc, &t.td, sizeof(t.td)));
+    PG_CUDA(cudaMemcpyToSymbol(dev::c_beta, t.beta, sizeof(t.beta)));
     return PG_OK;
 }
 
