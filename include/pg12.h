@@ -322,7 +322,7 @@ pg_status pg_hash_rows(const uint64_t *rows, size_t n_rows, size_t width, uint64
  *             `stream` and copies the root there.
  * Launches: the leaf sponges in one launch (the tensor-core kernel, or the
  * integer-pipe kernel under PG_ENGINE_INT; trees of at most 8,192 leaves:
- * the 16-lanes-per-state form), then one launch per level of more than 64
+ * the form with 16 or 32 lanes per state), then one launch per level of more than 64
  * nodes and one launch of an 8-block cluster for all levels of at most 64
  * nodes up to the root.  Level launches use programmatic
  * dependent launch: each may be scheduled while the previous one finishes,

@@ -12,7 +12,7 @@
 //               for the leaves only (then one launch per level); batches
 //               climb to every tree's root.
 //   k_merkle_top / k_merkle_top_leaf
-//               the levels with few nodes, 16 lanes per state (latency form).
+//               the levels with few nodes, 16 or 32 lanes per state (latency form).
 //   k_merkle_top_tail
 //               every level of at most 64 nodes up to the root in one launch
 //               of an 8-block cluster, a cluster barrier between levels.
