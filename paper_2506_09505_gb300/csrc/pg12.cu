@@ -1037,9 +1037,9 @@ __global__ void __launch_bounds__(TcShape<TPS>::kThreads, 1) k_tc_verify(const u
 namespace {
 
 // tensor engine: tree levels of at least this many nodes use the tensor-core
-// kernel (one-group CTAs while a level has fewer units than the GPU has
-// groups).  Measured on the 2^22 x 8 tree: 2^15 10.25 ms, 2^13 10.11 ms,
-// 2^12 10.14 ms; below that the 16-lane latency form is faster per level.
+// kernel (four threads per state while a level has at most one unit per SM,
+// tc_small).  Measured on the 2^22 x 8 tree with an earlier version of both
+// forms: 2^15 10.25 ms, 2^13 10.11 ms, 2^12 10.14 ms.
 #ifndef PG12_TC_MIN_NODES
 #define PG12_TC_MIN_NODES (1ull << 13)
 #endif
@@ -1433,8 +1433,8 @@ pg_status launch_tc_sponge(const uint64_t *rows, uint64_t n, uint64_t w, uint64_
     return PG_OK;
 }
 
-// The leaf launch of a streamed host-rows build (k_tc_leaves_stream), in
-// the same CTA shapes as launch_tc_sponge.
+// The leaf launch of a streamed host-rows build (k_tc_leaves_stream), with
+// one thread per state whatever the number of units.
 pg_status launch_leaves_stream(const uint64_t *rows, uint64_t n, uint64_t w, uint64_t *out, const uint32_t *ready,
                                const dev::ChunkMap &cm, cudaStream_t st) {
     const int vec16 = ((w % 2) == 0 && (reinterpret_cast<uintptr_t>(rows) % 16) == 0) ? 1 : 0;
