@@ -620,6 +620,15 @@ __device__ __noinline__ void tc_climb_small(uint8_t *scratch, int bar, int t, ui
     }
 }
 
+// Raises the done flag of a tree whose root this group has stored.  The root's
+// words come from several threads (four warps with four threads per state), and
+// thread 0's fence orders only what it has observed, so the group meets first.
+template <int TPS>
+__device__ __forceinline__ void group_signal_root(const TcGroup<TPS> &G, const TreePlan &tp) {
+    group_sync(G.bar, TcGroup<TPS>::kThreads);
+    if (G.t == 0) signal_root(tp, 0);
+}
+
 template <int TPS>
 __global__ void __launch_bounds__(TcShape<TPS>::kThreads, 1) k_tc_batch(const TreePlan *__restrict__ plans, uint32_t n_trees,
                                                             uint32_t total_tasks, uint32_t fuse,
@@ -651,8 +660,8 @@ __global__ void __launch_bounds__(TcShape<TPS>::kThreads, 1) k_tc_batch(const Tr
         for (uint32_t l = 0;; ++l) {
             for (uint64_t i = 0; i < cnt && ok; ++i) ok = tc_unit(G, tp, l, lo + i);
             if (!ok) break;
-            if (l == log_n) {
-                if (G.t == 0) signal_root(tp, 0);
+            if (l == log_n) {  // a tree of one leaf
+                group_signal_root(G, tp);
                 break;
             }
             if (l == top) break;  // the levels above are built by k_batch_top
@@ -668,7 +677,7 @@ __global__ void __launch_bounds__(TcShape<TPS>::kThreads, 1) k_tc_batch(const Tr
                 // the rest of the tree (the children below are this group's: one unit)
                 group_sync(G.bar, TcGroup<TPS>::kThreads);
                 tc_climb_small<TPS>(G.a, G.bar, G.t, tp.nodes, n, l + 1, log_n);
-                if (G.t == 0) signal_root(tp, 0);
+                group_signal_root(G, tp);
                 break;
             }
             if (tc_units(n, l) >= 2) {
