@@ -518,7 +518,7 @@ __global__ void __launch_bounds__(NT) k_ntt_pass(const Pass ps) {
 }
 
 // Swaps rows i and bitrev(i) (i < bitrev(i)) of a 2^log_n-row array.
-__global__ void k_ntt_bitrev(uint64_t *__restrict__ data, uint32_t log_n, uint64_t ncols) {
+__global__ void k_ntt_bitrev(uint64_t *data, uint32_t log_n, uint64_t ncols) {
     const uint64_t total = (ncols << log_n);
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     pdl_trigger();

@@ -77,11 +77,28 @@ __device__ __forceinline__ uint64_t level_off(uint64_t n, uint32_t level) {
 }
 
 // ------------------------------------------------------------- memory
-__device__ __forceinline__ void ld2_nc(const uint64_t *p, uint64_t &a, uint64_t &b) {
-    asm volatile("ld.global.nc.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p));
+// Callers' words and nodes are read with coherent loads that no compiler moves
+// across a wait.  A dependent launch is resident while the kernel before it still
+// writes them, so ld.global.nc and __ldg (memory nobody writes while the kernel
+// lives) do not apply, nor do the invariant loads that `const __restrict__`
+// permits: kernels launched through launch_dependent declare no data pointer
+// __restrict__.  _cg: through L2 only, for words other blocks of the same launch
+// (or a copy beside it) write.
+__device__ __forceinline__ uint64_t ld1(const uint64_t *p) {
+    uint64_t a;
+    asm volatile("ld.global.u64 %0, [%1];" : "=l"(a) : "l"(p) : "memory");
+    return a;
+}
+__device__ __forceinline__ void ld2(const uint64_t *p, uint64_t &a, uint64_t &b) {
+    asm volatile("ld.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
+}
+__device__ __forceinline__ uint64_t ld1_cg(const uint64_t *p) {
+    uint64_t a;
+    asm volatile("ld.global.cg.u64 %0, [%1];" : "=l"(a) : "l"(p) : "memory");
+    return a;
 }
 __device__ __forceinline__ void ld2_cg(const uint64_t *p, uint64_t &a, uint64_t &b) {
-    asm volatile("ld.global.cg.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p));
+    asm volatile("ld.global.cg.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
 }
 __device__ __forceinline__ void st2(uint64_t *p, uint64_t a, uint64_t b) {
     asm volatile("st.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(a), "l"(b) : "memory");
@@ -94,14 +111,14 @@ __device__ __forceinline__ void load_chunk(const uint64_t *row, uint64_t w, uint
     if (base + kRate <= w) {
         if (vec16) {
 #pragma unroll
-            for (int i = 0; i < kRate; i += 2) ld2_nc(row + base + i, ch[i], ch[i + 1]);
+            for (int i = 0; i < kRate; i += 2) ld2(row + base + i, ch[i], ch[i + 1]);
         } else {
 #pragma unroll
-            for (int i = 0; i < kRate; ++i) ch[i] = __ldg(row + base + i);
+            for (int i = 0; i < kRate; ++i) ch[i] = ld1(row + base + i);
         }
     } else {
 #pragma unroll
-        for (int i = 0; i < kRate; ++i) ch[i] = (base + i < w) ? __ldg(row + base + i) : 0ull;
+        for (int i = 0; i < kRate; ++i) ch[i] = (base + i < w) ? ld1(row + base + i) : 0ull;
     }
 }
 
@@ -114,7 +131,7 @@ __device__ __forceinline__ void load_chunk_cg(const uint64_t *row, uint64_t w, u
         for (int i = 0; i < kRate; i += 2) ld2_cg(row + base + i, ch[i], ch[i + 1]);
     } else {
 #pragma unroll
-        for (int i = 0; i < kRate; ++i) ch[i] = (base + i < w) ? __ldcg(row + base + i) : 0ull;
+        for (int i = 0; i < kRate; ++i) ch[i] = (base + i < w) ? ld1_cg(row + base + i) : 0ull;
     }
 }
 
@@ -137,12 +154,13 @@ __device__ __forceinline__ void sponge_slot(const uint64_t *row, uint64_t w, boo
 // ------------------------------------------------------------- kernels
 constexpr int kSmallBlock = 128;
 
-// Programmatic dependent launch.  The level kernels of a tree are launched
-// with programmatic stream serialisation: each may be scheduled while the
-// kernel before it is still running, once every block of that kernel has
-// executed pdl_trigger().  Until pdl_wait() returns it only copies the
-// constant tables (never written during a build); pdl_wait() returns when
-// the kernel before it has completed and its stores are visible.  For a
+// Programmatic dependent launch.  Tree levels, the tensor-core permutation and
+// sponge, openings, path checks and the transforms' passes (ntt.cu) are launched
+// with programmatic stream serialisation (launch_dependent): each may be
+// scheduled while the kernel before it is still running, once every block of
+// that kernel has executed pdl_trigger().  Until pdl_wait() returns it only
+// copies the constant tables (never written by a kernel); pdl_wait() returns
+// when the kernel before it has completed and its stores are visible.  For a
 // kernel launched without the attribute both are no-ops.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
@@ -158,7 +176,7 @@ __global__ void __launch_bounds__(kSmallBlock) k_permute(uint64_t *__restrict__ 
 #pragma unroll
             for (int i = 0; i < kT; i += 2) {
                 uint64_t a, b;
-                ld2_nc(p + i, a, b);
+                ld2(p + i, a, b);
                 slot[i * kSmallBlock] = a;
                 slot[(i + 1) * kSmallBlock] = b;
             }
@@ -195,8 +213,8 @@ __global__ void __launch_bounds__(kSmallBlock) k_hash_rows(const uint64_t *__res
 // words of children 2k and 2k+1 (contiguous in the level below, 16-byte
 // aligned), i.e. perm([L, R, 0^4])[0..3].
 template <int MDS>
-__global__ void __launch_bounds__(kSmallBlock) k_merkle_level(const uint64_t *__restrict__ below, uint64_t count,
-                                                              uint64_t *__restrict__ here) {
+__global__ void __launch_bounds__(kSmallBlock) k_merkle_level(const uint64_t *below, uint64_t count,
+                                                              uint64_t *here) {
     __shared__ uint64_t slots[kT * kSmallBlock];
     uint64_t *slot = slots + threadIdx.x;
     pdl_trigger();
@@ -250,7 +268,7 @@ __device__ __forceinline__ void load_words(const TcGroup<TPS> &G, const uint64_t
 #pragma unroll
         for (int i = 0; i < kRate / TPS; ++i) {
             const uint64_t k = c * kRate + G.word(i);
-            ch[i] = k < w ? (L2 ? __ldcg(row + k) : __ldg(row + k)) : 0ull;
+            ch[i] = k < w ? (L2 ? ld1_cg(row + k) : ld1(row + k)) : 0ull;
         }
     }
 }
@@ -266,7 +284,7 @@ __device__ __forceinline__ void store_digest(const TcGroup<TPS> &G, uint64_t *ou
 }
 
 template <int TPS>
-__global__ void __launch_bounds__(TcShape<TPS>::kThreads, 1) k_tc_permute(uint64_t *__restrict__ st, uint64_t n, int vec16) {
+__global__ void __launch_bounds__(TcShape<TPS>::kThreads, 1) k_tc_permute(uint64_t *st, uint64_t n, int vec16) {
     extern __shared__ __align__(1024) uint8_t tc_sm[];
     constexpr int kGroups = TcShape<TPS>::kGroups;
     pdl_trigger();
@@ -282,10 +300,10 @@ __global__ void __launch_bounds__(TcShape<TPS>::kThreads, 1) k_tc_permute(uint64
         uint64_t x[kT / TPS];
         if (TPS == 1 && valid && vec16) {
 #pragma unroll
-            for (int i = 0; i < kT / TPS; i += 2) ld2_nc(p + i, x[i], x[i + 1]);
+            for (int i = 0; i < kT / TPS; i += 2) ld2(p + i, x[i], x[i + 1]);
         } else {
 #pragma unroll
-            for (int i = 0; i < kT / TPS; ++i) x[i] = valid ? p[G.word(i)] : 0ull;
+            for (int i = 0; i < kT / TPS; ++i) x[i] = valid ? ld1(p + G.word(i)) : 0ull;
         }
         if (!tc_permute(G, x, false, false)) break;
         if (valid) {
@@ -306,8 +324,8 @@ __global__ void __launch_bounds__(TcShape<TPS>::kThreads, 1) k_tc_permute(uint64
 // pg_hash_rows.  Launched as a dependent launch it may set up while the
 // kernel before it finishes, and reads `rows` only after pdl_wait().
 template <int TPS>
-__global__ void __launch_bounds__(TcShape<TPS>::kThreads, 1) k_tc_sponge(const uint64_t *__restrict__ rows, uint64_t n,
-                                                                         uint64_t w, int vec16, uint64_t *__restrict__ out) {
+__global__ void __launch_bounds__(TcShape<TPS>::kThreads, 1) k_tc_sponge(const uint64_t *rows, uint64_t n,
+                                                                         uint64_t w, int vec16, uint64_t *out) {
     extern __shared__ __align__(1024) uint8_t tc_sm[];
     constexpr int kGroups = TcShape<TPS>::kGroups;
     pdl_trigger();
@@ -364,8 +382,8 @@ __device__ __forceinline__ bool wait_ready(const uint32_t *ready, uint32_t want)
 }
 
 __global__ void __launch_bounds__(TcShape<1>::kThreads, 1)
-    k_tc_leaves_stream(const uint64_t *__restrict__ rows, uint64_t n, uint64_t w, int vec16,
-                       uint64_t *__restrict__ out, const uint32_t *__restrict__ ready, const ChunkMap cm) {
+    k_tc_leaves_stream(const uint64_t *rows, uint64_t n, uint64_t w, int vec16, uint64_t *out,
+                       const uint32_t *ready, const ChunkMap cm) {
     extern __shared__ __align__(1024) uint8_t tc_sm[];
     TcGroup<1> G = tc_setup<1, kTcGroups>(tc_sm);
     tc_tables_ready<1, kTcGroups>(tc_sm, G);
@@ -606,7 +624,7 @@ __device__ __noinline__ void tc_climb_small(uint8_t *scratch, int bar, int t, ui
                 const uint64_t k = valid ? node : 0;
                 uint64_t x = 0;
                 if (l16 < 2 * kDigest) {
-                    if (l == level) asm volatile("ld.global.cg.u64 %0, [%1];" : "=l"(x) : "l"(below + 2 * kDigest * k + l16));
+                    if (l == level) x = ld1_cg(below + 2 * kDigest * k + l16);
                     else x = S.dig[(l - level - 1) & 1][2 * kDigest * k + l16];
                 }
                 x = canon(permute_wide(x, S.buf, g_wide, (unsigned)t));
@@ -715,9 +733,7 @@ __global__ void __launch_bounds__(kBatchTopThreads) k_batch_top(const TreePlan *
             const uint64_t node = valid ? gid : 0;
             const uint64_t *kids = tp.nodes + kDigest * (level_off(n, level - 1) + 2 * node);
             uint64_t x = 0;
-            if (l16 < 2 * kDigest) {
-                asm volatile("ld.global.cg.u64 %0, [%1];" : "=l"(x) : "l"(kids + l16));
-            }
+            if (l16 < 2 * kDigest) x = ld1_cg(kids + l16);
             x = permute_wide(x, buf, K, threadIdx.x);
             if (valid && l16 < kDigest) tp.nodes[kDigest * (level_off(n, level) + node) + l16] = canon(x);
         }
@@ -791,7 +807,7 @@ constexpr int kTailCtas = 8;
 constexpr int kTailBlock = 256;
 constexpr uint64_t kTailNodes = kTailCtas * kTailBlock / 32;
 __global__ void __cluster_dims__(kTailCtas, 1, 1) __launch_bounds__(kTailBlock)
-    k_merkle_top_tail(uint64_t *__restrict__ nodes, uint64_t n, uint32_t first) {
+    k_merkle_top_tail(uint64_t *nodes, uint64_t n, uint32_t first) {
     __shared__ __align__(16) WideConsts K;
     __shared__ __align__(16) WideBuf<32, kTailBlock> buf;
     __shared__ uint64_t dig[2][kTailBlock / 32 * kDigest];  // digests of this block's nodes of a level, in turn
@@ -819,7 +835,7 @@ __global__ void __cluster_dims__(kTailCtas, 1, 1) __launch_bounds__(kTailBlock)
         if (warp < per) {
             uint64_t x = 0;
             if (l16 < 2 * kDigest) {
-                if (level == first) asm volatile("ld.global.cg.u64 %0, [%1];" : "=l"(x) : "l"(below + 2 * kDigest * warp + l16));
+                if (level == first) x = ld1_cg(below + 2 * kDigest * warp + l16);
                 else x = dig[cur ^ 1][2 * kDigest * warp + l16];
             }
             build(level, base + warp, x, &dig[cur][kDigest * warp]);
@@ -849,7 +865,7 @@ __global__ void __cluster_dims__(kTailCtas, 1, 1) __launch_bounds__(kTailBlock)
 }
 
 template <int LANES>
-__global__ void __launch_bounds__(kTopBlock) k_merkle_top(uint64_t *__restrict__ nodes, uint64_t n, uint32_t level) {
+__global__ void __launch_bounds__(kTopBlock) k_merkle_top(uint64_t *nodes, uint64_t n, uint32_t level) {
     __shared__ __align__(16) WideConsts K;
     __shared__ __align__(16) WideBuf<LANES, kTopBlock> buf;
     load_consts(K);
@@ -862,9 +878,7 @@ __global__ void __launch_bounds__(kTopBlock) k_merkle_top(uint64_t *__restrict__
     const uint64_t node = valid ? gid : 0;
     const uint64_t *kids = nodes + kDigest * (level_off(n, level - 1) + 2 * node);
     uint64_t x = 0;
-    if (l16 < 2 * kDigest) {
-        asm volatile("ld.global.cg.u64 %0, [%1];" : "=l"(x) : "l"(kids + l16));
-    }
+    if (l16 < 2 * kDigest) x = ld1_cg(kids + l16);
     x = permute_wide(x, buf, K, threadIdx.x);
     if (valid && (threadIdx.x & (LANES - 1)) < kDigest) nodes[kDigest * (level_off(n, level) + node) + l16] = canon(x);
 }
@@ -872,8 +886,8 @@ __global__ void __launch_bounds__(kTopBlock) k_merkle_top(uint64_t *__restrict__
 // Leaf level of a small tree with the wide permutation: one group per row,
 // lanes 0..7 absorb the chunk words, lanes 8..11 carry the capacity.
 template <int LANES>
-__global__ void __launch_bounds__(kTopBlock) k_merkle_top_leaf(const uint64_t *__restrict__ rows, uint64_t n,
-                                                               uint64_t w, uint64_t *__restrict__ nodes) {
+__global__ void __launch_bounds__(kTopBlock) k_merkle_top_leaf(const uint64_t *rows, uint64_t n,
+                                                               uint64_t w, uint64_t *nodes) {
     __shared__ __align__(16) WideConsts K;
     __shared__ __align__(16) WideBuf<LANES, kTopBlock> buf;
     load_consts(K);
@@ -888,7 +902,7 @@ __global__ void __launch_bounds__(kTopBlock) k_merkle_top_leaf(const uint64_t *_
     for (uint64_t c = 0; c < chunks; ++c) {
         if (l16 < kRate) {
             const uint64_t k = c * kRate + l16;
-            x = k < w ? __ldg(row + k) : 0ull;
+            x = k < w ? ld1(row + k) : 0ull;
         }
         x = permute_wide(x, buf, K, threadIdx.x);
     }
@@ -897,15 +911,15 @@ __global__ void __launch_bounds__(kTopBlock) k_merkle_top_leaf(const uint64_t *_
 
 
 // Authentication paths: thread per (query, level) copies one sibling digest.
-__global__ void k_merkle_open(const uint64_t *__restrict__ nodes, uint64_t n, uint32_t depth,
-                              const uint64_t *__restrict__ idx, uint64_t k, uint64_t *__restrict__ paths) {
+__global__ void k_merkle_open(const uint64_t *nodes, uint64_t n, uint32_t depth, const uint64_t *idx, uint64_t k,
+                              uint64_t *paths) {
     pdl_trigger();
     pdl_wait();
     const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= k * depth) return;
     const uint64_t q = t / depth;
     const uint32_t l = (uint32_t)(t % depth);
-    const uint64_t leaf = idx[q];
+    const uint64_t leaf = ld1(idx + q);
     uint64_t *dst = paths + kDigest * t;
     if (leaf >= n) {
         for (int i = 0; i < kDigest; ++i) dst[i] = ~0ull;
@@ -913,7 +927,11 @@ __global__ void k_merkle_open(const uint64_t *__restrict__ nodes, uint64_t n, ui
     }
     const uint64_t sib = (leaf >> l) ^ 1ull;
     const uint64_t *src = nodes + kDigest * (level_off(n, l) + sib);
-    for (int i = 0; i < kDigest; ++i) dst[i] = src[i];
+    uint64_t d[kDigest];
+#pragma unroll
+    for (int i = 0; i < kDigest; ++i) d[i] = ld1(src + i);
+#pragma unroll
+    for (int i = 0; i < kDigest; ++i) dst[i] = d[i];
 }
 
 // Path verification: one thread per query climbs log2(N) permutations.
@@ -954,11 +972,10 @@ __global__ void __launch_bounds__(kVerifyBlock) k_merkle_verify(const uint64_t *
 // are it and the sibling in the order of the position's bit.
 constexpr int kVerifyWideBlock = 128;
 template <int LANES>
-__global__ void __launch_bounds__(kVerifyWideBlock) k_merkle_verify_wide(const uint64_t *__restrict__ root, uint32_t depth,
-                                                                         uint64_t n, const uint64_t *__restrict__ leaves,
-                                                                         const uint64_t *__restrict__ idx, uint64_t k,
-                                                                         const uint64_t *__restrict__ paths,
-                                                                         uint8_t *__restrict__ ok) {
+__global__ void __launch_bounds__(kVerifyWideBlock) k_merkle_verify_wide(const uint64_t *root, uint32_t depth,
+                                                                         uint64_t n, const uint64_t *leaves,
+                                                                         const uint64_t *idx, uint64_t k,
+                                                                         const uint64_t *paths, uint8_t *ok) {
     __shared__ __align__(16) WideConsts K;
     __shared__ __align__(16) WideBuf<LANES, kVerifyWideBlock> buf;
     pdl_trigger();
@@ -968,20 +985,20 @@ __global__ void __launch_bounds__(kVerifyWideBlock) k_merkle_verify_wide(const u
     const uint64_t gid = ((uint64_t)blockIdx.x * kVerifyWideBlock + threadIdx.x) / LANES;
     const uint64_t q = gid < k ? gid : 0;  // groups past the end repeat query 0 and store nothing
     const int l16 = threadIdx.x & 15, l4 = l16 & 3, base = (threadIdx.x & 31) & ~15;
-    uint64_t cur = leaves[kDigest * q + l4];
-    const uint64_t pos = idx[q];
+    uint64_t cur = ld1(leaves + kDigest * q + l4);
+    const uint64_t pos = ld1(idx + q), want = ld1(root + l4);
     const uint64_t *path = paths + kDigest * q * depth + l4;
-    uint64_t next = depth > 0 ? path[0] : 0;
+    uint64_t next = depth > 0 ? ld1(path) : 0;
     for (uint32_t l = 0; l < depth; ++l) {
         const uint64_t sib = next;
-        if (l + 1 < depth) next = path[kDigest * (l + 1)];  // in flight during the permutation
+        if (l + 1 < depth) next = ld1(path + kDigest * (l + 1));  // in flight during the permutation
         const uint64_t right = (pos >> l) & 1u;
         uint64_t x = (uint64_t)(l16 >> 2) == right ? cur : sib;
         if (l16 >= kRate) x = 0;
         x = canon(permute_wide(x, buf, K, threadIdx.x));
         cur = __shfl_sync(full, x, base + l4);
     }
-    const bool same = cur == root[l4];
+    const bool same = cur == want;
     const unsigned vote = __ballot_sync(full, same) >> base;
     if (gid < k && (threadIdx.x & (LANES - 1)) == 0) ok[q] = (pos < n && (vote & 15u) == 15u) ? 1 : 0;
 }
@@ -989,11 +1006,10 @@ __global__ void __launch_bounds__(kVerifyWideBlock) k_merkle_verify_wide(const u
 // The same with 128 queries per tensor-core group: a unit is 128 queries, and
 // each level is one permutation of the group.
 template <int TPS>
-__global__ void __launch_bounds__(TcShape<TPS>::kThreads, 1) k_tc_verify(const uint64_t *__restrict__ root, uint32_t depth,
-                                                                         uint64_t n, const uint64_t *__restrict__ leaves,
-                                                                         const uint64_t *__restrict__ idx, uint64_t k,
-                                                                         const uint64_t *__restrict__ paths,
-                                                                         uint8_t *__restrict__ ok) {
+__global__ void __launch_bounds__(TcShape<TPS>::kThreads, 1) k_tc_verify(const uint64_t *root, uint32_t depth,
+                                                                         uint64_t n, const uint64_t *leaves,
+                                                                         const uint64_t *idx, uint64_t k,
+                                                                         const uint64_t *paths, uint8_t *ok) {
     extern __shared__ __align__(1024) uint8_t tc_sm[];
     constexpr int kGroups = TcShape<TPS>::kGroups, kOwn = kDigest / TPS, kThreads = TcGroup<TPS>::kThreads;
     pdl_trigger();
@@ -1008,14 +1024,14 @@ __global__ void __launch_bounds__(TcShape<TPS>::kThreads, 1) k_tc_verify(const u
         const uint64_t q = gid < k ? gid : 0;
         uint64_t x[kT / TPS];  // words: left child, right child, zero capacity
 #pragma unroll
-        for (int i = 0; i < kOwn; ++i) x[i] = leaves[kDigest * q + G.word(i)];
-        const uint64_t pos = idx[q];
+        for (int i = 0; i < kOwn; ++i) x[i] = ld1(leaves + kDigest * q + G.word(i));
+        const uint64_t pos = ld1(idx + q);
         for (uint32_t l = 0; l < depth && fine; ++l) {
             const uint64_t *sib = paths + kDigest * (q * depth + l);
             const bool right = (pos >> l) & 1u;
 #pragma unroll
             for (int i = 0; i < kOwn; ++i) {
-                const uint64_t s = sib[G.word(i)], c = x[i];
+                const uint64_t s = ld1(sib + G.word(i)), c = x[i];
                 x[i] = right ? s : c;
                 x[kOwn + i] = right ? c : s;
                 x[2 * kOwn + i] = 0;
@@ -1027,7 +1043,7 @@ __global__ void __launch_bounds__(TcShape<TPS>::kThreads, 1) k_tc_verify(const u
         if (!fine) break;
         bool eq = pos < n;
 #pragma unroll
-        for (int i = 0; i < kOwn; ++i) eq = eq && x[i] == root[G.word(i)];
+        for (int i = 0; i < kOwn; ++i) eq &= x[i] == ld1(root + G.word(i));
         if constexpr (TPS > 1) {  // the parts' answers through the idle A operand
             G.a[G.t] = eq ? 1 : 0;
             group_sync(G.bar, kThreads);

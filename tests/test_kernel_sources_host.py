@@ -39,3 +39,41 @@ def test_batch_kernel_raises_a_done_flag_only_after_its_group_has_met():
     assert "signal_root" not in body(text, "k_tc_batch").replace("group_signal_root", "")
     helper = body(text, "group_signal_root")
     assert 0 <= helper.find("group_sync(") < helper.find("signal_root(")
+
+
+def dependent_kernels():
+    """{kernel: source file} of what is launched through launch_dependent."""
+    found = {}
+    for name in ("pg12.cu", "ntt.cu"):
+        text = source(name)
+        for call in re.findall(r"launch_dependent\(([^;]*);", text):
+            for kernel in re.findall(r"\bk_\w+", call):
+                found[kernel] = name
+        if re.search(r"launch_dependent\(f,", text):
+            found["k_ntt_pass"] = name
+    return found
+
+
+def test_dependent_launches_read_their_input_with_coherent_loads_after_the_wait():
+    # a dependent launch is resident while the kernel before it writes: no load may
+    # promise that nobody writes, and none may be moved above the wait
+    kernels = dependent_kernels()
+    assert {"k_tc_permute", "k_tc_sponge", "k_merkle_level", "k_merkle_top", "k_merkle_top_tail", "k_merkle_open",
+            "k_merkle_verify_wide", "k_tc_verify", "k_ntt_pass", "k_ntt_bitrev"} <= set(kernels)
+    for kernel, name in kernels.items():
+        text = source(name)
+        sig = re.search(r"\b%s\(([^)]*)\)\s*\{" % kernel, text).group(1)
+        assert "__restrict__" not in sig, kernel
+        code = body(text, kernel)
+        wait = code.find("pdl_wait();")
+        assert wait > 0, kernel
+        assert not re.search(r"\b(ld1|ld2|ld1_cg|ld2_cg|load_words|load_chunk)\b", code[:wait]), kernel
+    for name in ("pg12.cu", "ntt.cu", "tc_perm.cuh", "tcgen05.cuh", "poseidon.cuh"):
+        text = source(name)
+        assert "ld.global.nc" not in text and "__ldcg" not in text, name
+        # only the constant tables, which no kernel writes
+        assert "__ldg" not in text.replace(body(text, "load_consts"), "") if name == "poseidon.cuh" else "__ldg" not in text
+    # the loads themselves are ordered against the wait
+    for line in source("pg12.cu").splitlines():
+        if re.search(r"\bld\.global\.(u64|v2|cg)", line):
+            assert "volatile" in line and '"memory"' in line, line
