@@ -812,6 +812,9 @@ __global__ void __cluster_dims__(kTailCtas, 1, 1) __launch_bounds__(kTailBlock)
     __shared__ __align__(16) WideBuf<32, kTailBlock> buf;
     __shared__ uint64_t dig[2][kTailBlock / 32 * kDigest];  // digests of this block's nodes of a level, in turn
     __shared__ uint64_t sub[kTailCtas * kDigest];           // block 0: every block's last node
+    // every block of the cluster has started once the wait before the remote
+    // stores returns: only then may another block's shared memory be written
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     load_consts(K);
     pdl_trigger();
     pdl_wait();
@@ -844,6 +847,7 @@ __global__ void __cluster_dims__(kTailCtas, 1, 1) __launch_bounds__(kTailBlock)
         cur ^= 1;
         base >>= 1;
     }
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     if (count0 < kTailCtas) return;  // block 0 has built the root
     // the blocks' last nodes to block 0
     if (threadIdx.x < kDigest) {

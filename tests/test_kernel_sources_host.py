@@ -77,3 +77,16 @@ def test_dependent_launches_read_their_input_with_coherent_loads_after_the_wait(
     for line in source("pg12.cu").splitlines():
         if re.search(r"\bld\.global\.(u64|v2|cg)", line):
             assert "volatile" in line and '"memory"' in line, line
+
+
+def test_remote_shared_memory_is_written_only_once_its_block_has_started():
+    # blocks of a cluster are scheduled together, but one may not have begun when
+    # another stores into its shared memory: a cluster barrier comes first
+    code = body(source("pg12.cu"), "k_merkle_top_tail")
+    store = code.find("st.shared::cluster")
+    first = code.find("barrier.cluster.wait")
+    assert 0 <= code.find("barrier.cluster.arrive") < first < store
+    # every block of the cluster takes that wait: no return or branch on the block comes before it
+    assert "return" not in code[:first].split("auto build")[0] and "if (blockIdx" not in code[:first]
+    # and a second barrier hands the stores over
+    assert store < code.find("barrier.cluster.arrive", store) < code.find("barrier.cluster.wait", store)
