@@ -380,14 +380,18 @@ __device__ __forceinline__ uint32_t group_fetch_add(TcGroup<TPS> &G, uint32_t *c
 }
 
 // Epilogue: every group is done with tensor memory; the allocating warp
-// frees it.  A group whose wait ran out records the fault and gives its
-// last contraction one more bounded wait before the memory is freed.
+// frees it.  A group whose wait ran out records the fault and gives the table
+// copy and its last contraction one more bounded wait each before the memory is
+// freed: neither may land in shared or tensor memory that is no longer ours.
 template <int TPS, int GROUPS>
 __device__ __forceinline__ void tc_teardown(uint8_t *sm, TcGroup<TPS> &G) {
     using L = TcLayout<GROUPS>;
     if (G.failed) {
         atomicExch(&g_tc_fault, 1);
-        if (G.t == 0) mbar_wait(G.mbar, G.phase ^ 1u);
+        if (G.t == 0) {
+            mbar_wait(reinterpret_cast<uint64_t *>(sm + L::kTabBar), 0);
+            mbar_wait(G.mbar, G.phase ^ 1u);
+        }
     }
     tc_fence_before();
     __syncthreads();

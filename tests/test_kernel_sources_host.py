@@ -90,3 +90,12 @@ def test_remote_shared_memory_is_written_only_once_its_block_has_started():
     assert "return" not in code[:first].split("auto build")[0] and "if (blockIdx" not in code[:first]
     # and a second barrier hands the stores over
     assert store < code.find("barrier.cluster.arrive", store) < code.find("barrier.cluster.wait", store)
+
+
+def test_a_failed_tensor_core_kernel_waits_for_its_copies_before_it_ends():
+    # after a wait has run out: one more bounded wait for the table copy and for the
+    # last contraction, then the block meets and tensor memory is freed
+    code = body(source("tc_perm.cuh"), "tc_teardown")
+    failed = block(code, code.find("if (G.failed)"))
+    assert "mbar_wait(reinterpret_cast<uint64_t *>(sm + L::kTabBar), 0)" in failed and "mbar_wait(G.mbar" in failed
+    assert code.find(failed) < code.find("__syncthreads()") < code.find("tcgen05.dealloc")
