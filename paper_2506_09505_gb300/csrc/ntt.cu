@@ -740,6 +740,7 @@ int ntt_upload_constants() {
     }
     for (int d = 0; d < 3; ++d) powers(host_pow(kShift, 1ull << (10 * d)), 1024, h.coset[d]);
     cudaError_t e = cudaMemcpyToSymbol(g_ntt, &h, sizeof h);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
     if (e != cudaSuccess) return set_error(PG_ERR_CUDA, "NTT constants: %s", cudaGetErrorString(e));
     return PG_OK;
 }

@@ -1248,7 +1248,10 @@ SetTables g_tables[2];
 
 // Constant tables of the active parameter set onto the current device: the
 // permutation constants of both permutation forms and the digit tables of
-// the tensor-core contractions.
+// the tensor-core contractions.  A copy from pageable memory may return before
+// its transfer to the device has happened, and a kernel on a stream that does not
+// wait for the legacy stream could then read the old words: every upload ends by
+// waiting for it.
 pg_status upload_tables() {
     SetTables &t = g_tables[g.params_set];
     if (!t.ready) {
@@ -1268,6 +1271,7 @@ pg_status upload_tables() {
     PG_CUDA(cudaMemcpyToSymbol(dev::g_wide, &t.wc, sizeof(t.wc)));
     PG_CUDA(cudaMemcpyToSymbol(dev::g_tc, &t.td, sizeof(t.td)));
     PG_CUDA(cudaMemcpyToSymbol(dev::c_beta, t.beta, sizeof(t.beta)));
+    PG_CUDA(cudaStreamSynchronize(cudaStreamLegacy));
     return PG_OK;
 }
 
@@ -2713,6 +2717,7 @@ pg_status pg_merkle_build_noalloc(const uint64_t *rows, size_t n_leaves, size_t 
             dev::DevConsts dc;
             dev::make_dev_consts(g.opt, dc);
             PG_CUDA(cudaMemcpyToSymbol(dev::c_dev, &dc, sizeof(dc)));
+            PG_CUDA(cudaStreamSynchronize(cudaStreamLegacy));
             consts_gen[device] = g.params_gen;
             PG_CUDA(cudaDeviceGetAttribute(&sm_count[device], cudaDevAttrMultiProcessorCount, device));
             int oa = 0, ob = 0;

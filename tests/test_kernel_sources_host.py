@@ -99,3 +99,12 @@ def test_a_failed_tensor_core_kernel_waits_for_its_copies_before_it_ends():
     failed = block(code, code.find("if (G.failed)"))
     assert "mbar_wait(reinterpret_cast<uint64_t *>(sm + L::kTabBar), 0)" in failed and "mbar_wait(G.mbar" in failed
     assert code.find(failed) < code.find("__syncthreads()") < code.find("tcgen05.dealloc")
+
+
+def test_table_uploads_end_with_a_wait_for_the_copy():
+    # a copy from pageable memory may return before the device holds the words
+    for name, function in (("pg12.cu", "upload_tables"), ("pg12.cu", "pg_merkle_build_noalloc"),
+                           ("ntt.cu", "ntt_upload_constants")):
+        code = body(source(name), function)
+        last = code.rfind("cudaMemcpyToSymbol")
+        assert 0 <= last < code.find("cudaStreamSynchronize(cudaStreamLegacy)", last) < last + 160, function
