@@ -542,11 +542,17 @@ __global__ void k_ntt_bitrev(uint64_t *data, uint32_t log_n, uint64_t ncols) {
 // would not fill the SMs several times over and a block's serial work counts:
 // 256 threads, on tiles that shrink until there are 2^9 of them (but not below
 // 2^6 rows: more passes then cost more than they spread).  2^16 rows x 3: 16.6 us
-// against 33 with 2^11-row tiles; 2^18 x 8: 44.6 against 51.6.
+// against 33 with 2^11-row tiles; 2^18 x 8: 44.6 against 51.6.  A transform whose
+// rows (times the tile's columns) are at most 2^11 words stays one pass: a
+// second launch costs more than one block's work.  2^8 rows x 3, calls back to
+// back: 9.1 us in one pass, 11.4 in two; extension of 2^8 x 3, blowup 1: 10.9
+// against 14.4 (2^11 words: 2^9 x 3 9.2 against 11.0; 2^12: 2^10 x 3 extended 17.9
+// in one pass, 15.1 in two).
 struct PassShape {
     uint32_t threads, tile;
 };
 constexpr uint32_t kBigLog = 19;
+constexpr uint32_t kOnePassLog = 11;
 
 // columns per tile: the smallest power of two >= min(ncols, 8)
 uint32_t tile_log_c(uint64_t ncols) {
@@ -555,13 +561,16 @@ uint32_t tile_log_c(uint64_t ncols) {
     return lc;
 }
 
-PassShape plan_shape(uint32_t log_n, uint64_t ncols) {
+// bits: the index bits the passes transform (fewer than log_n in an extension)
+PassShape plan_shape(uint32_t log_n, uint64_t ncols, uint32_t bits) {
     const uint32_t lc = tile_log_c(ncols);
     uint32_t work = log_n;  // log2 of rows x column chunks (rounded down)
     while ((2ull << (work - log_n)) <= ((ncols + (1ull << lc) - 1) >> lc)) ++work;
     if (work >= kBigLog) return {128, lc >= 2 ? 9u : lc == 1 ? 11u : 10u};
-    uint32_t tile = lc == 3 ? 10 : lc == 2 ? 11 : 12;
-    while (tile > 6 && work < tile + 9) --tile;
+    uint32_t tile = 9;
+    const uint32_t least = bits > 6 && bits + lc <= kOnePassLog ? bits : 6;
+    if (tile < least) tile = least;
+    while (tile > least && work < tile + 9) --tile;
     return {256, tile};
 }
 uint32_t max_t(const PassShape &sh) { return sh.tile < (uint32_t)kMaxT ? sh.tile : (uint32_t)kMaxT; }
@@ -672,7 +681,7 @@ int plan_passes(uint32_t bits, uint32_t tmax, bool low_first, uint32_t *t_out) {
 int run_dif(const uint64_t *src, uint64_t *dst, uint32_t log_n, uint64_t ncols, bool inverse, uint32_t scale,
             uint64_t scale_c, cudaStream_t st) {
     uint32_t ts[32];
-    const PassShape sh = plan_shape(log_n, ncols);
+    const PassShape sh = plan_shape(log_n, ncols, log_n);
     const int np = plan_passes(log_n, max_t(sh), false, ts);
     uint32_t top = log_n;
     for (int k = 0; k < np; ++k) {
@@ -804,7 +813,7 @@ pg_status pg_lde(const uint64_t *evals, size_t n, size_t ncols, uint32_t log_blo
     // DIT passes over bits [b, log N) of out; the first reads coefficient row i >> b
     const uint32_t log_big = log_n + log_blowup;
     uint32_t ts[32];
-    const PassShape sh = plan_shape(log_big, ncols);
+    const PassShape sh = plan_shape(log_big, ncols, log_n);
     const int np = plan_passes(log_n, max_t(sh), true, ts);
     uint32_t lo = log_blowup;
     for (int k = 0; k < np; ++k) {
