@@ -547,12 +547,17 @@ __global__ void k_ntt_bitrev(uint64_t *data, uint32_t log_n, uint64_t ncols) {
 // second launch costs more than one block's work.  2^8 rows x 3, calls back to
 // back: 9.1 us in one pass, 11.4 in two; extension of 2^8 x 3, blowup 1: 10.9
 // against 14.4 (2^11 words: 2^9 x 3 9.2 against 11.0; 2^12: 2^10 x 3 extended 17.9
-// in one pass, 15.1 in two).
+// in one pass, 15.1 in two).  One column: two passes of 2^10-row tiles (19 and 20
+// bits) leave the wide pass without low values, so that it reads and writes eight
+// bytes at a time; up to 20 bits 256 threads on tiles of 2^11 rows: 2^20 rows 43.0
+// against 54.3 us, extended by 8 235 against 297; from 21 bits on, three passes,
+// 2^10-row tiles: 2^22 rows 133 against 163.
 struct PassShape {
     uint32_t threads, tile;
 };
 constexpr uint32_t kBigLog = 19;
 constexpr uint32_t kOnePassLog = 11;
+constexpr uint32_t kTwoPassBits = 20;
 
 // columns per tile: the smallest power of two >= min(ncols, 8)
 uint32_t tile_log_c(uint64_t ncols) {
@@ -566,6 +571,7 @@ PassShape plan_shape(uint32_t log_n, uint64_t ncols, uint32_t bits) {
     const uint32_t lc = tile_log_c(ncols);
     uint32_t work = log_n;  // log2 of rows x column chunks (rounded down)
     while ((2ull << (work - log_n)) <= ((ncols + (1ull << lc) - 1) >> lc)) ++work;
+    if (work >= kBigLog && lc == 0 && bits <= kTwoPassBits) return {256, 11};
     if (work >= kBigLog) return {128, lc >= 2 ? 9u : lc == 1 ? 11u : 10u};
     uint32_t tile = 9;
     const uint32_t least = bits > 6 && bits + lc <= kOnePassLog ? bits : 6;
