@@ -551,13 +551,16 @@ __global__ void k_ntt_bitrev(uint64_t *data, uint32_t log_n, uint64_t ncols) {
 // bits) leave the wide pass without low values, so that it reads and writes eight
 // bytes at a time; up to 20 bits 256 threads on tiles of 2^11 rows: 2^20 rows 43.0
 // against 54.3 us, extended by 8 235 against 297; from 21 bits on, three passes,
-// 2^10-row tiles: 2^22 rows 133 against 163.
+// 2^10-row tiles: 2^22 rows 133 against 163; above 26 bits three passes of 2^10-row
+// tiles are as narrow again, and 256 threads on tiles of 2^12 rows take over:
+// 2^28 rows 14.0 against 17.0 ms, 2^27 extended by 8 32.4 against 48.8.
 struct PassShape {
     uint32_t threads, tile;
 };
 constexpr uint32_t kBigLog = 19;
 constexpr uint32_t kOnePassLog = 11;
 constexpr uint32_t kTwoPassBits = 20;
+constexpr uint32_t kThreePassBits = 26;
 
 // columns per tile: the smallest power of two >= min(ncols, 8)
 uint32_t tile_log_c(uint64_t ncols) {
@@ -572,6 +575,7 @@ PassShape plan_shape(uint32_t log_n, uint64_t ncols, uint32_t bits) {
     uint32_t work = log_n;  // log2 of rows x column chunks (rounded down)
     while ((2ull << (work - log_n)) <= ((ncols + (1ull << lc) - 1) >> lc)) ++work;
     if (work >= kBigLog && lc == 0 && bits <= kTwoPassBits) return {256, 11};
+    if (work >= kBigLog && lc == 0 && bits > kThreePassBits) return {256, 12};
     if (work >= kBigLog) return {128, lc >= 2 ? 9u : lc == 1 ? 11u : 10u};
     uint32_t tile = 9;
     const uint32_t least = bits > 6 && bits + lc <= kOnePassLog ? bits : 6;
