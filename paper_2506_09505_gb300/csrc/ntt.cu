@@ -553,12 +553,17 @@ __global__ void k_ntt_bitrev(uint64_t *data, uint32_t log_n, uint64_t ncols) {
 // against 54.3 us, extended by 8 235 against 297; from 21 bits on, three passes,
 // 2^10-row tiles: 2^22 rows 133 against 163; above 26 bits three passes of 2^10-row
 // tiles are as narrow again, and 256 threads on tiles of 2^12 rows take over:
-// 2^28 rows 14.0 against 17.0 ms, 2^27 extended by 8 32.4 against 48.8.
+// 2^28 rows 14.0 against 17.0 ms, 2^27 extended by 8 32.4 against 48.8.  Many
+// columns: the chunks alone fill the SMs, and 9 or 10 bits in one pass read and
+// write the data once: 2^9 rows x 2000 columns 14.6 us against 25.2 in two passes (with
+// fewer chunks than SMs two stay: an extension of 2^9 x 1000 28 us, 37 in one pass
+// each), 2^10 x 4000 50 against 70; 2^10 x 1500, below that line, 27 against 31.
 struct PassShape {
     uint32_t threads, tile;
 };
 constexpr uint32_t kBigLog = 19;
 constexpr uint32_t kOnePassLog = 11;
+constexpr uint64_t kSms = 152;
 constexpr uint32_t kTwoPassBits = 20;
 constexpr uint32_t kThreePassBits = 26;
 
@@ -572,13 +577,16 @@ uint32_t tile_log_c(uint64_t ncols) {
 // bits: the index bits the passes transform (fewer than log_n in an extension)
 PassShape plan_shape(uint32_t log_n, uint64_t ncols, uint32_t bits) {
     const uint32_t lc = tile_log_c(ncols);
+    const uint64_t chunks = (ncols + (1ull << lc) - 1) >> lc;
     uint32_t work = log_n;  // log2 of rows x column chunks (rounded down)
-    while ((2ull << (work - log_n)) <= ((ncols + (1ull << lc) - 1) >> lc)) ++work;
+    while ((2ull << (work - log_n)) <= chunks) ++work;
+    if (bits == 10 && lc >= 2 && work >= kBigLog - 1) return {256, 10};
     if (work >= kBigLog && lc == 0 && bits <= kTwoPassBits) return {256, 11};
     if (work >= kBigLog && lc == 0 && bits > kThreePassBits) return {256, 12};
     if (work >= kBigLog) return {128, lc >= 2 ? 9u : lc == 1 ? 11u : 10u};
     uint32_t tile = 9;
-    const uint32_t least = bits > 6 && bits + lc <= kOnePassLog ? bits : 6;
+    const bool one = bits + lc <= kOnePassLog || (bits == 9 && chunks > kSms);
+    const uint32_t least = bits > 6 && one ? bits : 6;
     if (tile < least) tile = least;
     while (tile > least && work < tile + 9) --tile;
     return {256, tile};
@@ -786,7 +794,7 @@ pg_status pg_ntt(uint64_t *data, size_t n, size_t ncols, int inverse, void *stre
         pg12::ProfScope prof(pg12::kIdNttBitrev, st, 0);
         const uint64_t total = (uint64_t)ncols << log_n;
         const uint64_t want = (total + 255) / 256;
-        const unsigned grid = (unsigned)(want < 152ull * 16 ? want : 152ull * 16);
+        const unsigned grid = (unsigned)(want < kSms * 16 ? want : kSms * 16);
         const cudaError_t e = launch_dependent(k_ntt_bitrev, grid, 256, 0, st, data, log_n, (uint64_t)ncols);
         if (e != cudaSuccess) return (pg_status)pg12::set_error(PG_ERR_CUDA, "k_ntt_bitrev: %s", cudaGetErrorString(e));
     }
