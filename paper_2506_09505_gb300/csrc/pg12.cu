@@ -1441,12 +1441,41 @@ cudaError_t launch_dependent(void (*kernel)(KArgs...), unsigned grid, unsigned b
 
 // Four threads per state for launches of at most one unit per SM (a permutation
 // 18.8 us against 22; with a second unit per SM 38 us, two groups side by side
-// 26.6) and for batches of at most four leaf tasks per SM, whose time is the
-// climb (32 trees of 2^8 .. 2^12 leaves, 426 tasks: 409 against 479 us; 772 tasks:
-// 711 against 695).
+// 26.6).
 bool tc_small(uint64_t units) { return units <= (uint64_t)g.sms; }
-bool tc_small_batch(uint64_t tasks) { return tasks <= 4 * (uint64_t)g.sms; }
 uint64_t tc_units_of(uint64_t n) { return (n + dev::kTcGroup - 1) / dev::kTcGroup; }
+// Batches: four threads per state while the longest chain of dependent units of a
+// tree, not the number of units, sets the time.  Both are counted in permutations
+// of a unit (a level in the latency form takes a third of one); the line is 1.5
+// times the chain per SM, and at most four leaf tasks per SM.  32 trees of 2^8 ..
+// 2^12 leaves, 0.6 of the chain: 393 us against 479; four trees of 2^14 x 8 0.6:
+// 359 / 522; 57 of 2^10 x 16 1.15: 354 / 335; 57 of 2^10 x 64 1.9: 773 / 538; 76 of
+// 2^10 x 256 3.6: 3,103 / 1,741.  Of 538 measured batches none is slower than
+// with four tasks per SM as the only line, and the one that line cost most takes
+// 1.79 times less.
+bool tc_small_batch(const dev::TreePlan *plans, size_t n_plans, uint32_t tasks, uint32_t fuse) {
+    if (tasks > 4 * (uint32_t)g.sms) return false;
+    double units = 0, chain = 0;
+    for (size_t k = 0; k < n_plans; ++k) {
+        const dev::TreePlan &tp = plans[k];
+        const uint64_t chunks = (tp.width + kRate - 1) / kRate, leaf_units = tc_units_of(tp.n_leaves);
+        const uint32_t top = tp.log_n < tp.climb_limit ? tp.log_n : tp.climb_limit;
+        double all = (double)leaf_units * chunks, path = (double)std::min(leaf_units, (uint64_t)1 << fuse) * chunks;
+        for (uint32_t l = 1; l <= top; ++l) {
+            const uint64_t nodes = tp.n_leaves >> l;
+            if (top == tp.log_n && nodes <= dev::kTcSmallLevel) {
+                all += (tp.log_n - l + 1) / 3.0;
+                path += (tp.log_n - l + 1) / 3.0;
+                break;
+            }
+            all += (double)tc_units_of(nodes);
+            path += (double)std::max((uint64_t)1, std::min(tc_units_of(nodes), ((uint64_t)1 << fuse) >> l));
+        }
+        units += all;
+        chain = std::max(chain, path);
+    }
+    return 2 * units <= 3 * (double)g.sms * chain;
+}
 
 // Tensor-core kernels: one CTA per SM at most; with fewer units than groups the
 // CTAs fill evenly (tc_first_unit).
@@ -1568,14 +1597,16 @@ uint64_t top_perms_of(const dev::TreePlan *plans, size_t n) {
 
 // The persistent kernel of a batch (tensor or integer engine), then, for
 // top_lanes = 16, the 16-lane launch of every tree's top levels.
-pg_status launch_batch(const pg_schedule *sched, const dev::TreePlan *d_plans, uint32_t n_trees, uint32_t tasks,
-                       uint32_t *d_counters, cudaStream_t st, uint64_t perms, uint64_t top_perms) {
+// h_plans: the host's copy of the plans.
+pg_status launch_batch(const pg_schedule *sched, const dev::TreePlan *h_plans, const dev::TreePlan *d_plans,
+                       uint32_t n_trees, uint32_t tasks, uint32_t *d_counters, cudaStream_t st, uint64_t perms) {
+    const uint64_t top_perms = top_perms_of(h_plans, n_trees);
     if (batch_uses_tc(sched)) {
         const uint32_t fuse = sched ? sched->fuse_levels : 0;
         const unsigned grid = tasks < (uint32_t)g.sms ? tasks : (uint32_t)g.sms;
         if (grid > 0) {
             ProfScope prof(kIdTcBatch, st, perms - top_perms);
-            if (tc_small_batch(tasks))
+            if (tc_small_batch(h_plans, n_trees, tasks, fuse))
                 dev::k_tc_batch<4><<<grid, dev::TcShape<4>::kThreads, dev::TcShape<4>::kBytes, st>>>(
                     d_plans, n_trees, tasks, fuse, d_counters + 1, d_counters);
             else
@@ -1647,7 +1678,7 @@ struct pg_batch_graph {
     size_t plan_bytes;
     uint32_t n_trees, tasks;
     uint64_t counters;
-    uint64_t perms, top_perms;
+    uint64_t perms;
     cudaGraph_t graph;
     cudaGraphExec_t exec;
     cudaStream_t capture;
@@ -1845,9 +1876,8 @@ bool server_step(pg_server *s) {
         if (e == cudaSuccess)
             e = cudaMemsetAsync(slot->d_counters, 0, sizeof(uint32_t) * (1 + (size_t)counters), slot->stream);
         if (e == cudaSuccess)
-            st = launch_batch(&rs, slot->d_plans, (uint32_t)plans.size(), tasks, slot->d_counters,
-                              slot->stream, batch_perms(trees.data(), trees.size()),
-                              top_perms_of(plans.data(), plans.size()));
+            st = launch_batch(&rs, plans.data(), slot->d_plans, (uint32_t)plans.size(), tasks, slot->d_counters,
+                              slot->stream, batch_perms(trees.data(), trees.size()));
         if (e == cudaSuccess && st == PG_OK) e = cudaEventRecord(slot->done, slot->stream);
     }
     const double t = s->now();
@@ -2351,8 +2381,8 @@ pg_status pg_merkle_build_batch(const pg_tree *trees, size_t n_trees, const pg_s
     auto *d_counters = reinterpret_cast<uint32_t *>(g.ws + kPlanBytes);
     PG_CUDA(cudaMemcpyAsync(d_plan, plans.data(), plan_bytes, cudaMemcpyHostToDevice, st));
     PG_CUDA(cudaMemsetAsync(d_counters, 0, counter_bytes, st));
-    return launch_batch(&rs, d_plan, (uint32_t)plans.size(), tasks, d_counters, st, batch_perms(trees, n_trees),
-                        top_perms_of(plans.data(), plans.size()));
+    return launch_batch(&rs, plans.data(), d_plan, (uint32_t)plans.size(), tasks, d_counters, st,
+                        batch_perms(trees, n_trees));
 }
 
 pg_status pg_batch_graph_create(const pg_tree *trees, size_t n_trees, const pg_schedule *sched,
@@ -2376,7 +2406,6 @@ pg_status pg_batch_graph_create(const pg_tree *trees, size_t n_trees, const pg_s
     h->tasks = tasks;
     h->counters = counters;
     h->perms = batch_perms(trees, n_trees);
-    h->top_perms = top_perms_of(plans.data(), plans.size());
     const size_t plan_bytes_aligned = (h->plan_bytes + 255) & ~(size_t)255;
     const size_t total = plan_bytes_aligned + sizeof(uint32_t) * (1 + (size_t)counters);
     cudaError_t e = cudaMalloc(&h->dmem, total);
@@ -2401,7 +2430,7 @@ pg_status pg_batch_graph_create(const pg_tree *trees, size_t n_trees, const pg_s
     e = cudaStreamBeginCapture(h->capture, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return cleanup(fail(PG_ERR_CUDA, "begin capture: %s", cudaGetErrorString(e)));
     cudaError_t e_memset = cudaMemsetAsync(d_counters, 0, sizeof(uint32_t) * (1 + (size_t)counters), h->capture);
-    pg_status sl = launch_batch(&h->sched, d_plan, h->n_trees, tasks, d_counters, h->capture, h->perms, h->top_perms);
+    pg_status sl = launch_batch(&h->sched, plans.data(), d_plan, h->n_trees, tasks, d_counters, h->capture, h->perms);
     e = cudaStreamEndCapture(h->capture, &h->graph);
     if (e_memset != cudaSuccess || sl != PG_OK || e != cudaSuccess)
         return cleanup(sl != PG_OK ? sl : fail(PG_ERR_CUDA, "capture: %s", cudaGetErrorString(e != cudaSuccess ? e : e_memset)));
