@@ -194,9 +194,11 @@ pg_status pg_set_engine(int engine);
 int pg_get_engine(void);
 
 /*
- * pg_tc_tables_export -- host copy of the tensor-core digit tables of the
- * active parameter set, for inspection and CPU tests: with out == NULL
- * returns the table size in bytes; else writes it to `out` (host, `bytes`
+ * pg_tc_tables_export -- digit tables of the active parameter set's
+ * contractions in their plain form (no Montgomery factors, no scaling of the
+ * chain, one bias): what the tables of pg_kernel_tables_export, which the
+ * kernels read, are derived like.  For inspection and CPU tests: with out ==
+ * NULL returns the table size in bytes; else writes it to `out` (host, `bytes`
  * long) and returns it, or returns 0 if `bytes` is too small.  Layout (all
  * little-endian fp16 bit patterns, K-major 8x8 core matrices of 128 bytes;
  * a table of n output rows and k input words holds row 8i+b, column 8j+a =
@@ -216,6 +218,35 @@ int pg_get_engine(void);
  * Host-only; works without a GPU.
  */
 size_t pg_tc_tables_export(void *out, size_t bytes);
+
+/*
+ * pg_kernel_tables_export -- host copy of the tables that pg_init and
+ * pg_params_select upload and the tensor-core and latency-form kernels read,
+ * for inspection and CPU tests; called like pg_tc_tables_export.  R = 2^64,
+ * f(x) = x^7 R^-6 the kernels' S-box, lambda and kappa the chain's scaling:
+ * lambda[22] = 1, kappa[q] = lambda[q+1] beta[q][q], lambda[q]^7 = kappa[q] R^6
+ * (beta, vp, w of pg_params_export_chain).  Layout, in this order:
+ *   fp16 bit patterns, core matrices and digits as in pg_tc_tables_export:
+ *   m    [96 x 96]  M R^6
+ *   pre  [96 x 96]  the transition matrix R^6, row 0 also times lambda[0]
+ *   b_bias [12 row groups x 2 core matrices]  row b of group i, column k =
+ *                   4 u_b of contraction kind k (0..7 the layer after full
+ *                   round k, 8 and 9 U, 10 the cells' updates): the kind's
+ *                   constants, added to the products
+ *   a_bias [10 core matrices]  Z, H_0 .. H_7, Z: H_j holds 2^-13 in column j;
+ *                   kind k < 8 multiplies (H_k, Z), kind k >= 8 (Z, H_(k-8))
+ *   a_zcap [4 core matrices]  bytes of f(c_0[j]), j = 8..11, every row
+ *   vpa  [80 x 96], vpb [96 x 96]  row q of vp times R^6 lambda[q+1]
+ *   bs   [96 x 96], w1 [96 x 96], w2 [96 x 96]  as in pg_tc_tables_export, of
+ *                   beta[q][r] lambda[q+1] / kappa[r] and w[i][r] / kappa[r]
+ *   64-bit words, times R where a kernel multiplies by them, entry e of 16 per
+ *   row the lane's (e < 12: cell e; chain tables a: row q = e, b: q = 16 + e):
+ *   rc0, add[8], m[12], pre[12], ua[12], ub[12], ua_add, ub_add, x_add,
+ *   ba[22], bb[22], w[22]
+ *   beta [22 x 22]  beta[q][r] lambda[q+1] / kappa[r] times R
+ * Host-only; works without a GPU.
+ */
+size_t pg_kernel_tables_export(void *out, size_t bytes);
 
 /*
  * pg_params_export_chain -- host copy of the unrolled form of the 22 partial

@@ -97,6 +97,7 @@ SIGNATURES = {
     "pg_params_name": (ctypes.c_char_p, []),
     "pg_set_engine": (ctypes.c_int, [ctypes.c_int]),
     "pg_tc_tables_export": (ctypes.c_size_t, [ctypes.c_void_p, ctypes.c_size_t]),
+    "pg_kernel_tables_export": (ctypes.c_size_t, [ctypes.c_void_p, ctypes.c_size_t]),
     "pg_params_export_chain": (ctypes.c_int, [_u64p, _u64p, _u64p]),
     "pg_get_engine": (ctypes.c_int, []),
     "pg_device_faults": (ctypes.c_int, [ctypes.POINTER(ctypes.c_uint32)]),
@@ -258,6 +259,15 @@ def tc_tables_export() -> bytes:
     buf = ctypes.create_string_buffer(n)
     if int(load().pg_tc_tables_export(buf, n)) != n:
         raise PGError(6, "tensor-core tables unavailable: " + last_error())
+    return buf.raw
+
+
+def kernel_tables_export() -> bytes:
+    """The tables the kernels of the active parameter set read (see include/pg12.h)."""
+    n = int(load().pg_kernel_tables_export(None, 0))
+    buf = ctypes.create_string_buffer(n)
+    if int(load().pg_kernel_tables_export(buf, n)) != n:
+        raise PGError(6, "kernel tables unavailable: " + last_error())
     return buf.raw
 
 

@@ -1240,11 +1240,25 @@ pg_status ensure_params() {
 struct SetTables {
     bool ready = false;
     dev::DevConsts dc;
-    WideConsts wc;
-    TcDev td;
-    uint64_t beta[kRP][kRP];
+    KernelTables kt;
 };
 SetTables g_tables[2];
+
+pg_status build_tables(SetTables &t) {
+    if (t.ready) return PG_OK;
+    const char *set = g.params_set == 1 ? "pg12_small" : "pg12_v1";
+    static KernelParams kp;
+    dev::make_dev_consts(g.opt, t.dc);
+    if (!host::derive_kernel(g.opt, kp))
+        return fail(PG_ERR_PARAMS, "parameter set %s: a partial round's coefficient is zero", set);
+    host::build_wide(kp, t.kt.wide);
+    if (!host::build_tc_dev(g.opt, kp, t.kt.tc))
+        return fail(PG_ERR_PARAMS, "parameter set %s: a tensor-core sum could leave the exact fp32 window", set);
+    for (int q = 0; q < kRP; ++q)
+        for (int r = 0; r < kRP; ++r) t.kt.beta[q][r] = host::fp_mul(kp.beta[q][r], kEps);
+    t.ready = true;
+    return PG_OK;
+}
 
 // Constant tables of the active parameter set onto the current device: the
 // permutation constants of both permutation forms and the digit tables of
@@ -1254,23 +1268,12 @@ SetTables g_tables[2];
 // waiting for it.
 pg_status upload_tables() {
     SetTables &t = g_tables[g.params_set];
-    if (!t.ready) {
-        const char *set = g.params_set == 1 ? "pg12_small" : "pg12_v1";
-        static KernelParams kp;
-        dev::make_dev_consts(g.opt, t.dc);
-        if (!host::derive_kernel(g.opt, kp))
-            return fail(PG_ERR_PARAMS, "parameter set %s: a partial round's coefficient is zero", set);
-        host::build_wide(kp, t.wc);
-        if (!host::build_tc_dev(g.opt, kp, t.td))
-            return fail(PG_ERR_PARAMS, "parameter set %s: a tensor-core sum could leave the exact fp32 window", set);
-        for (int q = 0; q < kRP; ++q)
-            for (int r = 0; r < kRP; ++r) t.beta[q][r] = host::fp_mul(kp.beta[q][r], kEps);
-        t.ready = true;
-    }
+    const pg_status s = build_tables(t);
+    if (s != PG_OK) return s;
     PG_CUDA(cudaMemcpyToSymbol(dev::c_dev, &t.dc, sizeof(t.dc)));
-    PG_CUDA(cudaMemcpyToSymbol(dev::g_wide, &t.wc, sizeof(t.wc)));
-    PG_CUDA(cudaMemcpyToSymbol(dev::g_tc, &t.td, sizeof(t.td)));
-    PG_CUDA(cudaMemcpyToSymbol(dev::c_beta, t.beta, sizeof(t.beta)));
+    PG_CUDA(cudaMemcpyToSymbol(dev::g_wide, &t.kt.wide, sizeof(t.kt.wide)));
+    PG_CUDA(cudaMemcpyToSymbol(dev::g_tc, &t.kt.tc, sizeof(t.kt.tc)));
+    PG_CUDA(cudaMemcpyToSymbol(dev::c_beta, t.kt.beta, sizeof(t.kt.beta)));
     PG_CUDA(cudaStreamSynchronize(cudaStreamLegacy));
     return PG_OK;
 }
@@ -2006,8 +2009,17 @@ size_t pg_tc_tables_export(void *out, size_t bytes) {
     if (bytes < sizeof(TcTables)) return 0;
     std::lock_guard<std::mutex> lk(g_mu);
     if (ensure_params() != PG_OK) return 0;
-    host::build_tc_tables(g.opt, *static_cast<TcTables *>(out));
+    if (!host::build_tc_tables(g.opt, *static_cast<TcTables *>(out))) return 0;
     return sizeof(TcTables);
+}
+
+size_t pg_kernel_tables_export(void *out, size_t bytes) {
+    if (out == nullptr) return sizeof(KernelTables);
+    if (bytes < sizeof(KernelTables)) return 0;
+    std::lock_guard<std::mutex> lk(g_mu);
+    if (ensure_params() != PG_OK || build_tables(g_tables[g.params_set]) != PG_OK) return 0;
+    std::memcpy(out, &g_tables[g.params_set].kt, sizeof(KernelTables));
+    return sizeof(KernelTables);
 }
 
 pg_status pg_params_export_chain(uint64_t *vp, uint64_t *beta, uint64_t *w) {

@@ -124,8 +124,8 @@ struct KernelParams {
     uint64_t x_add[kT];
 };
 
-// The tables the kernels read (TcTables is the exported form): KernelParams'
-// matrices as digit tables, and
+// The tables the kernels read (TcTables has the same matrices without the
+// scaling): KernelParams' matrices as digit tables, and
 //   - a_zcap holds the S-box outputs f(c_0[j]);
 //   - the bias carries the constants that follow the contraction: the bias of
 //     kind k (TcBias) makes row i come out as (M y)_i + const_k[i], so no round
@@ -172,6 +172,15 @@ struct WideConsts {
     uint64_t w[kRP][kWide];          // w~[i][r] by r
 };
 static_assert(sizeof(WideConsts) % 16 == 0, "constant tables are copied in 16-byte pieces");
+
+// What the Montgomery kernels read, as uploaded and as pg_kernel_tables_export
+// hands it out; beta: the tensor-core chain's coefficients beta~ times R.
+struct KernelTables {
+    TcDev tc;
+    WideConsts wide;
+    uint64_t beta[kRP][kRP];
+};
+static_assert(sizeof(KernelTables) == sizeof(TcDev) + sizeof(WideConsts) + 8 * kRP * kRP, "no padding in the exported form");
 
 // Records the text returned by pg_last_error() and passes `status` through.
 int set_error(int status, const char *fmt, ...);
