@@ -39,7 +39,7 @@ MUL_RESULTS_PER_PERM = 118 * (2 * 6 + 2 * 8) + 8 * 144 * 8 + 22 * 23 * 8
 # pg12_small: the seven full rounds with the 8-bit matrix take two 32x8-bit
 # IMAD.WIDE per term (4 results); round 3's transition matrix stays full width.
 MUL_RESULTS_PER_PERM_SMALL = 118 * (2 * 6 + 2 * 8) + 7 * 144 * 4 + 144 * 8 + 22 * 23 * 8
-# In the one-thread-per-state kernels a permutation whose capacity cells enter
+# In the integer engine's one-thread-per-state kernels a permutation whose capacity cells enter
 # as zero (node compressions, the first chunk of a sponge) skips 4 S-boxes and
 # 48 products of round 0, and one whose result is a digest (nodes, the last
 # chunk of a sponge) computes 4 of the 12 rows of the last dense layer (96
@@ -52,6 +52,30 @@ DIGEST_SAVED_SMALL = 96 * 4
 ZCAP_KERNELS = ("k_merkle", "k_merkle_level", "k_hash_rows", "k_tc_sponge:leaves", "k_tc_sponge:level",
                 "k_tc_sponge:rows")
 LEVEL_KERNELS = ("k_merkle_level", "k_tc_sponge:level")
+# The tensor-core kernels run every linear layer on the tensor cores: what their
+# threads multiply is 118 S-boxes of four products and the 90 products of the
+# chain of partial rounds (8 results each); a zero capacity saves four S-boxes.
+TC_MUL_RESULTS_PER_PERM = 118 * 4 * 8 + 90 * 8
+TC_ZCAP_SAVED = 4 * 4 * 8
+PIPE_WORK = {"fmaheavy": "the 32-bit multiply-adds of the field products", "alu": "the carry arithmetic of the reductions",
+             "tensor": "the linear layers"}
+INT_KERNELS = ("k_merkle", "k_merkle_level", "k_merkle_single", "k_permute", "k_hash_rows")
+
+
+def executed_mul32_per_perm(kernel, chunks, small=False):
+    """32-bit multiply results a kernel's threads execute per permutation; None for
+    the latency form (its lanes repeat the chain) and kernels without permutations."""
+    # node launches: every permutation starts from a zero capacity and ends in a
+    # digest; leaf launches: the first and the last of each leaf's chunks
+    share = (1.0 if kernel in LEVEL_KERNELS else 1.0 / chunks) if kernel in ZCAP_KERNELS else 0.0
+    if kernel.startswith("k_tc_"):
+        return TC_MUL_RESULTS_PER_PERM - share * TC_ZCAP_SAVED
+    if kernel not in INT_KERNELS:
+        return None
+    saved = (ZCAP_SAVED_SMALL + DIGEST_SAVED_SMALL) if small else (ZCAP_SAVED + DIGEST_SAVED)
+    return (MUL_RESULTS_PER_PERM_SMALL if small else MUL_RESULTS_PER_PERM) - share * saved
+
+
 LEAF_KERNELS = ("k_merkle", "k_merkle_top_leaf", "k_tc_sponge:leaves")
 IMAD_RESULTS_PER_CLK_SM = 64  # 32-bit multiply results per clock per SM
 L2_BYTES = 129 * 10**6  # GB300 L2
@@ -427,10 +451,12 @@ def run_ours(args):
     e_steps = max(3, min(args.steps, 10))
     e_sampler = ClockSampler(gpu_id)
     time.sleep(0.4)
-    t0 = time.perf_counter()
+    marks = [time.perf_counter()]
     for _ in range(e_steps):
         pg.merkle_build_host(host_rows, dev_rows, nodes, want_root=True)
-    e_s = time.perf_counter() - t0
+        marks.append(time.perf_counter())
+    e_s = marks[-1] - marks[0]
+    e_each = [1e3 * (b - a) for a, b in zip(marks, marks[1:])]
     e_clocks = e_sampler.stop()
     # the same rows as one plain pinned copy: the host link's bandwidth on this machine, which
     # bounds the end-to-end step when the copy outlasts the leaf hashing it overlaps
@@ -446,7 +472,8 @@ def run_ours(args):
         e_s = float(t.item())
     e2e = {"value": perms * world * e_steps / e_s, "unit": "perms/s",
            "h2d_bytes_per_step": int(rows_np.nbytes), "d2h_bytes_per_step": 32,
-           "ms_per_step": 1e3 * e_s / e_steps, "clocks": e_clocks,
+           "ms_per_step": 1e3 * e_s / e_steps, "ms_min": min(e_each), "ms_median": statistics.median(e_each),
+           "ms_max": max(e_each), "clocks": e_clocks,
            "h2d_copy_gbs": h2d_gbs, "h2d_copy_ms": rows_np.nbytes / h2d_gbs / 1e6}
 
     peaks = measured_peaks()
@@ -457,16 +484,7 @@ def run_ours(args):
     tot_kernel_ms = sum(v["total_ms"] for v in kernels.values())
 
     small = args.params == "pg12_small"
-    saved = (ZCAP_SAVED_SMALL + DIGEST_SAVED_SMALL) if small else (ZCAP_SAVED + DIGEST_SAVED)
     chunks = max(1, (args.width + 7) // 8)
-
-    def executed_per_perm(name):
-        # node launches: every permutation starts from a zero capacity and ends
-        # in a digest; leaf launches: the first and the last of each leaf's chunks
-        if name not in ZCAP_KERNELS:
-            return mul_per_perm
-        share = 1.0 if name in LEVEL_KERNELS else 1.0 / chunks
-        return mul_per_perm - share * saved
 
     km = kernel_metrics()
     traffic_table = km.get("traffic_bytes_per_launch", {}).get(f"merkle_2e{args.log_n}_w{args.width}", {}) \
@@ -477,9 +495,10 @@ def run_ours(args):
         launch_ms = v["total_ms"] / v["launches"]      # average launch, event-timed
         per_launch = v["perms"] // v["launches"]       # permutations per launch
         ach = per_launch * mul_per_perm / (launch_ms / 1e3) / 1e12
-        ach_x = per_launch * executed_per_perm(name) / (launch_ms / 1e3) / 1e12
+        executed = executed_mul32_per_perm(name, chunks, small)
+        frac_x = per_launch * executed / (launch_ms / 1e3) / 1e12 / peak if executed is not None else None
         return {"achieved": ach, "frac": ach / peak, "launch_ms": launch_ms, "perms_per_launch": per_launch,
-                "frac_executed": ach_x / peak, "executed_mul32_results_per_perm": executed_per_perm(name),
+                "frac_executed": frac_x, "executed_mul32_results_per_perm": executed,
                 "mul32_results_per_launch": per_launch * mul_per_perm,
                 "algorithmic_bytes_per_launch": algorithmic_bytes(name, per_launch, args.width),
                 "traffic": traffic_table.get(name)}
@@ -496,7 +515,7 @@ def run_ours(args):
                  "frac": rk["perms_per_launch"] / (rk["launch_ms"] / 1e3) / issue_ceiling,
                  "issue_active_pct_ncu": kmet["issue_active_pct"]}
         bound_basis = (f"ncu on {metrics_kernel(dom)}: pipes busy {kmet['pipes_pct']} (% of peak); the busiest, "
-                       f"'{busiest}', carries the carry arithmetic of the field products")
+                       f"'{busiest}', carries {PIPE_WORK.get(busiest, 'most of the work')}")
     else:
         bound, issue, bound_basis = "alu", None, "no ncu capture of the current kernel sources"
     roofline = {
