@@ -10,7 +10,7 @@
 //
 // Everything runs as passes of one kernel.  A block loads the 2^t rows of
 // up to eight columns whose row indices differ only in bits [lo, lo + t)
-// (a tile of 4 to 64 KiB, plan_shape; t <= 11), performs
+// (a tile of at most 64 KiB, plan_shape; t <= 11), performs
 // the t radix-2 stages of those bits in shared memory and stores the rows
 // back; a transform of 2^L rows reads and writes its data ceil(L / t) times.
 //   DIF (Gentleman-Sande) stages: natural order in, bit-reversed order out;
@@ -134,7 +134,7 @@ __device__ __forceinline__ uint64_t sub_w(uint64_t a, uint64_t b) {
 // Value l0 + l1 2^32 + t 2^64 with t a signed 32-bit word: a sum or
 // difference of two such values is one three-word carry chain, with no
 // correction.  Inside a small DFT |t| stays below 2^28 (the largest comes from
-// a 2^24 shift of a value with |t| <= 2); products by 2^48 and 2^72 stay lazy
+// a 2^24 shift of a value with |t| <= 3); products by 2^48 and 2^72 stay lazy
 // too.
 struct Lz {
     uint32_t l0, l1, t;
@@ -535,29 +535,30 @@ __global__ void k_ntt_bitrev(uint64_t *data, uint32_t log_n, uint64_t ncols) {
 }
 
 // Threads per block and log2 of the tile's rows (transformed x low values) of a
-// transform's passes.  Large transforms: blocks of 128 threads, six of them
-// resident per SM at 36 KB each (eight columns), so that the barrier after a step
-// holds up four warps; 21 rows-bits x 8 columns, blowup 2: 0.80 ms against 0.84
-// with 256 threads on 72 KB.  Below 2^19 rows (times column chunks) the grid
-// would not fill the SMs several times over and a block's serial work counts:
-// 256 threads, on tiles that shrink until there are 2^9 of them (but not below
-// 2^6 rows: more passes then cost more than they spread).  2^16 rows x 3: 16.6 us
-// against 33 with 2^11-row tiles; 2^18 x 8: 44.6 against 51.6.  A transform whose
-// rows (times the tile's columns) are at most 2^11 words stays one pass: a
-// second launch costs more than one block's work.  2^8 rows x 3, calls back to
-// back: 9.1 us in one pass, 11.4 in two; extension of 2^8 x 3, blowup 1: 10.9
-// against 14.4 (2^11 words: 2^9 x 3 9.2 against 11.0; 2^12: 2^10 x 3 extended 17.9
-// in one pass, 15.1 in two).  One column: two passes of 2^10-row tiles (19 and 20
-// bits) leave the wide pass without low values, so that it reads and writes eight
-// bytes at a time; up to 20 bits 256 threads on tiles of 2^11 rows: 2^20 rows 43.0
-// against 54.3 us, extended by 8 235 against 297; from 21 bits on, three passes,
-// 2^10-row tiles: 2^22 rows 133 against 163; above 26 bits three passes of 2^10-row
-// tiles are as narrow again, and 256 threads on tiles of 2^12 rows take over:
-// 2^28 rows 14.0 against 17.0 ms, 2^27 extended by 8 32.4 against 48.8.  Many
-// columns: the chunks alone fill the SMs, and 9 or 10 bits in one pass read and
-// write the data once: 2^9 rows x 2000 columns 14.6 us against 25.2 in two passes (with
-// fewer chunks than SMs two stay: an extension of 2^9 x 1000 28 us, 37 in one pass
-// each), 2^10 x 4000 50 against 70; 2^10 x 1500, below that line, 27 against 31.
+// transform's passes.  `work` is the rows times column chunks; times are calls back
+// to back.
+//   Large (work >= 2^19): 128 threads, six blocks resident per SM at 36 KB each
+//   (eight columns), so that the barrier after a step holds up four warps: 2^21 rows x
+//   8, extended by 2, 0.80 ms against 0.84 with 256 threads on 72 KB.
+//   Small: the grid would not fill the SMs several times over and a block's serial
+//   work counts: 256 threads, on tiles that shrink until there are 2^9 of them (but
+//   not below 2^6 rows: more passes then cost more than they spread).  2^16 rows x 3
+//   16.6 us against 33 with 2^11-row tiles; 2^18 x 8 44.6 against 51.6.
+// Except where a shape would add a pass or narrow the accesses:
+//   One pass: a transform of at most 2^11 words a tile (rows x tile columns), since a
+//   second launch costs more than one block's work: 2^8 rows x 3 9.1 us against 11.4
+//   in two passes, extended by 2 10.9 against 14.4 (2^9 x 3 9.2 / 11.0; one step
+//   further, 2^10 x 3 extended, 17.9 / 15.1).
+//   Many columns: the chunks alone fill the SMs, and 9 or 10 bits in one pass read and
+//   write the data once: 2^9 rows x 2000 columns 14.6 us against 25.2, 2^10 x 4000 50
+//   against 70.  Below the lines two passes: 2^9 x 1000 extended 28 us against 37,
+//   2^10 x 1500 27 against 31.
+//   One column: a pass over as many bits as the tile holds has no low values and reads
+//   and writes eight bytes at a time.  That is two passes of 2^10-row tiles at 19 and
+//   20 bits, so up to 20 bits 256 threads on tiles of 2^11 rows (2^20 rows 43.0 us
+//   against 54.3, extended by 8 235 against 297; at 22 bits 163 against 133 in three
+//   passes), and three passes above 26 bits, so there tiles of 2^12 rows (2^28 rows
+//   14.0 ms against 17.0, 2^27 extended by 8 32.4 against 48.8).
 struct PassShape {
     uint32_t threads, tile;
 };

@@ -15,10 +15,12 @@
 //               the levels with few nodes, 16 or 32 lanes per state (latency form).
 //   k_merkle_top_tail
 //               every level of at most 64 nodes up to the root in one launch
-//               of an 8-block cluster, a cluster barrier between levels.
-//   k_merkle_open / k_merkle_verify  authentication paths (Sec. 2.4).
-// The level launches of a single-tree build use programmatic dependent
-// launch (pdl_trigger / pdl_wait below).
+//               of an 8-block cluster; digests go up through shared memory,
+//               the blocks' last ones to block 0.
+//   k_merkle_open / k_merkle_verify  authentication paths (Sec. 2.4);
+//               k_merkle_verify_wide in the latency form.
+//   k_tc_*      the tensor-core forms of permutation, sponge, batch and path check.
+// Most launches use programmatic dependent launch (pdl_trigger / pdl_wait below).
 #include "pg12.h"
 #include "pg12_internal.h"
 #include "poseidon.cuh"
@@ -1067,11 +1069,16 @@ namespace {
 
 // tensor engine: tree levels of at least this many nodes use the tensor-core
 // kernel (four threads per state while a level has at most one unit per SM,
-// tc_small).  Measured on the 2^22 x 8 tree with an earlier version of both
-// forms: 2^15 10.25 ms, 2^13 10.11 ms, 2^12 10.14 ms.
+// tc_small).  With the line at 2^12 / 2^13 / 2^14 nodes: tree of 2^22 x 8 4,967 /
+// 4,959 / 4,951 us, of 2^16 x 8 274 / 269 / 256 (a level of 2^13 nodes takes 13 us less
+// on 16 lanes, one of 2^12 4 us less).
 #ifndef PG12_TC_MIN_NODES
 #define PG12_TC_MIN_NODES (1ull << 13)
 #endif
+// Trees of at most this many leaves hash them in the latency form.  With the line
+// at 2^12 / 2^13 / 2^14 leaves: trees of 2^13 x 8 176 / 155 / 155 us, of 2^14 x 8 192 /
+// 192 / 227; of rows of many chunks the tensor cores would take the smaller ones
+// sooner (2^13 x 64 310 us against 348 in the latency form).
 #ifndef PG12_TC_SMALL_TREE
 #define PG12_TC_SMALL_TREE 8192
 #endif
@@ -1147,29 +1154,31 @@ namespace {
 
 constexpr size_t kWorkspaceBytes = 32u << 20;  // tree plans + arrival counters
 // pg_merkle_build's split of a tree between kernels.  Trees of at most
-// kSmallTree leaves run entirely in the 16-lanes-per-state kernels.  In
+// kSmallTree leaves run entirely in the latency form (16 or 32 lanes per state).  In
 // larger trees one launch hashes the leaves and every level is one launch
 // (one launch per level measured faster than climbing with arrival counters
 // in one persistent launch: 16.7 against 17.4 ms for a 2^22 x 8 tree on the
 // integer pipes, 10.20 against 10.73 ms with the tensor-core kernel): the
 // tensor-core kernel for levels of at least tc_min_nodes nodes, one thread
 // per node (k_merkle_level) while the level has more than kWideNodes nodes
-// (integer engine), the 16-lanes-per-state kernel above that, and one
-// cluster launch for the levels of at most 64 nodes.
+// (integer engine), the latency form above that, and one cluster launch for the
+// levels of at most 64 nodes.  Integer engine with kWideNodes 2^12 / 2^13 / 2^14:
+// trees of 2^13 x 8 239 / 155 / 155 us, 2^14 x 8 294 / 236 / 212, 2^22 x 8 14.91 / 14.86 /
+// 14.83 ms.
 #ifndef PG12_WIDE_NODES
 #define PG12_WIDE_NODES 8192
 #endif
 constexpr uint64_t kWideNodes = PG12_WIDE_NODES;
 constexpr uint64_t kSmallTree = kWideNodes;
-// tensor engine: trees of at most this many leaves run in the 16-lane form
 constexpr uint64_t kTcSmallTree = PG12_TC_SMALL_TREE;
 // Latency form: 32 lanes per state while that is at most one warp per
 // scheduler, above 16 (20-level paths of 608 / 1021 queries: 132 / 174 us on 32
 // lanes, 145 / 149 us on 16).
 unsigned wide_lanes(uint64_t states);
-// pg_merkle_verify: up to this many queries in the latency form (4,864 queries
-// of 20 levels: 363 us on 16 lanes; the tensor-core kernel takes 430 us for any
-// number up to 19,456, one unit of 128 per SM).
+// pg_merkle_verify: up to this many queries in the latency form.  The tensor-core
+// kernel takes 378 us for 20 levels of any number of queries up to 19,456 (one unit
+// of 128 per SM); 16 lanes take 267 us for 3,648 queries, 345 for 4,864 (32 per SM)
+// and, with a ninth warp on some schedulers, 422 for 5,120.
 constexpr uint64_t kVerifyWideMax = 5120;
 constexpr size_t kPlanBytes = 4u << 20;        // first part: plans; rest: counters
 
@@ -1422,7 +1431,7 @@ pg_status plan_batch(const pg_tree *trees, size_t n_trees, const pg_schedule *sc
 
 // One launch per level for levels first..log2(n_leaves) of a tree whose
 // lower levels are in `nodes`: one thread per node (k_merkle_level) while a
-// level has more than kWideNodes nodes, the 16-lanes-per-state kernel above.
+// level has more than kWideNodes nodes, the latency form above.
 // Launch a level kernel with programmatic stream serialisation (see
 // pdl_trigger / pdl_wait): it may start, and copy its constants, while the
 // kernel before it on `st` finishes.
@@ -2223,7 +2232,7 @@ pg_status pg_merkle_build(const uint64_t *rows, size_t n_leaves, size_t width, u
     // nothing but rows and nodes is read or written, so concurrent builds on
     // different streams are independent
     const uint32_t first_top = 1;
-    if ((uint64_t)n_leaves <= (g.engine == 1 ? kTcSmallTree : kSmallTree)) {  // whole tree in the 16-lane form
+    if ((uint64_t)n_leaves <= (g.engine == 1 ? kTcSmallTree : kSmallTree)) {  // leaves in the latency form
         const bool w32 = wide_lanes(n_leaves) == 32;
         const uint64_t threads = (uint64_t)n_leaves * (w32 ? 32 : 16);
         const unsigned grid = (unsigned)((threads + dev::kTopBlock - 1) / dev::kTopBlock);
